@@ -87,7 +87,8 @@ typedef enum {
 typedef enum { S2W_DT_BACKWARD = 0, S2W_DT_NONE = 1 } s2w_dt_mode;
 
 /* Contraction engine for s2w_waveforms.  STREAM: CUDA-core kernels that
- * stream the resident spectra once per rupture (any storage precision).
+ * stream the resident spectra once per up to 8 ruptures (FP32, BF16 and
+ * BF16_HILO storage; memory permitting) or once per rupture (FP8, FP32_HILO).
  * TENSOR: tcgen05 tensor-core GEMMs over the whole rupture batch (one pass
  * over the spectra per sub-batch); needs prec_g = BF16, BF16_HILO or
  * FP8_E4M3, Nt <= 256, No <= 128.  With BF16 the activations (slip and
@@ -348,7 +349,7 @@ typedef struct {
  * CTAs; with the BF16 hi/lo split, only counts at or above the default,
  * since each chunk is one FP32 accumulation and a longer one costs that
  * precision accuracy), and the batch size from which AUTO uses the tensor engine instead
- * of streaming the spectra once per rupture.  The choices are kept in the
+ * of streaming the spectra.  The choices are kept in the
  * context (and written to opts.tune_cache when one is set); an entry already
  * in that cache is applied without timing.  Options the caller fixed
  * (tc_bsub, tc_pair other than AUTO, tc_s2_chunks) are not searched.

@@ -118,7 +118,13 @@ __global__ void __launch_bounds__(kDfThreads) k_df_retransform(const float2* __r
                                                                long long ld_m, int L, const float4* __restrict__ tw,
                                                                float inv_dt_hi, float inv_dt_lo, int dt_mode,
                                                                float2* vhat, float2* vhat_lo, long long ld_v,
-                                                               float* seafloor) {
+                                                               float* seafloor, long long mhat_ld_b,
+                                                               long long vhat_ld_b) {
+  mhat += blockIdx.y * mhat_ld_b;
+  mhat_lo += blockIdx.y * mhat_ld_b;
+  vhat += blockIdx.y * vhat_ld_b;
+  vhat_lo += blockIdx.y * vhat_ld_b;
+  if (seafloor != nullptr) seafloor += static_cast<long long>(blockIdx.y) * Ng * (L / 2);
   extern __shared__ __align__(16) unsigned char smraw[];
   const int N = L / 2;
   float4* tws = reinterpret_cast<float4*>(smraw);
@@ -222,15 +228,17 @@ cudaError_t launch_df_rfft_rows(const float* x, long long rows, int n_in, int Nt
 
 cudaError_t launch_df_retransform(const float2* mhat, const float2* mhat_lo, long long Ng, long long ld_m, int Nt,
                                   const float4* tw, double inv_dt, int dt_mode, float2* vhat, float2* vhat_lo,
-                                  long long ld_v, float* seafloor, cudaStream_t st) {
-  if (Ng <= 0) return cudaSuccess;
+                                  long long ld_v, float* seafloor, cudaStream_t st, int nb, long long mhat_ld_b,
+                                  long long vhat_ld_b) {
+  if (Ng <= 0 || nb <= 0) return cudaSuccess;
   if (Nt < 1 || Nt > 512 || (dt_mode != S2W_DT_BACKWARD && dt_mode != S2W_DT_NONE)) return cudaErrorInvalidValue;
   const int L = 2 * Nt;
   const size_t sm = sizeof(float4) * (L + Nt + 1) + sizeof(float2) * 2 * Nt;
   const float ih = static_cast<float>(inv_dt);
   const float il = static_cast<float>(inv_dt - static_cast<double>(ih));
-  k_df_retransform<<<df_grid(Ng), kDfThreads, sm, st>>>(mhat, mhat_lo, Ng, ld_m, L, tw, ih, il, dt_mode, vhat,
-                                                         vhat_lo, ld_v, seafloor);
+  const dim3 grid(df_grid(Ng), static_cast<unsigned>(nb));
+  k_df_retransform<<<grid, kDfThreads, sm, st>>>(mhat, mhat_lo, Ng, ld_m, L, tw, ih, il, dt_mode, vhat, vhat_lo, ld_v,
+                                                 seafloor, mhat_ld_b, vhat_ld_b);
   return cudaGetLastError();
 }
 

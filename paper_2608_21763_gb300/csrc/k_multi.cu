@@ -1,0 +1,298 @@
+// Per-bin complex contractions for a handful of ruptures (2 .. 8) on
+// CUDA cores: y_b[f] = sum_c rows[f][c] x_b[c] for all of them while the row
+// is in shared memory, so that the batch reads the operator from HBM once
+// (k_stream.cu reads it once per rupture).
+//
+// A unit is (vector group, tile of up to 64 rows); persistent CTAs take units
+// round robin.  One elected lane streams K slabs through a shared-memory ring
+// by TMA: the tile's rows (512 bytes of each, 32 chunks of 16) and the same
+// columns of the R vectors, which come from L2 after their first use.  Warp w
+// owns eight of the rows, lane l chunk l of each slab, and the FP32
+// accumulators of all 8 x R products stay in registers over the whole row;
+// at the end one butterfly reduce-scatter over the lanes sums them.
+//
+// What bounds it: 4 FMAs per stored entry and rupture.  At eight ruptures an
+// FP32 entry costs 32 FMAs for 8 bytes, about 0.8 of the FMA rate when the
+// bytes arrive at the HBM rate, so the two meet there; a wider batch would be
+// bound by the FMAs, a narrower one by HBM.  Measured, whole call: 480 x
+// 37,758 x 32 x 256, 8 ruptures, 46.0 ms one by one, 8.05 ms here (stage 1
+// 42.2 -> 6.7, 5.5 at the copy rate); 333 x 4,999 x 17 x 512 with seafloor
+// output, 5 ruptures, 6.66 -> 1.42 ms.  Rows are cut into K slabs (not
+// whole rows per warp) because eight warps with eight whole rows each would
+// need 0.5 MB of shared memory, and eight rows per warp because each vector
+// entry read from shared memory must serve several rows: 16 bytes of rows and
+// vectors per 32 FMAs.
+//
+// Each lane sums its chunks l, l + 32, ... in column order into one
+// accumulator per component, then the lanes are added over xor 16, 8, 4, 2, 1:
+// the order of k_stream_dot, so a rupture's result is the same bits alone or
+// in a batch.
+#include <cuda.h>
+
+#include <type_traits>
+
+#include "chunk.cuh"
+
+namespace s2w {
+
+namespace {
+
+constexpr int kWarps = 8;
+// Two warpgroups of consumers and one whose first lane produces.  The launch
+// gives every thread 168 registers; the producer group hands most of its
+// share to the consumers, whose accumulators and operands need ~200
+// (2 x 128 x 232 + 128 x 40 = 384 x 168).
+constexpr int kThreads = 32 * (kWarps + 4);
+constexpr int kRegsConsumer = 232, kRegsProducer = 40;
+constexpr int kRows = 64;             // most rows per tile: eight per warp
+constexpr int kSlabBytes = 512;       // of each row per stage: one 16-byte chunk per lane
+constexpr int kMaxStages = 16;
+constexpr int kBudget = 208 * 1024;   // ring bytes
+
+struct MultiArgs {
+  int n_vec, rows_per_vec, tiles, mrows;  // tiles of mrows rows per vector group
+  int slabs, stages;
+  int nb;
+  int x_vec_first;  // the vector map's dimensions are (entry, vector, rupture), else (entry, rupture, vector)
+  long long y_ldb;
+  float2* y;
+  int* status;
+  unsigned long long wait_ns;
+  int fault_skip;
+};
+
+__device__ __forceinline__ void tma_words(void* sdst, const CUtensorMap* tm, int c0, int c1, int c2, uint64_t* bar,
+                                          uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, "
+      "%4}], [%5], %6;" ::"r"(smem_u32(sdst)),
+      "l"(reinterpret_cast<uint64_t>(tm)), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar)), "l"(policy)
+      : "memory");
+}
+
+__device__ __forceinline__ uint64_t l2_policy_evict_last() {
+  uint64_t pol;
+  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
+  return pol;
+}
+
+template <int EL, bool HILO, int R>
+__global__ void __launch_bounds__(kThreads, 1)
+    k_stream_multi(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmAlo,
+                   const __grid_constant__ CUtensorMap tmX, const MultiArgs a) {
+  using CH = Chunk<EL>;
+  constexpr int C = CH::C;
+  constexpr int XB = 32 * C * 8;  // vector bytes per rupture and slab
+  constexpr int kWordsA = kSlabBytes / 4, kWordsX = XB / 4;
+  extern __shared__ __align__(128) unsigned char sm[];
+  const int S = a.stages;
+  uint64_t* full = reinterpret_cast<uint64_t*>(sm);
+  uint64_t* empty = full + kMaxStages;
+  const int a_bytes = a.mrows * kSlabBytes;
+  const int stage_bytes = a_bytes * (HILO ? 2 : 1) + R * XB;
+  unsigned char* ring = sm + 2 * 8 * kMaxStages;
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  const long long units = static_cast<long long>(a.n_vec) * a.tiles;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < S; ++s) {
+      mbar_init(full + s, 1);
+      mbar_init(empty + s, kWarps);
+    }
+    fence_mbar_init();
+  }
+  __syncthreads();
+
+  if (warp >= kWarps) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsProducer));
+    if (warp == kWarps && lane == 0) {
+      const uint64_t first = l2_policy_evict_first(), last = l2_policy_evict_last();
+      int it = 0, s = 0;
+      uint32_t ph = 1;  // parity of the empty barrier's phase (first lap passes)
+      bool ok = true;
+      for (long long u = blockIdx.x; u < units && ok; u += gridDim.x) {
+        const int vec = static_cast<int>(u / a.tiles), tile = static_cast<int>(u % a.tiles);
+        for (int k = 0; k < a.slabs; ++k, ++it) {
+          if (it >= S && !mbar_wait_bounded(empty + s, ph, a.status, DEV_ERR_TIMEOUT_EMPTY, a.wait_ns)) {
+            ok = false;
+            break;
+          }
+          if (!(a.fault_skip && it == 0)) {  // (test hook: stage 0 never fills)
+            unsigned char* st = ring + s * stage_bytes;
+            mbar_arrive_expect_tx(full + s, stage_bytes);
+            tma_words(st, &tmA, k * kWordsA, tile * a.mrows, vec, full + s, first);
+            if (HILO) tma_words(st + a_bytes, &tmAlo, k * kWordsA, tile * a.mrows, vec, full + s, first);
+            tma_words(st + a_bytes * (HILO ? 2 : 1), &tmX, k * kWordsX, a.x_vec_first ? vec : 0,
+                      a.x_vec_first ? 0 : vec, full + s, last);
+          }
+          if (++s == S) s = 0, ph ^= 1;
+        }
+      }
+      // never leave the CTA with copies in flight
+      for (int kk = (it > S ? it - S : 0); kk < it; ++kk)
+        mbar_wait_bounded(full + kk % S, (kk / S) & 1, a.status, DEV_ERR_TIMEOUT_FULL, a.wait_ns);
+    }
+    return;
+  }
+
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsConsumer));
+  int s = 0;
+  uint32_t ph = 0;
+  for (long long u = blockIdx.x; u < units; u += gridDim.x) {
+    const int vec = static_cast<int>(u / a.tiles), tile = static_cast<int>(u % a.tiles);
+    const int nr = min(a.mrows, a.rows_per_vec - tile * a.mrows);
+    // a full tile gives each warp eight adjacent rows (64-byte stores), a
+    // partial one deals its rows out over the warps
+    const bool whole = nr == kRows;
+    const int r_w = whole ? 8 : 1, r_i = whole ? 1 : 8;
+    const int row0 = warp * r_w;
+    float acc[8 * R * 2];
+#pragma unroll
+    for (int k = 0; k < 8 * R * 2; ++k) acc[k] = 0.f;
+    for (int k = 0; k < a.slabs; ++k) {
+      if (!mbar_wait_bounded(full + s, ph, a.status, DEV_ERR_TIMEOUT_FULL, a.wait_ns)) return;
+      const unsigned char* st = ring + s * stage_bytes;
+      const uint4* rows = reinterpret_cast<const uint4*>(st) + lane;
+      const uint4* rows_lo = reinterpret_cast<const uint4*>(st + a_bytes) + lane;
+      const float4* xs = reinterpret_cast<const float4*>(st + a_bytes * (HILO ? 2 : 1)) + lane * (C / 2);
+      auto slab = [&](auto whole_tag) {
+        constexpr bool WHOLE = decltype(whole_tag)::value;
+#pragma unroll
+        for (int h = 0; h < C / 2; ++h) {  // two entries of the lane's chunk at a time
+          float4 x[R];
+#pragma unroll
+          for (int b = 0; b < R; ++b) x[b] = xs[b * (XB / 16) + h];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int row = WHOLE ? row0 + i : row0 + 8 * i;
+            if (!WHOLE && row >= nr) continue;
+            float2 g[C];
+            CH::unpack(rows[row * (kSlabBytes / 16)], g);
+            if (HILO) {
+              float2 gl[C];
+              CH::unpack(rows_lo[row * (kSlabBytes / 16)], gl);
+#pragma unroll
+              for (int q = 0; q < C; ++q) g[q] = cadd(g[q], gl[q]);
+            }
+            const float2 g0 = g[2 * h], g1 = g[2 * h + 1];
+#pragma unroll
+            for (int b = 0; b < R; ++b) {
+              float& ar = acc[(i * R + b) * 2];
+              float& ai = acc[(i * R + b) * 2 + 1];
+              ar = fmaf(g0.x, x[b].x, ar);
+              ar = fmaf(-g0.y, x[b].y, ar);
+              ai = fmaf(g0.x, x[b].y, ai);
+              ai = fmaf(g0.y, x[b].x, ai);
+              ar = fmaf(g1.x, x[b].z, ar);
+              ar = fmaf(-g1.y, x[b].w, ar);
+              ai = fmaf(g1.x, x[b].w, ai);
+              ai = fmaf(g1.y, x[b].z, ai);
+            }
+          }
+        }
+      };
+      if (whole)
+        slab(std::true_type{});
+      else
+        slab(std::false_type{});
+      __syncwarp();
+      if (lane == 0) mbar_arrive(empty + s);
+      if (++s == S) s = 0, ph ^= 1;
+    }
+    // reduce-scatter over the lanes: after the step with lane bit o a lane
+    // keeps the half of its values that the bit selects, summed with its
+    // partner's; value index ((row * R) + b) * 2 + component
+#pragma unroll
+    for (int o = 16, n = 8 * R; o > 0; o >>= 1, n >>= 1) {
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int k = 0; k < 8 * R; ++k) {
+        if (k < n) {
+          const float keep = up ? acc[k + n] : acc[k];
+          const float send = up ? acc[k] : acc[k + n];
+          acc[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+      }
+    }
+    const int row = row0 + (lane >> 2) * r_i;
+    if (row < nr) {
+      float2* y = a.y + static_cast<long long>(vec) * a.rows_per_vec + tile * a.mrows + row;
+#pragma unroll
+      for (int j = 0; j < R / 2; ++j) {
+        const int v = (lane & 3) * (R / 2) + j;
+        if ((v >> 1) < a.nb) reinterpret_cast<float*>(y + (v >> 1) * a.y_ldb)[v & 1] = acc[j];
+      }
+    }
+  }
+}
+
+template <int EL, bool HILO, int R>
+cudaError_t launch_r(const StreamArgs& a, int num_sms, cudaStream_t st) {
+  using CH = Chunk<EL>;
+  constexpr int XB = 32 * CH::C * 8;
+  const long long row_bytes = static_cast<long long>(a.row_len) * (16 / CH::C);
+  MultiArgs m{};
+  m.rows_per_vec = static_cast<int>(a.rows_per_vec);
+  m.n_vec = static_cast<int>(a.F / a.rows_per_vec);
+  m.mrows = a.rows_per_vec >= kRows ? kRows : static_cast<int>((a.rows_per_vec + 7) / 8 * 8);
+  m.tiles = (m.rows_per_vec + m.mrows - 1) / m.mrows;
+  m.slabs = static_cast<int>((row_bytes + kSlabBytes - 1) / kSlabBytes);
+  const int stage = m.mrows * kSlabBytes * (HILO ? 2 : 1) + R * XB;
+  m.stages = kBudget / stage < kMaxStages ? kBudget / stage : kMaxStages;
+  m.nb = a.nb;
+  m.y = a.y;
+  m.y_ldb = a.y_ldb;
+  m.status = a.status;
+  m.wait_ns = a.wait_ns ? a.wait_ns : kWaitLimitNs;
+  m.fault_skip = a.fault_skip;
+  CUtensorMap ta, tl, tx;
+  cudaError_t e;
+  const long long vec_bytes = row_bytes * a.rows_per_vec;
+  if ((e = tc_encode_words(&ta, a.rows, row_bytes / 4, a.rows_per_vec, row_bytes, m.n_vec, vec_bytes, kSlabBytes / 4,
+                           m.mrows)) != cudaSuccess)
+    return e;
+  tl = ta;
+  if (HILO && (e = tc_encode_words(&tl, a.rows_lo, row_bytes / 4, a.rows_per_vec, row_bytes, m.n_vec, vec_bytes,
+                                   kSlabBytes / 4, m.mrows)) != cudaSuccess)
+    return e;
+  // ruptures past nb read as zeros (TMA fill); their sums are never stored.
+  // The map's dimensions go up in pitch
+  m.x_vec_first = a.x_stride < a.x_ldb ? 1 : 0;
+  e = m.x_vec_first
+          ? tc_encode_words(&tx, a.x, 2LL * a.row_len, m.n_vec, 8 * a.x_stride, a.nb, 8 * a.x_ldb, XB / 4, 1, R)
+          : tc_encode_words(&tx, a.x, 2LL * a.row_len, a.nb, 8 * a.x_ldb, m.n_vec, 8 * a.x_stride, XB / 4, R);
+  if (e != cudaSuccess) return e;
+  const size_t smem = 2 * 8 * kMaxStages + static_cast<size_t>(m.stages) * stage;
+  if ((e = cudaFuncSetAttribute(k_stream_multi<EL, HILO, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                static_cast<int>(smem))) != cudaSuccess)
+    return e;
+  long long grid = static_cast<long long>(m.n_vec) * m.tiles;
+  if (grid > num_sms) grid = num_sms;
+  k_stream_multi<EL, HILO, R><<<static_cast<unsigned>(grid), kThreads, smem, st>>>(ta, tl, tx, m);
+  return cudaGetLastError();
+}
+
+template <int EL, bool HILO>
+cudaError_t launch_el(const StreamArgs& a, int num_sms, cudaStream_t st) {
+  if (a.nb <= 2) return launch_r<EL, HILO, 2>(a, num_sms, st);
+  if (a.nb <= 4) return launch_r<EL, HILO, 4>(a, num_sms, st);
+  if (a.nb <= 6) return launch_r<EL, HILO, 6>(a, num_sms, st);
+  return launch_r<EL, HILO, 8>(a, num_sms, st);
+}
+
+}  // namespace
+
+cudaError_t launch_stream_multi(const StreamArgs& a, int num_sms, cudaStream_t st) {
+  if (a.nb < 2 || a.nb > kStreamMulti || a.rows_per_vec < 1 || a.rows_per_vec > 0x7fffffff - kRows ||
+      a.F % a.rows_per_vec != 0)
+    return cudaErrorInvalidValue;
+  switch (a.el) {
+    case EL_FP32: return launch_el<EL_FP32, false>(a, num_sms, st);
+    case EL_BF16: return launch_el<EL_BF16, false>(a, num_sms, st);
+    case EL_BF16_HILO: return launch_el<EL_BF16, true>(a, num_sms, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+}  // namespace s2w

@@ -1,7 +1,8 @@
 // Per-bin complex contractions on the HBM-streaming path (Alg. 2 step 3,
 // yhat_l = Fhat_l xhat_l, for a small rupture batch).
 //
-// Both stages are one kernel.  The resident spectrum is a sequence of F
+// Both stages are one kernel (batches of FP32 / BF16 rows: k_multi.cu, and
+// the R > 1 variants here for short rows).  The resident spectrum is a sequence of F
 // contiguous rows of `row_len` complex entries; row f is dotted with the
 // vector x_vec(f) = x + (f / rows_per_vec) * x_stride:
 //   stage 1: rows (l, i) of Ghat [l][i][Ns_pad], x_vec = shat_l     -> mhat[l][i]
@@ -30,8 +31,8 @@
 // pairs (y, y_lo).
 #include <type_traits>
 
+#include "chunk.cuh"
 #include "df.cuh"
-#include "s2w_internal.cuh"
 
 namespace s2w {
 
@@ -42,66 +43,6 @@ constexpr int kStages = 3;
 constexpr int kThreads = 32 * (kConsumerWarps + 1);
 constexpr int kMaxRowLen = 1024;
 constexpr int kStagesT = 2;  // ring depth of the transposed kernel (its reduction buffer needs the room)
-
-template <int EL>
-struct Chunk;  // complex entries per 16-byte chunk and how to unpack them
-
-template <>
-struct Chunk<EL_FP32> {
-  static constexpr int C = 2;
-  __device__ __forceinline__ static void unpack(const uint4& u, float2 (&g)[C]) {
-    g[0] = make_float2(__uint_as_float(u.x), __uint_as_float(u.y));
-    g[1] = make_float2(__uint_as_float(u.z), __uint_as_float(u.w));
-  }
-};
-
-__device__ __forceinline__ float2 bf2_to_f2(unsigned w) {
-  // bf16 -> f32 is exact: the 16 bits move to the top of the word
-  return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
-}
-
-template <>
-struct Chunk<EL_BF16> {
-  static constexpr int C = 4;
-  __device__ __forceinline__ static void unpack(const uint4& u, float2 (&g)[C]) {
-    g[0] = bf2_to_f2(u.x);
-    g[1] = bf2_to_f2(u.y);
-    g[2] = bf2_to_f2(u.z);
-    g[3] = bf2_to_f2(u.w);
-  }
-};
-
-// Two e4m3 values (bytes 0, 1 of a 16-bit word) widened exactly to an FP16
-// pair, and a 32-bit word's two such pairs.
-__device__ __forceinline__ __half2 e4m3x2_to_h2(unsigned short v) {
-  unsigned r;
-  asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(r) : "h"(v));
-  return *reinterpret_cast<const __half2*>(&r);
-}
-__device__ __forceinline__ void e4m3x4_to_h2(unsigned w, __half2& lo, __half2& hi) {
-  unsigned short l16, h16;
-  asm("mov.b32 {%0, %1}, %2;" : "=h"(l16), "=h"(h16) : "r"(w));
-  lo = e4m3x2_to_h2(l16);
-  hi = e4m3x2_to_h2(h16);
-}
-
-__device__ __forceinline__ float2 fp8x2_to_f2(unsigned short s) {
-  const __half2_raw h = __nv_cvt_fp8x2_to_halfraw2(static_cast<__nv_fp8x2_storage_t>(s), __NV_E4M3);
-  return __half22float2(*reinterpret_cast<const __half2*>(&h));
-}
-
-template <>
-struct Chunk<EL_FP8> {
-  static constexpr int C = 8;
-  __device__ __forceinline__ static void unpack(const uint4& u, float2 (&g)[C]) {
-    const unsigned w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      g[2 * k] = fp8x2_to_f2(static_cast<unsigned short>(w[k] & 0xffffu));
-      g[2 * k + 1] = fp8x2_to_f2(static_cast<unsigned short>(w[k] >> 16));
-    }
-  }
-};
 
 // EL selects the unpacker (EL_BF16 also serves the hi/lo pair when HILO);
 // SHORT: rows of at most 64 chunks, shared by lane groups; DF (with EL_FP32
@@ -114,11 +55,16 @@ __host__ __device__ constexpr int stream_warps(int el, bool short_rows) {
   return (el == EL_FP8 && short_rows) ? 12 : 8;
 }
 
-template <int EL, bool HILO, bool SHORT, bool DF = false>
+// R > 1 (short FP32 / BF16 rows): the row meets the vectors of R ruptures,
+// each lane's slices of all R held in registers, so a batch reads the
+// operator once per R ruptures.  Otherwise a batch takes one grid slice (y)
+// per rupture.
+template <int EL, bool HILO, bool SHORT, bool DF = false, int R = 1>
 __global__ void __launch_bounds__(32 * (stream_warps(EL, SHORT) + 1), 1)
     k_stream_dot(const StreamArgs a, int stage_rows) {
   constexpr int kConsumerWarps = stream_warps(EL, SHORT);
   static_assert(!DF || (EL == EL_FP32 && HILO), "pair rows: FP32 hi and lo arrays");
+  static_assert(R == 1 || (SHORT && !DF && EL != EL_FP8), "several vectors: short FP32 or BF16 rows");
   using CH = Chunk<EL>;
   constexpr int C = CH::C;
   // chunk slots per lane: a short row gives each lane at most four chunks
@@ -136,6 +82,8 @@ __global__ void __launch_bounds__(32 * (stream_warps(EL, SHORT) + 1), 1)
   const long long r1 = a.F * (blockIdx.x + 1) / gridDim.x;
   const int nst = static_cast<int>((r1 - r0 + stage_rows - 1) / stage_rows);
   const unsigned long long wlim = a.wait_ns ? a.wait_ns : kWaitLimitNs;
+  const float2* const ax = a.x + blockIdx.y * a.x_ldb;
+  float2* const ay = a.y + blockIdx.y * a.y_ldb;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -184,7 +132,7 @@ __global__ void __launch_bounds__(32 * (stream_warps(EL, SHORT) + 1), 1)
   const int sub = lane % lpr;   // lane within its row group
   const int grp = lane / lpr;   // row group within the warp
   constexpr bool F8 = EL == EL_FP8;
-  float2 xr[F8 ? 1 : T][F8 ? 1 : C];
+  float2 xr[R][F8 ? 1 : T][F8 ? 1 : C];
   float2 xl[DF ? T : 1][DF ? C : 1];  // DF: low-order parts of x_vec
   // FP8: x_vec times a power of two sx (max |component| into [2, 4)) as FP16
   // pairs (Re, Re) and (Im, Im) for the packed products, and 1 / sx
@@ -209,7 +157,7 @@ __global__ void __launch_bounds__(32 * (stream_warps(EL, SHORT) + 1), 1)
           if (rs + base + j >= vec_end) {  // warp-uniform: every lane works on the same rows
             vec = (rs + base + j) / a.rows_per_vec;
             vec_end = (vec + 1) * a.rows_per_vec;
-            const float4* xv = reinterpret_cast<const float4*>(a.x + vec * a.x_stride);
+            const float4* xv = reinterpret_cast<const float4*>(ax + vec * a.x_stride);
             float amax = 0.f;
 #pragma unroll
             for (int t = 0; t < T; ++t) {
@@ -316,7 +264,7 @@ __global__ void __launch_bounds__(32 * (stream_warps(EL, SHORT) + 1), 1)
           if ((lane & 3) == 0 && r >= j && r < je) {
             const long long f = rs + base + r;
             const float sc = a.scale[vec * a.nblk + (f - (vec_end - a.rows_per_vec)) / 256] * x_unscale;
-            reinterpret_cast<float*>(a.y + f)[idx & 1] = v[0] * sc;
+            reinterpret_cast<float*>(ay + f)[idx & 1] = v[0] * sc;
           }
           j = je;
         }
@@ -338,7 +286,7 @@ __global__ void __launch_bounds__(32 * (stream_warps(EL, SHORT) + 1), 1)
       if (f >= vec_end) {
         vec = f / a.rows_per_vec;
         vec_end = (vec + 1) * a.rows_per_vec;
-        const float4* xv = reinterpret_cast<const float4*>(a.x + vec * a.x_stride);
+        const float4* xv = reinterpret_cast<const float4*>(ax + vec * a.x_stride);
         if constexpr (F8) {
           // two passes over the lane's slice (cached loads): the largest
           // magnitude over the row group's whole vector, then the scaled
@@ -377,11 +325,16 @@ __global__ void __launch_bounds__(32 * (stream_warps(EL, SHORT) + 1), 1)
             const int c = sub + lpr * t;
 #pragma unroll
             for (int q = 0; q < C / 2; ++q) {
-              const float4 v = (c < nchunk) ? __ldg(xv + c * (C / 2) + q) : make_float4(0.f, 0.f, 0.f, 0.f);
-              xr[t][2 * q] = make_float2(v.x, v.y);
-              xr[t][2 * q + 1] = make_float2(v.z, v.w);
+#pragma unroll
+              for (int b = 0; b < R; ++b) {  // (slots past the last rupture repeat it; never stored)
+                const float4* xb = b == 0 ? xv : xv + min(b, a.nb - 1) * (a.x_ldb / 2);
+                const float4 v = (c < nchunk) ? __ldg(xb + c * (C / 2) + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+                xr[b][t][2 * q] = make_float2(v.x, v.y);
+                xr[b][t][2 * q + 1] = make_float2(v.z, v.w);
+              }
               if constexpr (DF) {
-                const float4* xvl = reinterpret_cast<const float4*>(a.x_lo + vec * a.x_stride);
+                const float4* xvl =
+                    reinterpret_cast<const float4*>(a.x_lo + blockIdx.y * a.x_ldb + vec * a.x_stride);
                 const float4 w = (c < nchunk) ? __ldg(xvl + c * (C / 2) + q) : make_float4(0.f, 0.f, 0.f, 0.f);
                 xl[t][2 * q] = make_float2(w.x, w.y);
                 xl[t][2 * q + 1] = make_float2(w.z, w.w);
@@ -407,7 +360,7 @@ __global__ void __launch_bounds__(32 * (stream_warps(EL, SHORT) + 1), 1)
 #pragma unroll
             for (int q = 0; q < C; ++q) {
               const dfl gr{g[q].x, gl[q].x}, gi{g[q].y, gl[q].y};
-              const dfl xre{xr[t][q].x, xl[t][q].x}, xim{xr[t][q].y, xl[t][q].y};
+              const dfl xre{xr[0][t][q].x, xl[t][q].x}, xim{xr[0][t][q].y, xl[t][q].y};
               acc_mac(sr[q & 1], gr, xre);
               acc_mac(sr[q & 1], df_neg(gi), xim);
               acc_mac(si[q & 1], gr, xim);
@@ -424,8 +377,8 @@ __global__ void __launch_bounds__(32 * (stream_warps(EL, SHORT) + 1), 1)
         }
         if (valid && sub == 0) {
           const dfl yr = acc_get(ar), yi = acc_get(ai);
-          a.y[f] = make_float2(yr.hi, yi.hi);
-          a.y_lo[f] = make_float2(yr.lo, yi.lo);
+          ay[f] = make_float2(yr.hi, yi.hi);
+          a.y_lo[blockIdx.y * a.y_ldb + f] = make_float2(yr.lo, yi.lo);
         }
       } else if constexpr (F8) {
         // e4m3 pairs (Re, Im) widen exactly to FP16 pairs (one cvt per
@@ -468,41 +421,50 @@ __global__ void __launch_bounds__(32 * (stream_warps(EL, SHORT) + 1), 1)
         }
         if (valid && sub == 0) {
           const float sc = a.scale[vec * a.nblk + (f - (vec_end - a.rows_per_vec)) / 256] * x_unscale;
-          a.y[f] = make_float2(ar * sc, ai * sc);
+          ay[f] = make_float2(ar * sc, ai * sc);
         }
       } else {
-      float ar0 = 0.f, ai0 = 0.f, ar1 = 0.f, ai1 = 0.f;
+        // one chain per rupture and component, in column order: the order of
+        // k_stream_multi, so a rupture's result does not depend on the batch
+        float ar[R], ai[R];
 #pragma unroll
-      for (int t = 0; t < T; ++t) {
-        const int c = sub + lpr * t;
-        if (valid && c < nchunk) {
-          float2 g[C];
-          CH::unpack(row[c], g);
-          if (HILO) {
-            float2 gl[C];
-            CH::unpack(row_lo[c], gl);
+        for (int b = 0; b < R; ++b) ar[b] = ai[b] = 0.f;
 #pragma unroll
-            for (int q = 0; q < C; ++q) g[q] = cadd(g[q], gl[q]);
-          }
+        for (int t = 0; t < T; ++t) {
+          const int c = sub + lpr * t;
+          if (valid && c < nchunk) {
+            float2 g[C];
+            CH::unpack(row[c], g);
+            if (HILO) {
+              float2 gl[C];
+              CH::unpack(row_lo[c], gl);
 #pragma unroll
-          for (int q = 0; q < C; q += 2) {
-            ar0 = fmaf(g[q].x, xr[t][q].x, ar0);
-            ar0 = fmaf(-g[q].y, xr[t][q].y, ar0);
-            ai0 = fmaf(g[q].x, xr[t][q].y, ai0);
-            ai0 = fmaf(g[q].y, xr[t][q].x, ai0);
-            ar1 = fmaf(g[q + 1].x, xr[t][q + 1].x, ar1);
-            ar1 = fmaf(-g[q + 1].y, xr[t][q + 1].y, ar1);
-            ai1 = fmaf(g[q + 1].x, xr[t][q + 1].y, ai1);
-            ai1 = fmaf(g[q + 1].y, xr[t][q + 1].x, ai1);
+              for (int q = 0; q < C; ++q) g[q] = cadd(g[q], gl[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < C; ++q) {
+#pragma unroll
+              for (int b = 0; b < R; ++b) {
+                ar[b] = fmaf(g[q].x, xr[b][t][q].x, ar[b]);
+                ar[b] = fmaf(-g[q].y, xr[b][t][q].y, ar[b]);
+                ai[b] = fmaf(g[q].x, xr[b][t][q].y, ai[b]);
+                ai[b] = fmaf(g[q].y, xr[b][t][q].x, ai[b]);
+              }
+            }
           }
         }
-      }
-      float ar = ar0 + ar1, ai = ai0 + ai1;
-      for (int o = lpr / 2; o > 0; o >>= 1) {
-        ar += __shfl_xor_sync(0xffffffffu, ar, o);
-        ai += __shfl_xor_sync(0xffffffffu, ai, o);
-      }
-      if (valid && sub == 0) a.y[f] = make_float2(ar, ai);
+        for (int o = lpr / 2; o > 0; o >>= 1) {
+#pragma unroll
+          for (int b = 0; b < R; ++b) {
+            ar[b] += __shfl_xor_sync(0xffffffffu, ar[b], o);
+            ai[b] += __shfl_xor_sync(0xffffffffu, ai[b], o);
+          }
+        }
+        if (valid && sub == 0) {
+#pragma unroll
+          for (int b = 0; b < R; ++b)
+            if (R == 1 || b < a.nb) ay[b * a.y_ldb + f] = make_float2(ar[b], ai[b]);
+        }
       }
     }
     __syncwarp();
@@ -682,7 +644,7 @@ cudaError_t launch_tt(const StreamTArgs& a, int num_sms, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-template <int EL, bool HILO, bool SHORT, bool DF = false>
+template <int EL, bool HILO, bool SHORT, bool DF = false, int R = 1>
 cudaError_t launch_t(const StreamArgs& a, int num_sms, cudaStream_t st) {
   constexpr int C = Chunk<EL>::C;
   const int row_bytes = a.row_len * (16 / C);
@@ -691,14 +653,14 @@ cudaError_t launch_t(const StreamArgs& a, int num_sms, cudaStream_t st) {
   if (stage_rows >= 8) stage_rows -= stage_rows % 8;
   if (stage_rows < 1) stage_rows = 1;
   const size_t smem = 128 + static_cast<size_t>(kStages) * stage_rows * row_bytes * (HILO ? 2 : 1);
-  cudaError_t e = cudaFuncSetAttribute(k_stream_dot<EL, HILO, SHORT, DF>,
+  cudaError_t e = cudaFuncSetAttribute(k_stream_dot<EL, HILO, SHORT, DF, R>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   long long grid = num_sms;
   if (grid > a.F) grid = a.F;
   if (grid < 1) grid = 1;
-  k_stream_dot<EL, HILO, SHORT, DF><<<static_cast<unsigned>(grid), 32 * (stream_warps(EL, SHORT) + 1), smem, st>>>(
-      a, stage_rows);
+  const dim3 g(static_cast<unsigned>(grid), R == 1 ? static_cast<unsigned>(a.nb) : 1u);
+  k_stream_dot<EL, HILO, SHORT, DF, R><<<g, 32 * (stream_warps(EL, SHORT) + 1), smem, st>>>(a, stage_rows);
   return cudaGetLastError();
 }
 
@@ -708,19 +670,38 @@ bool short_rows(const StreamArgs& a, int C) { return a.row_len / C <= 64; }
 
 }  // namespace
 
+namespace {
+// One launch for a.nb ruptures of FP32 / BF16 storage (nb <= kStreamMulti).
+template <int EL, bool HILO>
+cudaError_t launch_plain(const StreamArgs& a, int num_sms, cudaStream_t st) {
+  if (!short_rows(a, Chunk<EL>::C))
+    return a.nb == 1 ? launch_t<EL, HILO, false>(a, num_sms, st) : launch_stream_multi(a, num_sms, st);
+  if (a.nb == 1) return launch_t<EL, HILO, true>(a, num_sms, st);
+  if (a.nb == 2) return launch_t<EL, HILO, true, false, 2>(a, num_sms, st);
+  if (a.nb <= 4) return launch_t<EL, HILO, true, false, 4>(a, num_sms, st);
+  if constexpr (EL == EL_FP32) {  // a lane's slices of eight vectors: 128 registers
+    return launch_t<EL, HILO, true, false, 8>(a, num_sms, st);
+  } else {  // BF16 chunks hold twice the entries: four vectors at a time
+    StreamArgs h = a;
+    h.nb = 4;
+    const cudaError_t e = launch_t<EL, HILO, true, false, 4>(h, num_sms, st);
+    if (e != cudaSuccess) return e;
+    h.nb = a.nb - 4;
+    h.x = a.x + 4 * a.x_ldb;
+    h.y = a.y + 4 * a.y_ldb;
+    return launch_t<EL, HILO, true, false, 4>(h, num_sms, st);
+  }
+}
+}  // namespace
+
 cudaError_t launch_stream_dot(const StreamArgs& a, int num_sms, cudaStream_t st) {
-  if (a.F <= 0) return cudaSuccess;
-  if (a.row_len <= 0 || a.row_len > kMaxRowLen || (a.row_len % 8) != 0) return cudaErrorInvalidValue;
+  if (a.F <= 0 || a.nb <= 0) return cudaSuccess;
+  if (a.row_len <= 0 || a.row_len > kMaxRowLen || (a.row_len % 8) != 0 || a.nb > kStreamMulti)
+    return cudaErrorInvalidValue;
   switch (a.el) {
-    case EL_FP32:
-      return short_rows(a, 2) ? launch_t<EL_FP32, false, true>(a, num_sms, st)
-                              : launch_t<EL_FP32, false, false>(a, num_sms, st);
-    case EL_BF16:
-      return short_rows(a, 4) ? launch_t<EL_BF16, false, true>(a, num_sms, st)
-                              : launch_t<EL_BF16, false, false>(a, num_sms, st);
-    case EL_BF16_HILO:
-      return short_rows(a, 4) ? launch_t<EL_BF16, true, true>(a, num_sms, st)
-                              : launch_t<EL_BF16, true, false>(a, num_sms, st);
+    case EL_FP32: return launch_plain<EL_FP32, false>(a, num_sms, st);
+    case EL_BF16: return launch_plain<EL_BF16, false>(a, num_sms, st);
+    case EL_BF16_HILO: return launch_plain<EL_BF16, true>(a, num_sms, st);
     case EL_FP8:
       return short_rows(a, 8) ? launch_t<EL_FP8, false, true>(a, num_sms, st)
                               : launch_t<EL_FP8, false, false>(a, num_sms, st);

@@ -1677,6 +1677,21 @@ cudaError_t tc_encode_3d_u8(CUtensorMap* out, const void* base, long long K, lon
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+cudaError_t tc_encode_words(CUtensorMap* out, const void* base, long long words, long long rows, long long row_pitch,
+                            long long nbatch, long long batch_pitch, int box_words, int box_rows, int box_batch) {
+  if (g_encode == nullptr && resolve_encode() != cudaSuccess) return cudaErrorNotSupported;
+  const cuuint64_t dims[3] = {static_cast<cuuint64_t>(words), static_cast<cuuint64_t>(rows),
+                              static_cast<cuuint64_t>(nbatch)};
+  const cuuint64_t strides[2] = {static_cast<cuuint64_t>(row_pitch), static_cast<cuuint64_t>(batch_pitch)};
+  const cuuint32_t box[3] = {static_cast<cuuint32_t>(box_words), static_cast<cuuint32_t>(box_rows),
+                             static_cast<cuuint32_t>(box_batch)};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = g_encode(out, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, const_cast<void*>(base), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 int tc_block_k(int N, int split, int pair) {
   if (pair) {  // half of B per CTA: 128-byte swizzle whenever four such stages fit
     const int stage64 = (kBlockM + N / 2) * 64 * 2 * (1 + split);

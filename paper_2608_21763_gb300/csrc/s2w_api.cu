@@ -4,9 +4,9 @@
 // Pipeline of one s2w_waveforms call (Alg. 1 steps 2-4, each matvec by
 // Alg. 2):
 //   K1  rfft of every slip row, zero-padded to 2 Nt      -> shat [l][b][Ns_pad]
-//   per rupture b:
-//     K2  stage-1 per-bin contraction (HBM stream of Ghat) -> mhat [l][Ng]
-//     K3  IFFT + Truncate, D_t, ZeroPad + FFT              -> vhat [l][nseg*RL]
+//   per pass of up to 8 ruptures b:
+//     K2  stage-1 per-bin contraction (HBM stream of Ghat) -> mhat [b][l][Ng]
+//     K3  IFFT + Truncate, D_t, ZeroPad + FFT              -> vhat [b][l][nseg*RL]
 //     K4  stage-2 per-bin contraction over grid segments   -> partial [b][l][seg][o]
 //   K5  sum of segment partials (the in-device ReduceSum of Alg. 1 step 5)
 //       fused with IFFT + Truncate                        -> q [b][o][Nt]
@@ -50,8 +50,9 @@ struct s2w_ctx {
   // workspaces
   float* ws_slip = nullptr;
   float2* ws_shat = nullptr;
-  float2* ws_mhat = nullptr;
-  float2* ws_vhat = nullptr;
+  int multi = 1;               // ruptures per streaming launch: ws_mhat, ws_vhat hold this many
+  float2* ws_mhat = nullptr;   // [multi][Nb][Ng]
+  float2* ws_vhat = nullptr;   // [multi][Nb][nseg * RL]
   float2* ws_part = nullptr;
   float* ws_q = nullptr;
   float* ws_seafloor = nullptr;
@@ -908,9 +909,6 @@ int s2w_create(int Ns, int Ng, int No, int Nt, const s2w_opts* opts, s2w_ctx** o
     const long long Bsh = std::min<long long>(B, kStreamGroup);
     if ((e = dalloc(&ctx->ws_shat_lo, sizeof(float2) * Nb * Bsh * ctx->Ns_pad)) != cudaSuccess)
       return bad(e, "slip spectra lo");
-    if ((e = dalloc(&ctx->ws_mhat_lo, sizeof(float2) * Nb * Ng)) != cudaSuccess) return bad(e, "seafloor spectra lo");
-    if ((e = dalloc(&ctx->ws_vhat_lo, sizeof(float2) * Nb * ctx->nseg * ctx->RL)) != cudaSuccess)
-      return bad(e, "velocity spectra lo");
     if ((e = dalloc(&ctx->ws_part_lo, sizeof(float2) * Bsh * Nb * ctx->nseg * No)) != cudaSuccess)
       return bad(e, "stage-2 partials lo");
   }
@@ -919,9 +917,6 @@ int s2w_create(int Ns, int Ng, int No, int Nt, const s2w_opts* opts, s2w_ctx** o
   const long long Bsh = std::min<long long>(B, 256);  // slip spectra serve one group / sub-batch at a time
   if ((e = dalloc(&ctx->ws_shat, sizeof(float2) * Nb * Bsh * ctx->Ns_pad)) != cudaSuccess)
     return bad(e, "slip spectra");
-  if ((e = dalloc(&ctx->ws_mhat, sizeof(float2) * Nb * Ng)) != cudaSuccess) return bad(e, "seafloor spectra");
-  if ((e = dalloc(&ctx->ws_vhat, sizeof(float2) * Nb * ctx->nseg * ctx->RL)) != cudaSuccess)
-    return bad(e, "velocity spectra");
   if ((e = dalloc(&ctx->ws_part, sizeof(float2) * std::min<long long>(B, kStreamGroup) * Nb * ctx->nseg * No)) !=
       cudaSuccess)
     return bad(e, "stage-2 partials");
@@ -1052,6 +1047,24 @@ int s2w_create(int Ns, int Ng, int No, int Nt, const s2w_opts* opts, s2w_ctx** o
       if (ctx->tc_adj &&
           (e = upload(true, &ctx->tc_Ta, &ctx->tc_Ta_lo, &ctx->tc_tmTa, &ctx->tc_tmTa2, &ctx->tc_tmTap)) != cudaSuccess)
         return bad(e, "adjoint retransform matrix");
+    }
+  }
+  // Seafloor and velocity spectra of the streaming kernels, last: room for
+  // kStreamMulti ruptures per launch when that takes at most 1/8 of the
+  // memory still free, for fewer (at least the one that every call needs)
+  // otherwise.  Results do not depend on the count.
+  {
+    const size_t mh = sizeof(float2) * Nb * Ng, vh = sizeof(float2) * Nb * ctx->nseg * ctx->RL;
+    size_t free_b = 0, total_b = 0;
+    if ((e = cudaMemGetInfo(&free_b, &total_b)) != cudaSuccess) return bad(e, "free memory");
+    int m = static_cast<int>(std::min<long long>(B, kStreamMulti));
+    while (m > 1 && static_cast<size_t>(m) * (mh + vh) * (ctx->df ? 2 : 1) > free_b / 8) m /= 2;
+    ctx->multi = m;
+    if ((e = dalloc(&ctx->ws_mhat, m * mh)) != cudaSuccess) return bad(e, "seafloor spectra");
+    if ((e = dalloc(&ctx->ws_vhat, m * vh)) != cudaSuccess) return bad(e, "velocity spectra");
+    if (ctx->df) {
+      if ((e = dalloc(&ctx->ws_mhat_lo, m * mh)) != cudaSuccess) return bad(e, "seafloor spectra lo");
+      if ((e = dalloc(&ctx->ws_vhat_lo, m * vh)) != cudaSuccess) return bad(e, "velocity spectra lo");
     }
   }
   if ((e = launch_twiddles(ctx->tw, ctx->L, nullptr)) != cudaSuccess) return bad(e, "twiddles");
@@ -1388,8 +1401,13 @@ int s2w_waveforms(s2w_ctx* ctx, const float* slip, int B, float* q, float* seafl
                             ctx->cur_lens ? ctx->cur_lens + g0 : nullptr));
     }
     const long long part_b = Nb * ctx->nseg * No;
-    for (int b = 0; b < Bg; ++b) {
-      const long long bg = g0 + b;  // rupture index in the call
+    const long long vcols = static_cast<long long>(ctx->nseg) * ctx->RL;
+    const long long mhat_b = Nb * Ng, vhat_b = Nb * vcols;  // per rupture
+    // the group's ruptures in equal passes of at most ctx->multi
+    const int npass = (Bg + ctx->multi - 1) / ctx->multi;
+    for (int p = 0, b = 0, nb = 0; p < npass; ++p, b += nb) {
+      nb = (Bg - b + npass - p - 1) / (npass - p);
+      const long long bg = g0 + b;  // first rupture of the pass, in the call
       // K2
       StreamArgs a1{};
       a1.rows = ctx->G;
@@ -1397,12 +1415,15 @@ int s2w_waveforms(s2w_ctx* ctx, const float* slip, int B, float* q, float* seafl
       a1.F = Nb * Ng;
       a1.row_len = static_cast<int>(Ns_pad);
       a1.el = ctx->opts.prec_g;
+      a1.nb = nb;
       a1.x = ctx->ws_shat + b * Ns_pad;
       a1.x_stride = Bg * Ns_pad;
+      a1.x_ldb = Ns_pad;
       a1.rows_per_vec = Ng;
       a1.scale = ctx->G_scale;
       a1.nblk = ctx->nblk;
       a1.y = ctx->ws_mhat;
+      a1.y_ldb = mhat_b;
       if (ctx->df) {
         a1.x_lo = ctx->ws_shat_lo + b * Ns_pad;
         a1.y_lo = ctx->ws_mhat_lo;
@@ -1415,36 +1436,45 @@ int s2w_waveforms(s2w_ctx* ctx, const float* slip, int B, float* q, float* seafl
         CK(launch_stream_dot(a1, ctx->num_sms, st));
       }
       // K3
-      float* sf = nullptr;
-      if (seafloor) sf = kf == 1 ? seafloor + bg * Ng * Nt : ctx->ws_seafloor;
       if (ctx->single_pass) {  // mhat goes to stage 2 as it is, in the segment layout
         StageTimer t(ctx, 2, st, 0);
-        CK(cudaMemcpy2DAsync(ctx->ws_vhat, sizeof(float2) * ctx->nseg * ctx->RL, ctx->ws_mhat, sizeof(float2) * Ng,
-                             sizeof(float2) * Ng, Nb, cudaMemcpyDeviceToDevice, st));
-      } else if (ctx->df) {
-        StageTimer t(ctx, 2, st);
-        CK(launch_df_retransform(ctx->ws_mhat, ctx->ws_mhat_lo, Ng, Ng, static_cast<int>(Nt), ctx->tw_df,
-                                 1.0 / ctx->opts.dt, ctx->opts.dt_mode, ctx->ws_vhat, ctx->ws_vhat_lo,
-                                 static_cast<long long>(ctx->nseg) * ctx->RL, sf, st));
+        CK(cudaMemcpy2DAsync(ctx->ws_vhat, sizeof(float2) * vcols, ctx->ws_mhat, sizeof(float2) * Ng,
+                             sizeof(float2) * Ng, nb * Nb, cudaMemcpyDeviceToDevice, st));
       } else {
-        StageTimer t(ctx, 2, st);
-        CK(launch_retransform(ctx->ws_mhat, Ng, Ng, static_cast<int>(Nt), ctx->tw,
-                              static_cast<float>(1.0 / ctx->opts.dt), ctx->opts.dt_mode, ctx->ws_vhat,
-                              static_cast<long long>(ctx->nseg) * ctx->RL, sf, st));
+        // a seafloor field in host memory goes through a buffer for one rupture
+        const bool one = seafloor != nullptr && kf == 0;
+        for (int k = 0; k < nb; k += one ? 1 : nb) {
+          float* sf = seafloor == nullptr ? nullptr : (one ? ctx->ws_seafloor : seafloor + bg * Ng * Nt);
+          {
+            StageTimer t(ctx, 2, st);
+            if (ctx->df)
+              CK(launch_df_retransform(ctx->ws_mhat + k * mhat_b, ctx->ws_mhat_lo + k * mhat_b, Ng, Ng,
+                                       static_cast<int>(Nt), ctx->tw_df, 1.0 / ctx->opts.dt, ctx->opts.dt_mode,
+                                       ctx->ws_vhat + k * vhat_b, ctx->ws_vhat_lo + k * vhat_b, vcols, sf, st,
+                                       one ? 1 : nb, mhat_b, vhat_b));
+            else
+              CK(launch_retransform(ctx->ws_mhat + k * mhat_b, Ng, Ng, static_cast<int>(Nt), ctx->tw,
+                                    static_cast<float>(1.0 / ctx->opts.dt), ctx->opts.dt_mode,
+                                    ctx->ws_vhat + k * vhat_b, vcols, sf, st, one ? 1 : nb, mhat_b, vhat_b));
+          }
+          if (one)
+            CK(cudaMemcpyAsync(seafloor + (bg + k) * Ng * Nt, ctx->ws_seafloor, sizeof(float) * Ng * Nt,
+                               cudaMemcpyDeviceToHost, st));
+        }
       }
-      if (seafloor && kf == 0)
-        CK(cudaMemcpyAsync(seafloor + bg * Ng * Nt, ctx->ws_seafloor, sizeof(float) * Ng * Nt,
-                           cudaMemcpyDeviceToHost, st));
       // K4
       StreamArgs a2{};
       a2.rows = ctx->P;
       a2.F = Nb * ctx->nseg * No;
       a2.row_len = ctx->RL;
       a2.el = ctx->opts.prec_p;
+      a2.nb = nb;
       a2.x = ctx->ws_vhat;
       a2.x_stride = ctx->RL;
+      a2.x_ldb = vhat_b;
       a2.rows_per_vec = No;
       a2.y = ctx->ws_part + b * part_b;
+      a2.y_ldb = part_b;
       if (ctx->df) {
         a2.rows_lo = ctx->P_lo;
         a2.x_lo = ctx->ws_vhat_lo;
@@ -1931,13 +1961,16 @@ int s2w_autotune(s2w_ctx* ctx, int B, s2w_tuning* out, void* stream) {
       set_s2_chunks(ctx, best_c);
     }
     r.tc_s2_chunks = ctx->tc_nkc;
-    // 3. the smallest batch whose tensor pass beats that many stream passes
+    // 3. the smallest batch whose tensor pass beats the stream engine
     const int sizes[7] = {1, 2, 4, 8, 16, 32, 64};
     int min_b = 0;
     for (int k = 0; k < 7 && rc == S2W_OK; ++k) {
       if (sizes[k] > B || sizes[k] > ctx->tc_bsub) break;
       rc = timed(sizes[k], S2W_ENGINE_TENSOR, &r.ms_tensor_batch[k]);
-      if (rc == S2W_OK && min_b == 0 && r.ms_tensor_batch[k] < sizes[k] * r.ms_stream_per_rupture) min_b = sizes[k];
+      if (rc != S2W_OK || min_b != 0) continue;
+      float ms_stream = r.ms_stream_per_rupture;  // the stream engine on the same batch
+      if (sizes[k] > 1) rc = timed(sizes[k], S2W_ENGINE_STREAM, &ms_stream);
+      if (rc == S2W_OK && r.ms_tensor_batch[k] < ms_stream) min_b = sizes[k];
     }
     if (min_b == 0) min_b = r.ms_tensor_batch[0] > 0.f ? ctx->tc_bsub + 1 : ctx->tc_min_batch;
     ctx->tc_min_batch = min_b;
@@ -2121,6 +2154,7 @@ extern "C" int s2w_waveforms_noalloc(s2w_ctx* ctx, const float* slip, float* q, 
   a1.F = Nb * Ng;
   a1.row_len = static_cast<int>(Ns_pad);
   a1.el = ctx->opts.prec_g;
+  a1.nb = 1;
   a1.x = shat;
   a1.x_lo = shat_lo;
   a1.x_stride = Ns_pad;
@@ -2143,6 +2177,7 @@ extern "C" int s2w_waveforms_noalloc(s2w_ctx* ctx, const float* slip, float* q, 
   a2.F = Nb * ctx->nseg * No;
   a2.row_len = ctx->RL;
   a2.el = ctx->opts.prec_p;
+  a2.nb = 1;
   a2.x = vhat;
   a2.x_lo = vhat_lo;
   a2.x_stride = ctx->RL;

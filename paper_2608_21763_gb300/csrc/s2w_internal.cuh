@@ -172,11 +172,12 @@ cudaError_t launch_twiddles_df(float4* tw, int L, cudaStream_t st);
 cudaError_t launch_df_rfft_rows(const float* x, long long rows, int n_in, int Nt, const float4* tw, float2* X,
                                 float2* X_lo, long long ld_l, long long rows_a, long long ld_a, cudaStream_t st,
                                 const int* lens = nullptr);
-// launch_retransform of one rupture with pairs in and out (dt_mode BACKWARD
-// or NONE; seafloor optional, rounded to FP32).
+// launch_retransform with pairs in and out (dt_mode BACKWARD or NONE;
+// seafloor optional, rounded to FP32).
 cudaError_t launch_df_retransform(const float2* mhat, const float2* mhat_lo, long long Ng, long long ld_m, int Nt,
                                   const float4* tw, double inv_dt, int dt_mode, float2* vhat, float2* vhat_lo,
-                                  long long ld_v, float* seafloor, cudaStream_t st);
+                                  long long ld_v, float* seafloor, cudaStream_t st, int nb = 1,
+                                  long long mhat_ld_b = 0, long long vhat_ld_b = 0);
 // launch_reduce_irfft with pair partials (FP32 output).
 cudaError_t launch_df_reduce_irfft(const float2* part, const float2* part_lo, int B, int No, int nseg, int Nt,
                                    long long s_b, long long s_l, long long s_s, const float4* tw, float* q,
@@ -202,8 +203,17 @@ struct StreamArgs {
   int* status;
   unsigned long long wait_ns;  // bound of every wait (0: kWaitLimitNs)
   int fault_skip;              // test hook: 1 = the producer skips its first copy (consumers' waits run out)
+  int nb;                      // ruptures (1 .. kStreamMulti); rupture b: x + b * x_ldb -> y + b * y_ldb
+  long long x_ldb, y_ldb;      // (x_lo and y_lo alike)
 };
+// Ruptures that one streaming launch takes: FP32 and BF16 rows meet them all
+// while the row is in shared memory, so the operator is read once for them.
+constexpr int kStreamMulti = 8;
 cudaError_t launch_stream_dot(const StreamArgs& a, int num_sms, cudaStream_t st);
+
+// k_multi.cu: the same for 2 .. kStreamMulti ruptures and FP32 / BF16 /
+// BF16 hi/lo rows of more than 64 16-byte chunks (launch_stream_dot calls it).
+cudaError_t launch_stream_multi(const StreamArgs& a, int num_sms, cudaStream_t st);
 
 // k_stream.cu, transposed: y[u][c] = sum_{f in unit u} conj(rows[f][c]) w_f,
 // unit u = chunk (u % nchunk) of Rc rows of group (u / nchunk) of G1 rows,
@@ -273,6 +283,10 @@ cudaError_t tc_encode_3d(CUtensorMap* out, const void* base, long long K, long l
 // K block (BF16 elements per swizzle row) and ring depth for N MMA columns
 // with `terms` = 1 + a_lo + b_lo operand tiles beyond the first A and B
 int tc_block_k(int N, int split = 0, int pair = 0);
+// Tensor map of 32-bit words, no swizzle: [nbatch][rows][words] with the
+// given byte pitches, boxes of box_words x box_rows x box_batch.
+cudaError_t tc_encode_words(CUtensorMap* out, const void* base, long long words, long long rows, long long row_pitch,
+                            long long nbatch, long long batch_pitch, int box_words, int box_rows, int box_batch = 1);
 int tc_stages_for(int N, int a_lo = 0, int b_lo = 0, int fp8 = 0, int mt = 1);
 int tc_stages_pair(int N, int split, int fp8 = 0);
 // Byte tensor map for FP8 A tiles: [nbatch][rows][K] bytes, box bk x box_rows, no swizzle
