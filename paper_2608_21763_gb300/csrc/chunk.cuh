@@ -66,4 +66,23 @@ struct Chunk<EL_FP8> {
   }
 };
 
+// Complex products on packed FP32 pairs: a stream of scalar FFMAs with three
+// register operands reaches 25.3 TFMA/s on this GPU (register reads), packed
+// ones 35.0 of 37.  y + g x in two instructions, from x prepared as (re, im)
+// and (-im, re): g.re times the one, then g.im times the other.  The same
+// FMAs in scalar form: cmac.
+__device__ __forceinline__ float4 cprep(float2 x) { return make_float4(x.x, x.y, -x.y, x.x); }
+__device__ __forceinline__ float2 cmac2_re(float2 g, float4 x, float2 y) {
+  return __ffma2_rn(make_float2(g.x, g.x), make_float2(x.x, x.y), y);
+}
+__device__ __forceinline__ float2 cmac2_im(float2 g, float4 x, float2 y) {
+  return __ffma2_rn(make_float2(g.y, g.y), make_float2(x.z, x.w), y);
+}
+__device__ __forceinline__ void cmac(float2 g, float2 x, float& re, float& im) {
+  re = fmaf(g.x, x.x, re);
+  im = fmaf(g.x, x.y, im);
+  re = fmaf(-g.y, x.y, re);
+  im = fmaf(g.y, x.x, im);
+}
+
 }  // namespace s2w

@@ -12,16 +12,19 @@
 // at the end one butterfly reduce-scatter over the lanes sums them.
 //
 // What bounds it: 4 FMAs per stored entry and rupture.  At eight ruptures an
-// FP32 entry costs 32 FMAs for 8 bytes, about 0.8 of the FMA rate when the
-// bytes arrive at the HBM rate, so the two meet there; a wider batch would be
-// bound by the FMAs, a narrower one by HBM.  Measured, whole call: 480 x
-// 37,758 x 32 x 256, 8 ruptures, 46.0 ms one by one, 8.05 ms here (stage 1
-// 42.2 -> 6.7, 5.5 at the copy rate); 333 x 4,999 x 17 x 512 with seafloor
-// output, 5 ruptures, 6.66 -> 1.42 ms.  Rows are cut into K slabs (not
-// whole rows per warp) because eight warps with eight whole rows each would
-// need 0.5 MB of shared memory, and eight rows per warp because each vector
-// entry read from shared memory must serve several rows: 16 bytes of rows and
-// vectors per 32 FMAs.
+// FP32 entry costs 32 FMAs for 8 bytes; scalar FFMAs with three register
+// operands run at 25 TFMA/s here, so the FMAs take as long as the bytes at
+// the copy rate at about six ruptures, and eight take 1.2x the time of one
+// (963 x 8,000 x 64 x 256: 2.46 ms for one, 2.50 for two, 2.54 for four, 2.96
+// for eight, 19.5 ms eight times over; 480 x 37,758 x 32 x 256, eight
+// ruptures: 46.0 -> 8.0 ms; 333 x 4,999 x 17 x 512 with seafloor output, five:
+// 6.66 -> 1.42 ms).  Rows are cut into K slabs (not whole rows per warp)
+// because eight warps with eight whole rows each would need 0.5 MB of shared
+// memory, and eight rows per warp because each vector entry read from shared
+// memory must serve several rows.  Packed FP32 products (35 TFMA/s) were
+// slower here: they want the vectors twice (rotated), in registers or in
+// shared-memory reads, at two warps per scheduler (8.8 ms; also twelve warps
+// with four or six rows each, 8.3 - 9.3 ms).
 //
 // Each lane sums its chunks l, l + 32, ... in column order into one
 // accumulator per component, then the lanes are added over xor 16, 8, 4, 2, 1:
@@ -44,14 +47,15 @@ constexpr int kWarps = 8;
 // (2 x 128 x 232 + 128 x 40 = 384 x 168).
 constexpr int kThreads = 32 * (kWarps + 4);
 constexpr int kRegsConsumer = 232, kRegsProducer = 40;
-constexpr int kRows = 64;             // most rows per tile: eight per warp
-constexpr int kSlabBytes = 512;       // of each row per stage: one 16-byte chunk per lane
+constexpr int RW = 8;                 // rows per warp, of a full tile
+constexpr int kSlabBytes = 512;       // most of each row per stage: one 16-byte chunk per lane
 constexpr int kMaxStages = 16;
 constexpr int kBudget = 208 * 1024;   // ring bytes
 
 struct MultiArgs {
   int n_vec, rows_per_vec, tiles, mrows;  // tiles of mrows rows per vector group
   int slabs, stages;
+  int slab_bytes;   // of each row per stage: kSlabBytes, or the whole of a shorter row
   int nb;
   int x_vec_first;  // the vector map's dimensions are (entry, vector, rupture), else (entry, rupture, vector)
   long long y_ldb;
@@ -76,20 +80,23 @@ __device__ __forceinline__ uint64_t l2_policy_evict_last() {
   return pol;
 }
 
-template <int EL, bool HILO, int R>
+// SHORT: rows shorter than a slab (the stage holds whole rows).
+template <int EL, bool HILO, int R, bool SHORT>
 __global__ void __launch_bounds__(kThreads, 1)
     k_stream_multi(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmAlo,
                    const __grid_constant__ CUtensorMap tmX, const MultiArgs a) {
   using CH = Chunk<EL>;
   constexpr int C = CH::C;
-  constexpr int XB = 32 * C * 8;  // vector bytes per rupture and slab
-  constexpr int kWordsA = kSlabBytes / 4, kWordsX = XB / 4;
+  const int slab_bytes = SHORT ? a.slab_bytes : kSlabBytes;
+  const int pitch = slab_bytes / 16;                  // 16-byte chunks of a row in a stage
+  const int x_bytes = slab_bytes * (C / 2);           // of a vector in a stage
   extern __shared__ __align__(128) unsigned char sm[];
   const int S = a.stages;
   uint64_t* full = reinterpret_cast<uint64_t*>(sm);
   uint64_t* empty = full + kMaxStages;
-  const int a_bytes = a.mrows * kSlabBytes;
-  const int stage_bytes = a_bytes * (HILO ? 2 : 1) + R * XB;
+  const int a_bytes = a.mrows * slab_bytes;
+  const int fill_bytes = a_bytes * (HILO ? 2 : 1) + R * x_bytes;  // what TMA brings per stage
+  const int stage_bytes = (fill_bytes + 127) & ~127;
   unsigned char* ring = sm + 2 * 8 * kMaxStages;
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -120,10 +127,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           if (!(a.fault_skip && it == 0)) {  // (test hook: stage 0 never fills)
             unsigned char* st = ring + s * stage_bytes;
-            mbar_arrive_expect_tx(full + s, stage_bytes);
-            tma_words(st, &tmA, k * kWordsA, tile * a.mrows, vec, full + s, first);
-            if (HILO) tma_words(st + a_bytes, &tmAlo, k * kWordsA, tile * a.mrows, vec, full + s, first);
-            tma_words(st + a_bytes * (HILO ? 2 : 1), &tmX, k * kWordsX, a.x_vec_first ? vec : 0,
+            mbar_arrive_expect_tx(full + s, fill_bytes);
+            tma_words(st, &tmA, k * (slab_bytes / 4), tile * a.mrows, vec, full + s, first);
+            if (HILO)
+              tma_words(st + a_bytes, &tmAlo, k * (slab_bytes / 4), tile * a.mrows, vec, full + s, first);
+            tma_words(st + a_bytes * (HILO ? 2 : 1), &tmX, k * (x_bytes / 4), a.x_vec_first ? vec : 0,
                       a.x_vec_first ? 0 : vec, full + s, last);
           }
           if (++s == S) s = 0, ph ^= 1;
@@ -144,12 +152,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int nr = min(a.mrows, a.rows_per_vec - tile * a.mrows);
     // a full tile gives each warp eight adjacent rows (64-byte stores), a
     // partial one deals its rows out over the warps
-    const bool whole = nr == kRows;
-    const int r_w = whole ? 8 : 1, r_i = whole ? 1 : 8;
+    const bool whole = nr == kWarps * RW;
+    const int r_w = whole ? RW : 1, r_i = whole ? 1 : kWarps;
     const int row0 = warp * r_w;
-    float acc[8 * R * 2];
+    float acc[RW * R * 2];
 #pragma unroll
-    for (int k = 0; k < 8 * R * 2; ++k) acc[k] = 0.f;
+    for (int k = 0; k < RW * R * 2; ++k) acc[k] = 0.f;
     for (int k = 0; k < a.slabs; ++k) {
       if (!mbar_wait_bounded(full + s, ph, a.status, DEV_ERR_TIMEOUT_FULL, a.wait_ns)) return;
       const unsigned char* st = ring + s * stage_bytes;
@@ -162,40 +170,34 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int h = 0; h < C / 2; ++h) {  // two entries of the lane's chunk at a time
           float4 x[R];
 #pragma unroll
-          for (int b = 0; b < R; ++b) x[b] = xs[b * (XB / 16) + h];
+          for (int b = 0; b < R; ++b) x[b] = xs[b * pitch * (C / 2) + h];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int row = WHOLE ? row0 + i : row0 + 8 * i;
+          for (int i = 0; i < RW; ++i) {
+            const int row = WHOLE ? row0 + i : row0 + kWarps * i;
             if (!WHOLE && row >= nr) continue;
             float2 g[C];
-            CH::unpack(rows[row * (kSlabBytes / 16)], g);
+            CH::unpack(rows[row * pitch], g);
             if (HILO) {
               float2 gl[C];
-              CH::unpack(rows_lo[row * (kSlabBytes / 16)], gl);
+              CH::unpack(rows_lo[row * pitch], gl);
 #pragma unroll
               for (int q = 0; q < C; ++q) g[q] = cadd(g[q], gl[q]);
             }
             const float2 g0 = g[2 * h], g1 = g[2 * h + 1];
 #pragma unroll
             for (int b = 0; b < R; ++b) {
-              float& ar = acc[(i * R + b) * 2];
-              float& ai = acc[(i * R + b) * 2 + 1];
-              ar = fmaf(g0.x, x[b].x, ar);
-              ar = fmaf(-g0.y, x[b].y, ar);
-              ai = fmaf(g0.x, x[b].y, ai);
-              ai = fmaf(g0.y, x[b].x, ai);
-              ar = fmaf(g1.x, x[b].z, ar);
-              ar = fmaf(-g1.y, x[b].w, ar);
-              ai = fmaf(g1.x, x[b].w, ai);
-              ai = fmaf(g1.y, x[b].z, ai);
+              cmac(g0, make_float2(x[b].x, x[b].y), acc[(i * R + b) * 2], acc[(i * R + b) * 2 + 1]);
+              cmac(g1, make_float2(x[b].z, x[b].w), acc[(i * R + b) * 2], acc[(i * R + b) * 2 + 1]);
             }
           }
         }
       };
-      if (whole)
-        slab(std::true_type{});
-      else
-        slab(std::false_type{});
+      if (!SHORT || lane < pitch) {  // (a row shorter than a slab leaves lanes without a chunk)
+        if (whole)
+          slab(std::true_type{});
+        else
+          slab(std::false_type{});
+      }
       __syncwarp();
       if (lane == 0) mbar_arrive(empty + s);
       if (++s == S) s = 0, ph ^= 1;
@@ -204,10 +206,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     // keeps the half of its values that the bit selects, summed with its
     // partner's; value index ((row * R) + b) * 2 + component
 #pragma unroll
-    for (int o = 16, n = 8 * R; o > 0; o >>= 1, n >>= 1) {
+    for (int o = 16, n = RW * R; o > 0; o >>= 1, n >>= 1) {
       const bool up = (lane & o) != 0;
 #pragma unroll
-      for (int k = 0; k < 8 * R; ++k) {
+      for (int k = 0; k < RW * R; ++k) {
         if (k < n) {
           const float keep = up ? acc[k + n] : acc[k];
           const float send = up ? acc[k] : acc[k + n];
@@ -215,30 +217,30 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
     }
-    const int row = row0 + (lane >> 2) * r_i;
-    if (row < nr) {
-      float2* y = a.y + static_cast<long long>(vec) * a.rows_per_vec + tile * a.mrows + row;
+    float2* y = a.y + static_cast<long long>(vec) * a.rows_per_vec + tile * a.mrows;
 #pragma unroll
-      for (int j = 0; j < R / 2; ++j) {
-        const int v = (lane & 3) * (R / 2) + j;
-        if ((v >> 1) < a.nb) reinterpret_cast<float*>(y + (v >> 1) * a.y_ldb)[v & 1] = acc[j];
-      }
+    for (int j = 0; j < RW * R / 16; ++j) {
+      const int v = lane * (RW * R / 16) + j;  // (each step's bit selects a half: lane major)
+      const int row = row0 + v / (2 * R) * r_i, b = v / 2 % R;
+      if (row < nr && b < a.nb) reinterpret_cast<float*>(y + b * a.y_ldb + row)[v & 1] = acc[j];
     }
   }
 }
 
-template <int EL, bool HILO, int R>
+template <int EL, bool HILO, int R, bool SHORT = false>
 cudaError_t launch_r(const StreamArgs& a, int num_sms, cudaStream_t st) {
   using CH = Chunk<EL>;
-  constexpr int XB = 32 * CH::C * 8;
   const long long row_bytes = static_cast<long long>(a.row_len) * (16 / CH::C);
   MultiArgs m{};
+  m.slab_bytes = row_bytes < kSlabBytes ? static_cast<int>(row_bytes) : kSlabBytes;
+  const int x_bytes = m.slab_bytes * (CH::C / 2);
   m.rows_per_vec = static_cast<int>(a.rows_per_vec);
   m.n_vec = static_cast<int>(a.F / a.rows_per_vec);
-  m.mrows = a.rows_per_vec >= kRows ? kRows : static_cast<int>((a.rows_per_vec + 7) / 8 * 8);
+  constexpr int tile_rows = kWarps * RW;
+  m.mrows = a.rows_per_vec >= tile_rows ? tile_rows : static_cast<int>((a.rows_per_vec + 7) / 8 * 8);
   m.tiles = (m.rows_per_vec + m.mrows - 1) / m.mrows;
   m.slabs = static_cast<int>((row_bytes + kSlabBytes - 1) / kSlabBytes);
-  const int stage = m.mrows * kSlabBytes * (HILO ? 2 : 1) + R * XB;
+  const int stage = (m.mrows * m.slab_bytes * (HILO ? 2 : 1) + R * x_bytes + 127) & ~127;
   m.stages = kBudget / stage < kMaxStages ? kBudget / stage : kMaxStages;
   m.nb = a.nb;
   m.y = a.y;
@@ -249,32 +251,34 @@ cudaError_t launch_r(const StreamArgs& a, int num_sms, cudaStream_t st) {
   CUtensorMap ta, tl, tx;
   cudaError_t e;
   const long long vec_bytes = row_bytes * a.rows_per_vec;
-  if ((e = tc_encode_words(&ta, a.rows, row_bytes / 4, a.rows_per_vec, row_bytes, m.n_vec, vec_bytes, kSlabBytes / 4,
+  if ((e = tc_encode_words(&ta, a.rows, row_bytes / 4, a.rows_per_vec, row_bytes, m.n_vec, vec_bytes, m.slab_bytes / 4,
                            m.mrows)) != cudaSuccess)
     return e;
   tl = ta;
   if (HILO && (e = tc_encode_words(&tl, a.rows_lo, row_bytes / 4, a.rows_per_vec, row_bytes, m.n_vec, vec_bytes,
-                                   kSlabBytes / 4, m.mrows)) != cudaSuccess)
+                                   m.slab_bytes / 4, m.mrows)) != cudaSuccess)
     return e;
   // ruptures past nb read as zeros (TMA fill); their sums are never stored.
   // The map's dimensions go up in pitch
   m.x_vec_first = a.x_stride < a.x_ldb ? 1 : 0;
   e = m.x_vec_first
-          ? tc_encode_words(&tx, a.x, 2LL * a.row_len, m.n_vec, 8 * a.x_stride, a.nb, 8 * a.x_ldb, XB / 4, 1, R)
-          : tc_encode_words(&tx, a.x, 2LL * a.row_len, a.nb, 8 * a.x_ldb, m.n_vec, 8 * a.x_stride, XB / 4, R);
+          ? tc_encode_words(&tx, a.x, 2LL * a.row_len, m.n_vec, 8 * a.x_stride, a.nb, 8 * a.x_ldb, x_bytes / 4, 1, R)
+          : tc_encode_words(&tx, a.x, 2LL * a.row_len, a.nb, 8 * a.x_ldb, m.n_vec, 8 * a.x_stride, x_bytes / 4, R);
   if (e != cudaSuccess) return e;
   const size_t smem = 2 * 8 * kMaxStages + static_cast<size_t>(m.stages) * stage;
-  if ((e = cudaFuncSetAttribute(k_stream_multi<EL, HILO, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if ((e = cudaFuncSetAttribute(k_stream_multi<EL, HILO, R, SHORT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 static_cast<int>(smem))) != cudaSuccess)
     return e;
   long long grid = static_cast<long long>(m.n_vec) * m.tiles;
   if (grid > num_sms) grid = num_sms;
-  k_stream_multi<EL, HILO, R><<<static_cast<unsigned>(grid), kThreads, smem, st>>>(ta, tl, tx, m);
+  k_stream_multi<EL, HILO, R, SHORT><<<static_cast<unsigned>(grid), kThreads, smem, st>>>(ta, tl, tx, m);
   return cudaGetLastError();
 }
 
 template <int EL, bool HILO>
 cudaError_t launch_el(const StreamArgs& a, int num_sms, cudaStream_t st) {
+  if (a.row_len * (16 / Chunk<EL>::C) < kSlabBytes)
+    return a.nb <= 4 ? launch_r<EL, HILO, 4, true>(a, num_sms, st) : launch_r<EL, HILO, 8, true>(a, num_sms, st);
   if (a.nb <= 2) return launch_r<EL, HILO, 2>(a, num_sms, st);
   if (a.nb <= 4) return launch_r<EL, HILO, 4>(a, num_sms, st);
   if (a.nb <= 6) return launch_r<EL, HILO, 6>(a, num_sms, st);
@@ -284,7 +288,7 @@ cudaError_t launch_el(const StreamArgs& a, int num_sms, cudaStream_t st) {
 }  // namespace
 
 cudaError_t launch_stream_multi(const StreamArgs& a, int num_sms, cudaStream_t st) {
-  if (a.nb < 2 || a.nb > kStreamMulti || a.rows_per_vec < 1 || a.rows_per_vec > 0x7fffffff - kRows ||
+  if (a.nb < 2 || a.nb > kStreamMulti || a.rows_per_vec < 1 || a.rows_per_vec > 0x7fffff00 ||
       a.F % a.rows_per_vec != 0)
     return cudaErrorInvalidValue;
   switch (a.el) {

@@ -38,11 +38,8 @@ namespace s2w {
 
 namespace {
 
-constexpr int kConsumerWarps = 8;  // the transposed kernel; k_stream_dot takes stream_warps(EL)
 constexpr int kStages = 3;
-constexpr int kThreads = 32 * (kConsumerWarps + 1);
 constexpr int kMaxRowLen = 1024;
-constexpr int kStagesT = 2;  // ring depth of the transposed kernel (its reduction buffer needs the room)
 
 // EL selects the unpacker (EL_BF16 also serves the hi/lo pair when HILO);
 // SHORT: rows of at most 64 chunks, shared by lane groups; DF (with EL_FP32
@@ -51,8 +48,9 @@ constexpr int kStagesT = 2;  // ring depth of the transposed kernel (its reducti
 // ones, so per-row work (the lane reduction, the scale) weighs more: long FP8
 // rows are taken four per warp pass (one reduction for the four), short ones
 // by twelve warps (more rows in flight; ~120 registers each, no spills).
-__host__ __device__ constexpr int stream_warps(int el, bool short_rows) {
-  return (el == EL_FP8 && short_rows) ? 12 : 8;
+// One rupture's short FP32 / BF16 rows take twelve warps too.
+__host__ __device__ constexpr int stream_warps(int el, bool short_rows, bool df, int r) {
+  return (short_rows && !df && r == 1) ? 12 : 8;
 }
 
 // R > 1 (short FP32 / BF16 rows): the row meets the vectors of R ruptures,
@@ -60,9 +58,9 @@ __host__ __device__ constexpr int stream_warps(int el, bool short_rows) {
 // operator once per R ruptures.  Otherwise a batch takes one grid slice (y)
 // per rupture.
 template <int EL, bool HILO, bool SHORT, bool DF = false, int R = 1>
-__global__ void __launch_bounds__(32 * (stream_warps(EL, SHORT) + 1), 1)
+__global__ void __launch_bounds__(32 * (stream_warps(EL, SHORT, DF, R) + 1), 1)
     k_stream_dot(const StreamArgs a, int stage_rows) {
-  constexpr int kConsumerWarps = stream_warps(EL, SHORT);
+  constexpr int kConsumerWarps = stream_warps(EL, SHORT, DF, R);
   static_assert(!DF || (EL == EL_FP32 && HILO), "pair rows: FP32 hi and lo arrays");
   static_assert(R == 1 || (SHORT && !DF && EL != EL_FP8), "several vectors: short FP32 or BF16 rows");
   using CH = Chunk<EL>;
@@ -424,14 +422,30 @@ __global__ void __launch_bounds__(32 * (stream_warps(EL, SHORT) + 1), 1)
           ay[f] = make_float2(ar * sc, ai * sc);
         }
       } else {
-        // one chain per rupture and component, in column order: the order of
-        // k_stream_multi, so a rupture's result does not depend on the batch
-        float ar[R], ai[R];
+        // The order of k_stream_multi (chunk c on lane c mod 32, one chain per
+        // component and lane, then the lanes added over xor 16, 8, .. 1), so
+        // that a rupture's result does not depend on the batch.  A short row's
+        // lane holds four of those lanes' chunks: with 16 lanes per row the
+        // chunks t and t + 2 are one chain, with fewer all four are apart.
+        constexpr int H = SHORT ? 2 : 1;  // chains per lane and component
+        float xa[H][R], xi[H][R], sa[H][R], si[H][R];
 #pragma unroll
-        for (int b = 0; b < R; ++b) ar[b] = ai[b] = 0.f;
+        for (int h = 0; h < H; ++h)
+#pragma unroll
+          for (int b = 0; b < R; ++b) xa[h][b] = xi[h][b] = sa[h][b] = si[h][b] = 0.f;
 #pragma unroll
         for (int t = 0; t < T; ++t) {
           const int c = sub + lpr * t;
+          if (SHORT && t == 2 && lpr < 16) {
+#pragma unroll
+            for (int h = 0; h < H; ++h)
+#pragma unroll
+              for (int b = 0; b < R; ++b) {
+                sa[h][b] = xa[h][b];
+                si[h][b] = xi[h][b];
+                xa[h][b] = xi[h][b] = 0.f;
+              }
+          }
           if (valid && c < nchunk) {
             float2 g[C];
             CH::unpack(row[c], g);
@@ -445,13 +459,16 @@ __global__ void __launch_bounds__(32 * (stream_warps(EL, SHORT) + 1), 1)
             for (int q = 0; q < C; ++q) {
 #pragma unroll
               for (int b = 0; b < R; ++b) {
-                ar[b] = fmaf(g[q].x, xr[b][t][q].x, ar[b]);
-                ar[b] = fmaf(-g[q].y, xr[b][t][q].y, ar[b]);
-                ai[b] = fmaf(g[q].x, xr[b][t][q].y, ai[b]);
-                ai[b] = fmaf(g[q].y, xr[b][t][q].x, ai[b]);
+                cmac(g[q], xr[b][t][q], xa[t % H][b], xi[t % H][b]);
               }
             }
           }
+        }
+        float ar[R], ai[R];
+#pragma unroll
+        for (int b = 0; b < R; ++b) {
+          ar[b] = SHORT ? (sa[0][b] + xa[0][b]) + (sa[H - 1][b] + xa[H - 1][b]) : xa[0][b];
+          ai[b] = SHORT ? (si[0][b] + xi[0][b]) + (si[H - 1][b] + xi[H - 1][b]) : xi[0][b];
         }
         for (int o = lpr / 2; o > 0; o >>= 1) {
 #pragma unroll
@@ -472,178 +489,6 @@ __global__ void __launch_bounds__(32 * (stream_warps(EL, SHORT) + 1), 1)
   }
 }
 
-// Transposed contraction (the adjoint, a correlation with the conjugate
-// spectra):  y[u][c] = sum_{f in unit u} conj(rows[f][c]) * w_f.
-// A unit is `Rc` consecutive rows of one group of G1 rows (chunk u % nchunk
-// of group u / nchunk); the row weight is w[w_base + (g / wa) * wb + (f - g G1)]
-// with g = f / G1, times the FP8 row scale when the rows are FP8.
-// One CTA per unit at a time; the 8 consumer warps accumulate their rows
-// column-wise in registers, then sum across warps through shared memory.
-template <int EL, bool HILO>
-__global__ void __launch_bounds__(kThreads, 1) k_stream_tdot(const StreamTArgs a, int stage_rows) {
-  using CH = Chunk<EL>;
-  constexpr int C = CH::C;
-  constexpr int T = kMaxRowLen / (32 * C);
-  extern __shared__ __align__(128) unsigned char sm[];
-  uint64_t* full = reinterpret_cast<uint64_t*>(sm);
-  uint64_t* empty = full + kStagesT;
-  unsigned char* buf = sm + 128;
-  const int row_bytes = a.row_len * (16 / C);
-  const int stage_bytes = stage_rows * row_bytes;
-  unsigned char* buf_lo = buf + kStagesT * stage_bytes;
-  float2* red = reinterpret_cast<float2*>(buf + (HILO ? 2 : 1) * kStagesT * stage_bytes);  // [8][row_len]
-  const int warp = threadIdx.x >> 5;
-  const int lane = threadIdx.x & 31;
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kStagesT; ++s) {
-      mbar_init(full + s, 1);
-      mbar_init(empty + s, kConsumerWarps);
-    }
-    fence_mbar_init();
-  }
-  __syncthreads();
-
-  auto unit_rows = [&](long long u, long long& f0, long long& f1) {
-    const long long g = u / a.nchunk;
-    const long long c = u % a.nchunk;
-    f0 = g * a.G1 + c * a.Rc;
-    f1 = g * a.G1 + min(static_cast<long long>(c + 1) * a.Rc, a.G1);
-  };
-
-  if (warp == kConsumerWarps) {
-    if (lane == 0) {
-      const uint64_t pol = l2_policy_evict_first();
-      int it = 0;
-      bool ok = true;
-      for (long long u = blockIdx.x; u < a.n_units && ok; u += gridDim.x) {
-        long long f0, f1;
-        unit_rows(u, f0, f1);
-        for (long long rs = f0; rs < f1; rs += stage_rows, ++it) {
-          const int s = it % kStagesT;
-          if (it >= kStagesT &&
-              !mbar_wait_bounded(empty + s, ((it / kStagesT) - 1) & 1, a.status, DEV_ERR_TIMEOUT_EMPTY)) {
-            ok = false;
-            break;
-          }
-          const int nr = static_cast<int>(min(static_cast<long long>(stage_rows), f1 - rs));
-          const uint32_t bytes = static_cast<uint32_t>(nr) * row_bytes;
-          mbar_arrive_expect_tx(full + s, HILO ? 2 * bytes : bytes);
-          bulk_g2s(buf + s * stage_bytes, static_cast<const unsigned char*>(a.rows) + rs * row_bytes, bytes,
-                   full + s, pol);
-          if (HILO)
-            bulk_g2s(buf_lo + s * stage_bytes, static_cast<const unsigned char*>(a.rows_lo) + rs * row_bytes, bytes,
-                     full + s, pol);
-        }
-      }
-      for (int kk = (it > kStagesT ? it - kStagesT : 0); kk < it; ++kk)
-        mbar_wait_bounded(full + kk % kStagesT, (kk / kStagesT) & 1, a.status, DEV_ERR_TIMEOUT_FULL);
-    }
-    return;
-  }
-
-  const int nchunk = row_bytes / 16;
-  int it = 0;
-  for (long long u = blockIdx.x; u < a.n_units; u += gridDim.x) {
-    long long f0, f1;
-    unit_rows(u, f0, f1);
-    float2 acc[T][C];
-#pragma unroll
-    for (int t = 0; t < T; ++t)
-#pragma unroll
-      for (int q = 0; q < C; ++q) acc[t][q] = make_float2(0.f, 0.f);
-    bool ok = true;
-    for (long long rs = f0; rs < f1; rs += stage_rows, ++it) {
-      const int s = it % kStagesT;
-      if (!mbar_wait_bounded(full + s, (it / kStagesT) & 1, a.status, DEV_ERR_TIMEOUT_FULL)) {
-        ok = false;
-        break;
-      }
-      const int nr = static_cast<int>(min(static_cast<long long>(stage_rows), f1 - rs));
-      for (int lr = warp; lr < nr; lr += kConsumerWarps) {
-        const long long f = rs + lr;
-        const long long g = f / a.G1;
-        const long long within = f - g * a.G1;
-        float2 w = a.w[a.w_base + (g / a.wa) * a.wb + within];
-        if (EL == EL_FP8) {
-          const float sc = a.scale[g * a.nblk + within / 256];
-          w.x *= sc;
-          w.y *= sc;
-        }
-        const uint4* row = reinterpret_cast<const uint4*>(buf + s * stage_bytes + lr * row_bytes);
-        const uint4* row_lo = reinterpret_cast<const uint4*>(buf_lo + s * stage_bytes + lr * row_bytes);
-#pragma unroll
-        for (int t = 0; t < T; ++t) {
-          const int c = lane + 32 * t;
-          if (c < nchunk) {
-            float2 gv[C];
-            CH::unpack(row[c], gv);
-            if (HILO) {
-              float2 gl[C];
-              CH::unpack(row_lo[c], gl);
-#pragma unroll
-              for (int q = 0; q < C; ++q) gv[q] = cadd(gv[q], gl[q]);
-            }
-#pragma unroll
-            for (int q = 0; q < C; ++q) {  // conj(g) * w
-              acc[t][q].x = fmaf(gv[q].x, w.x, fmaf(gv[q].y, w.y, acc[t][q].x));
-              acc[t][q].y = fmaf(gv[q].x, w.y, fmaf(-gv[q].y, w.x, acc[t][q].y));
-            }
-          }
-        }
-      }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(empty + s);
-    }
-    // cross-warp sum of the unit's column accumulators, in fixed warp order
-#pragma unroll
-    for (int t = 0; t < T; ++t) {
-      const int c = lane + 32 * t;
-      if (c < nchunk)
-#pragma unroll
-        for (int q = 0; q < C; ++q) red[warp * a.row_len + c * C + q] = acc[t][q];
-    }
-    asm volatile("bar.sync 1, %0;" ::"r"(kConsumerWarps * 32) : "memory");
-    for (int col = threadIdx.x; col < a.row_len; col += kConsumerWarps * 32) {
-      float2 sum = red[col];
-      for (int w2 = 1; w2 < kConsumerWarps; ++w2) sum = cadd(sum, red[w2 * a.row_len + col]);
-      a.y[u * a.row_len + col] = sum;
-    }
-    // second barrier doubles as a vote: if any consumer warp gave up on a
-    // wait, all of them leave together (none is left behind on this barrier)
-    int any_failed;
-    asm volatile(
-        "{\n\t.reg .pred pin, pout;\n\t"
-        "setp.eq.u32 pin, %1, 0;\n\t"
-        "bar.red.or.pred pout, 1, %2, pin;\n\t"
-        "selp.u32 %0, 1, 0, pout;\n\t}"
-        : "=r"(any_failed)
-        : "r"(ok ? 1u : 0u), "r"(kConsumerWarps * 32)
-        : "memory");
-    if (any_failed) return;
-  }
-}
-
-template <int EL, bool HILO>
-cudaError_t launch_tt(const StreamTArgs& a, int num_sms, cudaStream_t st) {
-  constexpr int C = Chunk<EL>::C;
-  const int row_bytes = a.row_len * (16 / C);
-  const int budget = HILO ? 32 * 1024 : 64 * 1024;
-  int stage_rows = budget / row_bytes;
-  if (stage_rows >= kConsumerWarps) stage_rows -= stage_rows % kConsumerWarps;
-  if (stage_rows < 1) stage_rows = 1;
-  const size_t smem = 128 + static_cast<size_t>(kStagesT) * stage_rows * row_bytes * (HILO ? 2 : 1) +
-                      sizeof(float2) * kConsumerWarps * a.row_len;
-  cudaError_t e = cudaFuncSetAttribute(k_stream_tdot<EL, HILO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
-  if (e != cudaSuccess) return e;
-  long long grid = num_sms;
-  if (grid > a.n_units) grid = a.n_units;
-  if (grid < 1) grid = 1;
-  k_stream_tdot<EL, HILO><<<static_cast<unsigned>(grid), kThreads, smem, st>>>(a, stage_rows);
-  return cudaGetLastError();
-}
-
 template <int EL, bool HILO, bool SHORT, bool DF = false, int R = 1>
 cudaError_t launch_t(const StreamArgs& a, int num_sms, cudaStream_t st) {
   constexpr int C = Chunk<EL>::C;
@@ -660,7 +505,7 @@ cudaError_t launch_t(const StreamArgs& a, int num_sms, cudaStream_t st) {
   if (grid > a.F) grid = a.F;
   if (grid < 1) grid = 1;
   const dim3 g(static_cast<unsigned>(grid), R == 1 ? static_cast<unsigned>(a.nb) : 1u);
-  k_stream_dot<EL, HILO, SHORT, DF, R><<<g, 32 * (stream_warps(EL, SHORT) + 1), smem, st>>>(a, stage_rows);
+  k_stream_dot<EL, HILO, SHORT, DF, R><<<g, 32 * (stream_warps(EL, SHORT, DF, R) + 1), smem, st>>>(a, stage_rows);
   return cudaGetLastError();
 }
 
@@ -671,26 +516,28 @@ bool short_rows(const StreamArgs& a, int C) { return a.row_len / C <= 64; }
 }  // namespace
 
 namespace {
+// Rows of at most this many chunks stay on the lane groups in a batch.
+constexpr int kShortestChunks = 16;
 // One launch for a.nb ruptures of FP32 / BF16 storage (nb <= kStreamMulti).
 template <int EL, bool HILO>
 cudaError_t launch_plain(const StreamArgs& a, int num_sms, cudaStream_t st) {
-  if (!short_rows(a, Chunk<EL>::C))
-    return a.nb == 1 ? launch_t<EL, HILO, false>(a, num_sms, st) : launch_stream_multi(a, num_sms, st);
-  if (a.nb == 1) return launch_t<EL, HILO, true>(a, num_sms, st);
-  if (a.nb == 2) return launch_t<EL, HILO, true, false, 2>(a, num_sms, st);
-  if (a.nb <= 4) return launch_t<EL, HILO, true, false, 4>(a, num_sms, st);
-  if constexpr (EL == EL_FP32) {  // a lane's slices of eight vectors: 128 registers
-    return launch_t<EL, HILO, true, false, 8>(a, num_sms, st);
-  } else {  // BF16 chunks hold twice the entries: four vectors at a time
+  if (a.nb == 1)
+    return short_rows(a, Chunk<EL>::C) ? launch_t<EL, HILO, true>(a, num_sms, st)
+                                       : launch_t<EL, HILO, false>(a, num_sms, st);
+  // A batch: k_stream_multi, whose warps take eight rows at about the same
+  // cost however short they are; the shortest rows in lane groups here, at
+  // most kMostVectors at a time (a lane holds its slices of every vector)
+  if (a.row_len / Chunk<EL>::C > kShortestChunks) return launch_stream_multi(a, num_sms, st);
+  constexpr int kMostVectors = EL == EL_FP32 ? 4 : 2;
+  for (int b = 0; b < a.nb; b += kMostVectors) {
     StreamArgs h = a;
-    h.nb = 4;
-    const cudaError_t e = launch_t<EL, HILO, true, false, 4>(h, num_sms, st);
+    h.nb = a.nb - b < kMostVectors ? a.nb - b : kMostVectors;
+    h.x = a.x + b * a.x_ldb;
+    h.y = a.y + b * a.y_ldb;
+    const cudaError_t e = launch_t<EL, HILO, true, false, kMostVectors>(h, num_sms, st);
     if (e != cudaSuccess) return e;
-    h.nb = a.nb - 4;
-    h.x = a.x + 4 * a.x_ldb;
-    h.y = a.y + 4 * a.y_ldb;
-    return launch_t<EL, HILO, true, false, 4>(h, num_sms, st);
   }
+  return cudaSuccess;
 }
 }  // namespace
 
@@ -709,23 +556,6 @@ cudaError_t launch_stream_dot(const StreamArgs& a, int num_sms, cudaStream_t st)
       if (a.rows_lo == nullptr || a.x_lo == nullptr || a.y_lo == nullptr) return cudaErrorInvalidValue;
       return short_rows(a, 2) ? launch_t<EL_FP32, true, true, true>(a, num_sms, st)
                               : launch_t<EL_FP32, true, false, true>(a, num_sms, st);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-}  // namespace s2w
-
-namespace s2w {
-
-cudaError_t launch_stream_tdot(const StreamTArgs& a, int num_sms, cudaStream_t st) {
-  if (a.n_units <= 0) return cudaSuccess;
-  if (a.row_len <= 0 || a.row_len > kMaxRowLen || (a.row_len % 8) != 0 || a.Rc < 1 || a.nchunk < 1)
-    return cudaErrorInvalidValue;
-  switch (a.el) {
-    case EL_FP32: return launch_tt<EL_FP32, false>(a, num_sms, st);
-    case EL_BF16: return launch_tt<EL_BF16, false>(a, num_sms, st);
-    case EL_BF16_HILO: return launch_tt<EL_BF16, true>(a, num_sms, st);
-    case EL_FP8: return launch_tt<EL_FP8, false>(a, num_sms, st);
     default: return cudaErrorInvalidValue;
   }
 }

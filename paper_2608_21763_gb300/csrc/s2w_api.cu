@@ -60,7 +60,7 @@ struct s2w_ctx {
   float* ws_resid = nullptr;   // misfit gradient: q then r = q - d, [b][No][Nt]
   float* ws_d = nullptr;       // misfit gradient: staged targets, [b][No][Nt]
   float* ws_loss = nullptr;    // misfit gradient: per-rupture loss
-  float2* ws_gpart = nullptr;  // adjoint: stage-1 chunk partials [l][chunk][Ns_pad]
+  float2* ws_gpart = nullptr;  // adjoint: stage-1 chunk partials [multi][l][chunk][Ns_pad]
   int adj_rc = 512;            // adjoint: grid rows per stage-1 chunk
   int adj_nchunk = 1;
   int* d_status = nullptr;
@@ -931,8 +931,6 @@ int s2w_create(int Ns, int Ng, int No, int Nt, const s2w_opts* opts, s2w_ctx** o
   if ((e = dalloc(&ctx->ws_loss, sizeof(float) * B)) != cudaSuccess) return bad(e, "losses");
   if ((e = dalloc(&ctx->ws_lens, sizeof(int) * B)) != cudaSuccess) return bad(e, "active lengths");
   if ((e = dalloc(&ctx->d_amax, sizeof(unsigned))) != cudaSuccess) return bad(e, "operand range word");
-  if ((e = dalloc(&ctx->ws_gpart, sizeof(float2) * Nb * ctx->adj_nchunk * ctx->Ns_pad)) != cudaSuccess)
-    return bad(e, "adjoint partials");
   // AUTO keeps the tensor engine ready at any max_batch: single ruptures go
   // to it only if s2w_autotune measured it faster (tc_min_batch = 1)
   ctx->tc_on = !ctx->single_pass && o.prec_g != S2W_PREC_FP32 && !ctx->df && 2 * No <= 256 &&
@@ -1049,19 +1047,21 @@ int s2w_create(int Ns, int Ng, int No, int Nt, const s2w_opts* opts, s2w_ctx** o
         return bad(e, "adjoint retransform matrix");
     }
   }
-  // Seafloor and velocity spectra of the streaming kernels, last: room for
-  // kStreamMulti ruptures per launch when that takes at most 1/8 of the
-  // memory still free, for fewer (at least the one that every call needs)
-  // otherwise.  Results do not depend on the count.
+  // Seafloor and velocity spectra and the adjoint's partials of the streaming
+  // kernels, last: room for kStreamMulti ruptures per launch when that takes
+  // at most 1/8 of the memory still free, for fewer (at least the one that
+  // every call needs) otherwise.  Results do not depend on the count.
   {
     const size_t mh = sizeof(float2) * Nb * Ng, vh = sizeof(float2) * Nb * ctx->nseg * ctx->RL;
+    const size_t gp = sizeof(float2) * Nb * ctx->adj_nchunk * ctx->Ns_pad;
     size_t free_b = 0, total_b = 0;
     if ((e = cudaMemGetInfo(&free_b, &total_b)) != cudaSuccess) return bad(e, "free memory");
     int m = static_cast<int>(std::min<long long>(B, kStreamMulti));
-    while (m > 1 && static_cast<size_t>(m) * (mh + vh) * (ctx->df ? 2 : 1) > free_b / 8) m /= 2;
+    while (m > 1 && static_cast<size_t>(m) * ((mh + vh) * (ctx->df ? 2 : 1) + gp) > free_b / 8) m /= 2;
     ctx->multi = m;
     if ((e = dalloc(&ctx->ws_mhat, m * mh)) != cudaSuccess) return bad(e, "seafloor spectra");
     if ((e = dalloc(&ctx->ws_vhat, m * vh)) != cudaSuccess) return bad(e, "velocity spectra");
+    if ((e = dalloc(&ctx->ws_gpart, m * gp)) != cudaSuccess) return bad(e, "adjoint partials");
     if (ctx->df) {
       if ((e = dalloc(&ctx->ws_mhat_lo, m * mh)) != cudaSuccess) return bad(e, "seafloor spectra lo");
       if ((e = dalloc(&ctx->ws_vhat_lo, m * vh)) != cudaSuccess) return bad(e, "velocity spectra lo");
@@ -1569,7 +1569,11 @@ int s2w_adjoint(s2w_ctx* ctx, const float* r, int B, float* grad_s, void* stream
                         No, st));
   }
   const int dt_t = ctx->opts.dt_mode == S2W_DT_NONE ? S2W_DT_NONE : kDtTranspose;
-  for (int b = 0; b < B; ++b) {
+  const long long vcols = static_cast<long long>(ctx->nseg) * ctx->RL;
+  const long long mhat_b = Nb * Ng, vhat_b = Nb * vcols, gpart_b = Nb * ctx->adj_nchunk * Ns_pad;  // per rupture
+  const int npass = (B + ctx->multi - 1) / ctx->multi;
+  for (int p = 0, b = 0, nb = 0; p < npass; ++p, b += nb) {
+    nb = (B - b + npass - p - 1) / (npass - p);  // equal passes of at most ctx->multi ruptures
     {  // stage-2 adjoint: what_l[i] = sum_o conj(Phat_l[o][i]) rhat_l[o]
       StageTimer t(ctx, 3, st);
       StreamTArgs a{};
@@ -1584,14 +1588,18 @@ int s2w_adjoint(s2w_ctx* ctx, const float* r, int B, float* grad_s, void* stream
       a.w_base = static_cast<long long>(b) * No;
       a.wa = ctx->nseg;
       a.wb = static_cast<long long>(B) * No;
+      a.nb = nb;
+      a.w_ldb = No;
       a.y = ctx->ws_vhat;
+      a.y_ldb = vhat_b;
       a.status = ctx->d_status;
       CK(launch_stream_tdot(a, ctx->num_sms, st));
     }
     {  // IFFT + Truncate, D_t^T, ZeroPad + FFT
       StageTimer t(ctx, 2, st);
-      CK(launch_retransform(ctx->ws_vhat, Ng, static_cast<long long>(ctx->nseg) * ctx->RL, static_cast<int>(Nt),
-                            ctx->tw, static_cast<float>(1.0 / ctx->opts.dt), dt_t, ctx->ws_mhat, Ng, nullptr, st));
+      CK(launch_retransform(ctx->ws_vhat, Ng, vcols, static_cast<int>(Nt), ctx->tw,
+                            static_cast<float>(1.0 / ctx->opts.dt), dt_t, ctx->ws_mhat, Ng, nullptr, st, nb, vhat_b,
+                            mhat_b));
     }
     {  // stage-1 adjoint: ghat_l[j] = sum_i conj(Ghat_l[i][j]) uhat_l[i], in row chunks
       StageTimer t(ctx, 1, st);
@@ -1610,13 +1618,16 @@ int s2w_adjoint(s2w_ctx* ctx, const float* r, int B, float* grad_s, void* stream
       a.wb = Ng;
       a.scale = ctx->G_scale;
       a.nblk = ctx->nblk;
+      a.nb = nb;
+      a.w_ldb = mhat_b;
       a.y = ctx->ws_gpart;
+      a.y_ldb = gpart_b;
       a.status = ctx->d_status;
       CK(launch_stream_tdot(a, ctx->num_sms, st));
     }
     {  // chunk reduction + IFFT + Truncate -> grad_s[b]
       StageTimer t(ctx, 4, st);
-      CK(launch_reduce_irfft(ctx->ws_gpart, 1, static_cast<int>(Ns), ctx->adj_nchunk, static_cast<int>(Nt), 0,
+      CK(launch_reduce_irfft(ctx->ws_gpart, nb, static_cast<int>(Ns), ctx->adj_nchunk, static_cast<int>(Nt), gpart_b,
                              static_cast<long long>(ctx->adj_nchunk) * Ns_pad, Ns_pad, ctx->tw,
                              g_d + static_cast<long long>(b) * Ns * Nt, st));
     }

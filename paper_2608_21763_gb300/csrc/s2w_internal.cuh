@@ -215,7 +215,7 @@ cudaError_t launch_stream_dot(const StreamArgs& a, int num_sms, cudaStream_t st)
 // BF16 hi/lo rows of more than 64 16-byte chunks (launch_stream_dot calls it).
 cudaError_t launch_stream_multi(const StreamArgs& a, int num_sms, cudaStream_t st);
 
-// k_stream.cu, transposed: y[u][c] = sum_{f in unit u} conj(rows[f][c]) w_f,
+// k_tdot.cu, transposed: y[u][c] = sum_{f in unit u} conj(rows[f][c]) w_f,
 // unit u = chunk (u % nchunk) of Rc rows of group (u / nchunk) of G1 rows,
 // w_f = w[w_base + (g / wa) * wb + (f - g G1)], g = f / G1 (times the FP8
 // scale[g * nblk + (f - g G1) / 256] for FP8 rows).
@@ -233,6 +233,8 @@ struct StreamTArgs {
   int nblk;
   float2* y;
   int* status;
+  int nb;                // ruptures (1 .. kStreamMulti): rupture b reads w + b * w_ldb, writes y + b * y_ldb
+  long long w_ldb, y_ldb;
 };
 cudaError_t launch_stream_tdot(const StreamTArgs& a, int num_sms, cudaStream_t st);
 

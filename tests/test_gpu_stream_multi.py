@@ -15,12 +15,13 @@ import paper_2608_21763_gb300 as s2w  # noqa: E402
 from test_gpu_parity import compact_box  # noqa: E402
 
 
-# FP32 rows are short up to Ns = 128, BF16 rows up to 256; stage 2's rows are
-# the grid segments (short up to 128 / 256 grid points)
+# rows of up to 16 chunks (Ns = 32 FP32, 64 BF16) stay on lane groups, longer
+# ones go to the tiled kernel; one rupture's short rows end at 64 chunks (Ns =
+# 128, 256); stage 2's rows are the grid segments
 @pytest.mark.parametrize("prec", ["fp32", "bf16", "bf16_hilo", "fp8"])
 @pytest.mark.parametrize("Ns,Ng,No,Nt,B", [(129, 63, 1, 32, 2), (128, 64, 9, 32, 9), (257, 65, 64, 32, 5),
                                            (1024, 130, 65, 64, 8), (300, 1100, 3, 32, 17), (5, 400, 120, 32, 6),
-                                           (264, 257, 8, 256, 3)])
+                                           (264, 257, 8, 256, 3), (40, 200, 3, 32, 8), (100, 90, 70, 64, 6), (70, 70, 9, 32, 4)])
 def test_batch_equals_single_ruptures_bitwise(prec, Ns, Ng, No, Nt, B):
     geom = compact_box(Ns, Ng, No, seed=Ns + Ng)
     slip = torch.tensor(np.random.default_rng(B).standard_normal((B, Ns, Nt)), dtype=torch.float32, device="cuda")
