@@ -386,8 +386,9 @@ int s2w_retransform_matrix(int Nt, int dt_mode, double dt, int transpose, double
  * Stages: 0 rfft of slip, 1 stage-1 contraction, 2 retransform (IFFT,
  * Truncate, D_t, ZeroPad, FFT), 3 stage-2 contraction, 4 partial reduction +
  * IFFT + Truncate, 5 host<->device copies made by s2w_waveforms, 6 packing
- * of tensor-engine operands (slip spectra into the stage-1 B operand), 7 a
- * whole replayed graph (s2w_waveforms_graph). */
+ * of tensor-engine operands (slip spectra into the stage-1 B operand; for
+ * BF16 and hi/lo operands one kernel with the rfft, counted here), 7 a whole
+ * replayed graph (s2w_waveforms_graph). */
 #define S2W_NUM_STAGES 8
 typedef struct {
   double ms[S2W_NUM_STAGES];           /* summed event-timed durations */

@@ -10,9 +10,12 @@
 //       through the warp's shared scratch gives each group of Q = 32 / P
 //       lanes one of them (lane q of group g holds the points q + Q j), and
 //       it splits again as 32 = P x Q: a P-point DFT over j in registers, a
-//       twiddle W_32^(q a), and a Q-point DFT across the group's lanes on
-//       log2(Q) shuffle stages.
-// fft_out<P>(lane, k) is the output bin that register k of `lane` holds.
+//       twiddle W_32^(q a), and a Q-point DFT across the group's lanes: its
+//       first log2(Q / min(Q, P)) radix-2 stages by shuffles, the others in
+//       registers after a second transpose, which also leaves the result in
+//       natural order: register t of lane l holds bin l + 32 t.  (The last
+//       stages by shuffles took about 220 instructions of 570 per 256-point
+//       transform; in registers they take 50.)
 //
 // A real signal of length L = 2N is packed as z[n] = x[2n] + i x[2n+1]; the
 // N + 1 bins of its real DFT follow from Z[k] and conj(Z[N - k]).  Twiddles
@@ -27,11 +30,6 @@ namespace s2w {
 
 __device__ __forceinline__ int rev5(int l) { return static_cast<int>(__brev(static_cast<unsigned>(l)) >> 27); }
 
-// Position of Z[i] in the per-warp scratch: XOR swizzle inside blocks of 16
-// complex entries, so that the scatter of the transform's outputs and the
-// natural-order reads of rfft_bin spread over the shared-memory banks.
-__device__ __forceinline__ int zsw(int i) { return i ^ ((i >> 4) & 15); }
-
 __host__ __device__ constexpr int ilog2c(int x) { return x <= 1 ? 0 : 1 + ilog2c(x / 2); }
 
 template <int P>
@@ -44,22 +42,23 @@ __host__ __device__ constexpr int bitrev_p(int k) {
   return r;
 }
 
-// Output bin held by register k of `lane` after warp_fft<P>.
+// Shape of the second split's last DFT (Q points) for N = 32 P: RQ of them in
+// registers after the shuffled stages, and the scratch of the transposes.
 template <int P>
-__device__ __forceinline__ int fft_out(int lane, int k) {
-  if (P == 1) return rev5(lane);
-  constexpr int Q = 32 / P;
-  constexpr int LQ = ilog2c(Q);
-  const int g = lane / Q, q = lane % Q;
-  const int rq = LQ > 0 ? static_cast<int>(__brev(static_cast<unsigned>(q)) >> (32 - LQ)) : 0;
-  return g + P * k + P * P * rq;
-}
+struct FftShape {
+  static constexpr int N = 32 * P;
+  static constexpr int Q = 32 / P;
+  static constexpr int RQ = P == 1 ? 1 : (Q < P ? Q : P);    // points of it in registers
+  static constexpr int BLK = N / RQ;                         // bins per register point
+  static constexpr int SKEW = P < 16 ? P : 0;                // keeps the transpose's writes on distinct banks
+  static constexpr int SCR = P == 1 ? N + 1 : (RQ * (BLK + SKEW) > N ? RQ * (BLK + SKEW) : N + 1);  // complex entries
+};
 
 // Per-lane twiddles of warp_fft<P>, read once per warp.
 template <int P>
 struct FftLane {
   static constexpr int Q = 32 / P;
-  static constexpr int NST = P == 1 ? 5 : ilog2c(Q);  // cross-lane radix-2 stages
+  static constexpr int NST = P == 1 ? 5 : ilog2c(Q / FftShape<P>::RQ);  // cross-lane radix-2 stages
   float2 tl[P];                        // W_N^(lane k)
   float2 tq[P];                        // W_32^(q a)
   float2 tc[NST > 0 ? NST : 1];        // stage twiddles of the cross-lane DFT
@@ -93,10 +92,10 @@ __device__ __forceinline__ FftLane<P> fft_lane(const float2* __restrict__ tw, in
 }
 
 // P-point DFT over registers (radix-2 DIF, uniform twiddles W_P^j = W_L^(j L / P)
-// of the length-L table), result in natural order.
-template <int P>
+// of the length-L table, L = 64 PT), result in natural order.
+template <int P, int PT = P>
 __device__ __forceinline__ void reg_dft(float2 (&v)[P], const float2* __restrict__ tw) {
-  constexpr int L = 64 * P;
+  constexpr int L = 64 * PT;
 #pragma unroll
   for (int h = P / 2; h >= 1; h >>= 1) {
 #pragma unroll
@@ -106,7 +105,13 @@ __device__ __forceinline__ void reg_dft(float2 (&v)[P], const float2* __restrict
         const float2 a = v[b + j];
         const float2 c = v[b + j + h];
         v[b + j] = cadd(a, c);
-        v[b + j + h] = (j == 0) ? csub(a, c) : cmul(csub(a, c), tw[j * (L / (2 * h))]);
+        const float2 d = csub(a, c);
+        if (j == 0)
+          v[b + j + h] = d;
+        else if (2 * j == h)  // W = -i
+          v[b + j + h] = make_float2(d.y, -d.x);
+        else
+          v[b + j + h] = cmul(d, tw[j * (L / (2 * h))]);
       }
     }
   }
@@ -117,8 +122,8 @@ __device__ __forceinline__ void reg_dft(float2 (&v)[P], const float2* __restrict
   for (int k = 0; k < P; ++k) v[k] = y[k];
 }
 
-// Forward complex DFT of N = 32 P points (see file comment for layouts);
-// scr: the warp's shared scratch of N complex entries (unused for P = 1).
+// Forward complex DFT of N = 32 P points, natural order in and out (see the
+// file comment); scr: the warp's shared scratch (unused for P = 1).
 template <int P>
 __device__ __forceinline__ void warp_fft(float2 (&v)[P], const float2* __restrict__ tw, const FftLane<P>& fl,
                                          int lane, float2* scr) {
@@ -137,9 +142,15 @@ __device__ __forceinline__ void warp_fft(float2 (&v)[P], const float2* __restric
       p.y = __shfl_xor_sync(0xffffffffu, v[0].y, h);
       v[0] = upper ? cmul(csub(p, v[0]), fl.tc[st]) : cadd(v[0], p);
     }
+    float2 n;  // natural order
+    n.x = __shfl_sync(0xffffffffu, v[0].x, rev5(lane));
+    n.y = __shfl_sync(0xffffffffu, v[0].y, rev5(lane));
+    v[0] = n;
     return;
   }
-  constexpr int Q = 32 / P;
+  using SH = FftShape<P>;
+  constexpr int Q = SH::Q, RQ = SH::RQ;
+  constexpr int NSH = ilog2c(Q / RQ);  // shuffled stages
   const int g = lane / Q, q = lane % Q;
   // (c) transpose: row k2 of the scratch holds the 32 points of DFT k2
   // (column XOR (Q k2) keeps the group reads below on distinct banks)
@@ -149,12 +160,11 @@ __device__ __forceinline__ void warp_fft(float2 (&v)[P], const float2* __restric
   __syncwarp();
 #pragma unroll
   for (int j = 0; j < P; ++j) v[j] = scr[g * 32 + ((q + Q * j) ^ ((Q * g) & 31))];
-  __syncwarp();
   reg_dft<P>(v, tw);
 #pragma unroll
   for (int a = 1; a < P; ++a) v[a] = cmul(v[a], fl.tq[a]);
 #pragma unroll
-  for (int st = 0; st < FftLane<P>::NST; ++st) {
+  for (int st = 0; st < NSH; ++st) {
     const int h = (Q / 2) >> st;
     const bool upper = (q & h) != 0;
 #pragma unroll
@@ -165,50 +175,67 @@ __device__ __forceinline__ void warp_fft(float2 (&v)[P], const float2* __restric
       v[a] = upper ? cmul(csub(p, v[a]), fl.tc[st]) : cadd(v[a], p);
     }
   }
-}
-
-// Forward real FFT, step 1: pack, transform, store Z[0..N) into the warp's
-// shared scratch `zs` (Z[i] at zs[zsw(i)]).  get(n) returns x[n] (0 past the
-// end).
-template <int P, class Get>
-__device__ __forceinline__ void warp_rfft_stage(Get get, float2* zs, const float2* __restrict__ tw,
-                                                const FftLane<P>& fl, int lane) {
-  float2 v[P];
+  // second transpose: point ql = q mod RQ of every RQ-point DFT; r counts the
+  // bins (g + P a) + P^2 rev(q / RQ) that the DFTs start at
+  const int ql = q % RQ;
+  const int rq = NSH > 0 ? static_cast<int>(__brev(static_cast<unsigned>(q / RQ)) >> (32 - (NSH > 0 ? NSH : 1))) : 0;
+  __syncwarp();
 #pragma unroll
-  for (int t = 0; t < P; ++t) {
-    const int n = lane + 32 * t;
-    v[t] = make_float2(get(2 * n), get(2 * n + 1));
+  for (int a = 0; a < P; ++a) scr[ql * (SH::BLK + SH::SKEW) + g + P * a + P * P * rq] = v[a];
+  __syncwarp();
+  constexpr int H = SH::BLK / 32;
+#pragma unroll
+  for (int h = 0; h < H; ++h) {
+    float2 u[RQ];
+#pragma unroll
+    for (int j = 0; j < RQ; ++j) u[j] = scr[j * (SH::BLK + SH::SKEW) + lane + 32 * h];
+    reg_dft<RQ, P>(u, tw);
+#pragma unroll
+    for (int j = 0; j < RQ; ++j) v[h + H * j] = u[j];
   }
-  warp_fft<P>(v, tw, fl, lane, zs);
-#pragma unroll
-  for (int k = 0; k < P; ++k) zs[zsw(fft_out<P>(lane, k))] = v[k];
   __syncwarp();
 }
 
-// Forward real FFT, step 2: bin k (0 <= k <= N) of the length-2N real DFT.
+// Bin k of the length-2N real DFT from zk = Z[k] and zc = conj(Z[N - k])
+// (Z[N] = Z[0]), w = tw[k]:
 //   X[k] = E[k] + W_L^k O[k],  E = (Z[k] + conj Z[N-k]) / 2,
-//   O = (Z[k] - conj Z[N-k]) / 2i,  with Z[N] = Z[0].
-template <int P>
-__device__ __forceinline__ float2 rfft_bin(const float2* zs, const float2* __restrict__ tw, int k) {
-  constexpr int N = 32 * P;
-  const float2 zk = zs[zsw(k & (N - 1))];
-  const float2 zc = cconj(zs[zsw((N - k) & (N - 1))]);
+//   O = (Z[k] - conj Z[N-k]) / 2i.
+__device__ __forceinline__ float2 rfft_bin(float2 zk, float2 zc, float2 w) {
   const float2 e = cscale(cadd(zk, zc), 0.5f);
   const float2 d = csub(zk, zc);
   const float2 o = make_float2(0.5f * d.y, -0.5f * d.x);
-  return cadd(e, cmul(tw[k], o));
+  return cadd(e, cmul(w, o));
+}
+
+// Forward real FFT: z[t] = x[2n] + i x[2n + 1], n = lane + 32 t (zero-padded
+// by the caller); hands bin k (0 <= k <= N) to put(k, X[k]).  scr: the warp's
+// shared scratch of FftShape<P>::SCR complex entries.
+template <int P, class Put>
+__device__ __forceinline__ void warp_rfft(float2 (&z)[P], Put put, const float2* __restrict__ tw,
+                                          const FftLane<P>& fl, int lane, float2* scr) {
+  constexpr int N = 32 * P;
+  warp_fft<P>(z, tw, fl, lane, scr);
+#pragma unroll
+  for (int t = 0; t < P; ++t) scr[lane + 32 * t] = z[t];
+  __syncwarp();
+#pragma unroll
+  for (int t = 0; t < P; ++t) {
+    const int k = lane + 32 * t;
+    put(k, rfft_bin(z[t], cconj(scr[(N - k) & (N - 1)]), tw[k]));
+  }
+  if (lane == 0) put(N, rfft_bin(z[0], cconj(z[0]), tw[N]));
+  __syncwarp();
 }
 
 // Inverse real FFT with truncation: from the N + 1 bins X[0..N] of a real
-// length-2N signal, produce its first N samples
+// length-2N signal, its first N samples
 //   x[n] = (1/L) sum_{k<L} X[k] W_L^(-n k),  n < N,
-// handing each to put(n, value).  getx(k) returns X[k] for 0 <= k <= N; scr
-// is the warp's shared scratch of N complex entries.
-template <int P, class GetX, class Put>
-__device__ __forceinline__ void warp_irfft_head(GetX getx, Put put, const float2* __restrict__ tw,
+// as z[t] = (x[2n], x[2n + 1]), n = lane + 32 t, for n < N / 2 (t < P / 2; lane
+// < 16 with P = 1).  getx(k) returns X[k] for 0 <= k <= N; scr as warp_rfft's.
+template <int P, class GetX>
+__device__ __forceinline__ void warp_irfft_head(GetX getx, float2 (&z)[P], const float2* __restrict__ tw,
                                                 const FftLane<P>& fl, int lane, float2* scr) {
   constexpr int N = 32 * P;
-  float2 v[P];
 #pragma unroll
   for (int t = 0; t < P; ++t) {
     const int k = lane + 32 * t;
@@ -217,18 +244,12 @@ __device__ __forceinline__ void warp_irfft_head(GetX getx, Put put, const float2
     const float2 e = cscale(cadd(xk, xc), 0.5f);
     const float2 o = cmul(cscale(csub(xk, xc), 0.5f), cconj(tw[k]));
     // Z = E + i O, fed to the forward transform conjugated (inverse by conjugation)
-    v[t] = make_float2(e.x - o.y, -(e.y + o.x));
+    z[t] = make_float2(e.x - o.y, -(e.y + o.x));
   }
-  warp_fft<P>(v, tw, fl, lane, scr);
+  warp_fft<P>(z, tw, fl, lane, scr);
   const float s = 1.0f / static_cast<float>(N);
 #pragma unroll
-  for (int k = 0; k < P; ++k) {
-    const int n = fft_out<P>(lane, k);
-    if (n < N / 2) {
-      put(2 * n, v[k].x * s);
-      put(2 * n + 1, -v[k].y * s);
-    }
-  }
+  for (int t = 0; t < P; ++t) z[t] = make_float2(z[t].x * s, -z[t].y * s);
 }
 
 }  // namespace s2w

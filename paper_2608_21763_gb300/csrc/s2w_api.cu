@@ -477,7 +477,7 @@ int tc_gemm_epi0(s2w_ctx* ctx, const void* A, const void* A_lo, long long M, lon
 //   uhat = FFT(ZeroPad(D_t^T(Truncate(IFFT(what)))))      (FP32 FFT retransform, writes B directly)
 //   ghat_l = Ghat_l^H uhat_l  (A = Ghat_l^T, K = grid);   g = Truncate(IFFT(ghat))
 int adjoint_tensor(s2w_ctx* ctx, const float* r_d, int B, float* g_d, cudaStream_t st) {
-  const long long Ns = ctx->Ns, Ng = ctx->Ng, No = ctx->No, Nt = ctx->Nt, Nb = ctx->Nb;
+  const long long Ns = ctx->Ns, Ng = ctx->Ng, No = ctx->No, Nt = ctx->Nt;
   const int sp = ctx->tc_split ? 1 : 0;
   const int dt_t = ctx->opts.dt_mode == S2W_DT_NONE ? S2W_DT_NONE : kDtTranspose;
   for (int b0 = 0; b0 < B; b0 += ctx->tc_bsub) {
@@ -485,14 +485,9 @@ int adjoint_tensor(s2w_ctx* ctx, const float* r_d, int B, float* g_d, cudaStream
     int N1 = static_cast<int>(round_up(2 * Bs, 16));
     if (N1 > 256) N1 = 512;
     {
-      StageTimer t(ctx, 0, st);
-      CK(launch_rfft_rows(r_d + static_cast<long long>(b0) * No * Nt, Bs * No, static_cast<int>(Nt),
-                          static_cast<int>(Nt), ctx->tw, ctx->ws_rhat, Bs * No, No, No, st));
-    }
-    {
       StageTimer t(ctx, 6, st);
-      CK(launch_pack_b(ctx->ws_rhat, static_cast<int>(Nb), Bs, No, static_cast<long long>(Bs) * No, No, 0, ctx->NoP,
-                       ctx->tc_n1max, 1, ctx->tc_rb, ctx->tc_rb_lo, st));
+      CK(launch_rfft_pack(r_d + static_cast<long long>(b0) * No * Nt, Bs * No, static_cast<int>(Nt), ctx->tw, No,
+                          ctx->NoP, ctx->tc_n1max, 1, ctx->tc_rb, ctx->tc_rb_lo, st));
     }
     float2* what = static_cast<float2*>(ctx->tc_mhat);
     // the GEMM retransform (D_t^T matrix) rounds what to BF16 anyway; the
@@ -567,24 +562,25 @@ int waveforms_tensor(s2w_ctx* ctx, const float* slip_d, int B, float* q_d, cudaS
     const bool f8f8 = f8 && ctx->tc_f8act && m1 >= 2;
     int N1 = static_cast<int>(round_up(2 * Bs, f8f8 ? 32 : 16));
     if (N1 > 256) N1 = 512;
-    {
+    const int* lens = ctx->cur_lens ? ctx->cur_lens + b0 : nullptr;
+    if (!f8) {  // BF16 operand, written by the transform itself (padding columns stay zero)
+      StageTimer t(ctx, 6, st);
+      CK(launch_rfft_pack(slip_d + static_cast<long long>(b0) * Ns * Nt, Bs * Ns, static_cast<int>(Nt), ctx->tw, Ns,
+                          Ns_pad, ctx->tc_n1max, 0, ctx->tc_bp1, ctx->tc_bp1_lo, st, lens));
+    } else {
       StageTimer t(ctx, 0, st);
       CK(launch_rfft_rows(slip_d + static_cast<long long>(b0) * Ns * Nt, Bs * Ns, static_cast<int>(Nt),
-                          static_cast<int>(Nt), ctx->tw, ctx->ws_shat, Bs * Ns_pad, Ns, Ns_pad, st,
-                          ctx->cur_lens ? ctx->cur_lens + b0 : nullptr));
+                          static_cast<int>(Nt), ctx->tw, ctx->ws_shat, Bs * Ns_pad, Ns, Ns_pad, st, lens));
     }
-    {
-      StageTimer t(ctx, 6, st, f8 && !f8f8 ? 2 : 1);
+    if (f8) {
+      StageTimer t(ctx, 6, st, f8f8 ? 1 : 2);
       if (f8f8)  // e4m3 operand (+ lo parts), one power-of-two scale per (bin, rupture)
         CK(launch_pack_b_f8(ctx->ws_shat, static_cast<int>(Nb), Bs, Ns_pad, static_cast<long long>(Bs) * Ns_pad,
                             Ns_pad, Ns_pad, ctx->tc_n1max, N1, ctx->tc_colscale, ctx->tc_n1max / 2, ctx->tc_bp1,
                             ctx->tc_f8lo ? ctx->tc_bp1_lo : nullptr, st));
-      else if (f8)  // FP16 operand for the FP16 MMAs of the FP8 path, scaled by a power of two from its amax
+      else  // FP16 operand for the FP16 MMAs of the FP8 path, scaled by a power of two from its amax
         CK(launch_pack_b_f16(ctx->ws_shat, static_cast<int>(Nb), Bs, Ns_pad, static_cast<long long>(Bs) * Ns_pad,
                              Ns_pad, Ns_pad, ctx->tc_n1max, ctx->d_amax, ctx->tc_bp1, st));
-      else
-        CK(launch_pack_b(ctx->ws_shat, static_cast<int>(Nb), Bs, Ns_pad, static_cast<long long>(Bs) * Ns_pad, Ns_pad,
-                         0, Ns_pad, ctx->tc_n1max, 0, ctx->tc_bp1, ctx->tc_bp1_lo, st));
     }
     if (f8f8) {
       StageTimer t(ctx, 1, st);
@@ -1055,8 +1051,8 @@ int s2w_create(int Ns, int Ng, int No, int Nt, const s2w_opts* opts, s2w_ctx** o
     const size_t mh = sizeof(float2) * Nb * Ng, vh = sizeof(float2) * Nb * ctx->nseg * ctx->RL;
     const size_t gp = sizeof(float2) * Nb * ctx->adj_nchunk * ctx->Ns_pad;
     size_t free_b = 0, total_b = 0;
-    if ((e = cudaMemGetInfo(&free_b, &total_b)) != cudaSuccess) return bad(e, "free memory");
     int m = static_cast<int>(std::min<long long>(B, kStreamMulti));
+    if (m > 1 && (e = cudaMemGetInfo(&free_b, &total_b)) != cudaSuccess) return bad(e, "free memory");
     while (m > 1 && static_cast<size_t>(m) * ((mh + vh) * (ctx->df ? 2 : 1) + gp) > free_b / 8) m /= 2;
     ctx->multi = m;
     if ((e = dalloc(&ctx->ws_mhat, m * mh)) != cudaSuccess) return bad(e, "seafloor spectra");

@@ -134,6 +134,13 @@ cudaError_t launch_twiddles(float2* tw, int L, cudaStream_t st);
 cudaError_t launch_rfft_rows(const float* x, long long rows, int n_in, int Nt, const float2* tw, float2* X,
                              long long ld_l, long long rows_a, long long ld_a, cudaStream_t st,
                              const int* lens = nullptr);
+// launch_rfft_rows of rows of Nt samples straight into the B operand of the
+// real embedding (launch_pack_b with complex columns row % rows_a of operand
+// rows 2t, 2t + 1, t = row / rows_a: dst[l][N_alloc][Kc], hi and optional lo;
+// conj 0 or 1).
+cudaError_t launch_rfft_pack(const float* x, long long rows, int Nt, const float2* tw, long long rows_a,
+                             long long Kc, int N_alloc, int conj, void* hi, void* lo, cudaStream_t st,
+                             const int* lens = nullptr);
 // Rows X[row][0..Nt] -> first Nt samples x[row][0..Nt) of the length-2Nt IFFT.
 cudaError_t launch_irfft_rows(const float2* X, long long rows, int Nt, const float2* tw, float* x, cudaStream_t st);
 // Retransform of `nb` ruptures (grid y): rupture y reads mhat + y * mhat_ld_b
