@@ -1968,16 +1968,13 @@ int s2w_autotune(s2w_ctx* ctx, int B, s2w_tuning* out, void* stream) {
       set_s2_chunks(ctx, best_c);
     }
     r.tc_s2_chunks = ctx->tc_nkc;
-    // 3. the smallest batch whose tensor pass beats the stream engine
+    // 3. the smallest batch whose tensor pass beats that many stream passes of one rupture
     const int sizes[7] = {1, 2, 4, 8, 16, 32, 64};
     int min_b = 0;
     for (int k = 0; k < 7 && rc == S2W_OK; ++k) {
       if (sizes[k] > B || sizes[k] > ctx->tc_bsub) break;
       rc = timed(sizes[k], S2W_ENGINE_TENSOR, &r.ms_tensor_batch[k]);
-      if (rc != S2W_OK || min_b != 0) continue;
-      float ms_stream = r.ms_stream_per_rupture;  // the stream engine on the same batch
-      if (sizes[k] > 1) rc = timed(sizes[k], S2W_ENGINE_STREAM, &ms_stream);
-      if (rc == S2W_OK && r.ms_tensor_batch[k] < ms_stream) min_b = sizes[k];
+      if (rc == S2W_OK && min_b == 0 && r.ms_tensor_batch[k] < sizes[k] * r.ms_stream_per_rupture) min_b = sizes[k];
     }
     if (min_b == 0) min_b = r.ms_tensor_batch[0] > 0.f ? ctx->tc_bsub + 1 : ctx->tc_min_batch;
     ctx->tc_min_batch = min_b;
