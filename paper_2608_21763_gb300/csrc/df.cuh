@@ -54,6 +54,38 @@ __device__ __forceinline__ dfl df_mul(dfl x, dfl y) {
   return fast_two_sum(p.hi, p.lo);
 }
 
+// x + y with the low parts added plainly: relative error a small multiple of
+// 2^-48 of |x| + |y| (not of |x + y|), which is what a transform's butterflies
+// need; 11 operations instead of 20.
+__device__ __forceinline__ dfl df_add_fast(dfl x, dfl y) {
+  const dfl s = two_sum(x.hi, y.hi);
+  return fast_two_sum(s.hi, s.lo + (x.lo + y.lo));
+}
+
+// Complex pairs: (re.hi, re.lo, im.hi, im.lo).
+struct dfc {
+  dfl re, im;
+};
+
+__device__ __forceinline__ dfc dc_add(dfc a, dfc b) { return {df_add_fast(a.re, b.re), df_add_fast(a.im, b.im)}; }
+__device__ __forceinline__ dfc dc_neg(dfc a) { return {df_neg(a.re), df_neg(a.im)}; }
+__device__ __forceinline__ dfc dc_sub(dfc a, dfc b) { return dc_add(a, dc_neg(b)); }
+__device__ __forceinline__ dfc dc_conj(dfc a) { return {a.re, df_neg(a.im)}; }
+// times a power of two
+__device__ __forceinline__ dfl df_scale(dfl a, float s) { return {a.hi * s, a.lo * s}; }
+__device__ __forceinline__ dfc dc_scale(dfc a, float s) { return {df_scale(a.re, s), df_scale(a.im, s)}; }
+// a b + c d: both products exact but for the lo * lo terms, one renormalisation
+__device__ __forceinline__ dfl df_mul2(dfl a, dfl b, dfl c, dfl d) {
+  const dfl p = two_prod(a.hi, b.hi), q = two_prod(c.hi, d.hi);
+  const float pc = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, p.lo));
+  const float qc = fmaf(c.hi, d.lo, fmaf(c.lo, d.hi, q.lo));
+  const dfl s = two_sum(p.hi, q.hi);
+  return fast_two_sum(s.hi, s.lo + (pc + qc));
+}
+__device__ __forceinline__ dfc dc_mul(dfc a, dfc b) {
+  return {df_mul2(a.re, b.re, df_neg(a.im), b.im), df_mul2(a.re, b.im, a.im, b.re)};
+}
+
 // Compensated sum of many pair products: the high parts are added by TwoSum
 // into s, every rounding error and low-order part into c (plain FP32: c
 // stays ~2^-24 of the terms, so its own rounding is ~2^-48 of them).

@@ -25,14 +25,10 @@
 // streamed byte costs about two instructions; long FP8 rows go four per warp
 // pass with one butterfly reduction over the lanes for the four;
 // the per-(bin, 256-row block) scale and the power of two are undone after
-// the dot product.  FP32_HILO rows (hi and lo FP32 arrays) meet
-// a vector of pairs (x, x_lo): each product is formed exactly (TwoProduct)
-// and summed by TwoSum into double-float accumulators (df.cuh), written as
-// pairs (y, y_lo).
+// the dot product.  FP32_HILO (FP32 pairs): k_dfdot.cu.
 #include <type_traits>
 
 #include "chunk.cuh"
-#include "df.cuh"
 
 namespace s2w {
 
@@ -42,27 +38,25 @@ constexpr int kStages = 3;
 constexpr int kMaxRowLen = 1024;
 
 // EL selects the unpacker (EL_BF16 also serves the hi/lo pair when HILO);
-// SHORT: rows of at most 64 chunks, shared by lane groups; DF (with EL_FP32
-// and HILO): FP32 pair rows and vectors, double-float sums.
+// SHORT: rows of at most 64 chunks, shared by lane groups.
 // Consumer warps of k_stream_dot.  FP8 rows carry half the bytes of BF16
 // ones, so per-row work (the lane reduction, the scale) weighs more: long FP8
 // rows are taken four per warp pass (one reduction for the four), short ones
 // by twelve warps (more rows in flight; ~120 registers each, no spills).
 // One rupture's short FP32 / BF16 rows take twelve warps too.
-__host__ __device__ constexpr int stream_warps(int el, bool short_rows, bool df, int r) {
-  return (short_rows && !df && r == 1) ? 12 : 8;
+__host__ __device__ constexpr int stream_warps(bool short_rows, int r) {
+  return (short_rows && r == 1) ? 12 : 8;
 }
 
 // R > 1 (short FP32 / BF16 rows): the row meets the vectors of R ruptures,
 // each lane's slices of all R held in registers, so a batch reads the
 // operator once per R ruptures.  Otherwise a batch takes one grid slice (y)
 // per rupture.
-template <int EL, bool HILO, bool SHORT, bool DF = false, int R = 1>
-__global__ void __launch_bounds__(32 * (stream_warps(EL, SHORT, DF, R) + 1), 1)
+template <int EL, bool HILO, bool SHORT, int R = 1>
+__global__ void __launch_bounds__(32 * (stream_warps(SHORT, R) + 1), 1)
     k_stream_dot(const StreamArgs a, int stage_rows) {
-  constexpr int kConsumerWarps = stream_warps(EL, SHORT, DF, R);
-  static_assert(!DF || (EL == EL_FP32 && HILO), "pair rows: FP32 hi and lo arrays");
-  static_assert(R == 1 || (SHORT && !DF && EL != EL_FP8), "several vectors: short FP32 or BF16 rows");
+  constexpr int kConsumerWarps = stream_warps(SHORT, R);
+  static_assert(R == 1 || (SHORT && EL != EL_FP8), "several vectors: short FP32 or BF16 rows");
   using CH = Chunk<EL>;
   constexpr int C = CH::C;
   // chunk slots per lane: a short row gives each lane at most four chunks
@@ -131,7 +125,6 @@ __global__ void __launch_bounds__(32 * (stream_warps(EL, SHORT, DF, R) + 1), 1)
   const int grp = lane / lpr;   // row group within the warp
   constexpr bool F8 = EL == EL_FP8;
   float2 xr[R][F8 ? 1 : T][F8 ? 1 : C];
-  float2 xl[DF ? T : 1][DF ? C : 1];  // DF: low-order parts of x_vec
   // FP8: x_vec times a power of two sx (max |component| into [2, 4)) as FP16
   // pairs (Re, Re) and (Im, Im) for the packed products, and 1 / sx
   __half2 xrr[F8 ? T : 1][F8 ? C : 1], xii[F8 ? T : 1][F8 ? C : 1];
@@ -330,13 +323,6 @@ __global__ void __launch_bounds__(32 * (stream_warps(EL, SHORT, DF, R) + 1), 1)
                 xr[b][t][2 * q] = make_float2(v.x, v.y);
                 xr[b][t][2 * q + 1] = make_float2(v.z, v.w);
               }
-              if constexpr (DF) {
-                const float4* xvl =
-                    reinterpret_cast<const float4*>(a.x_lo + blockIdx.y * a.x_ldb + vec * a.x_stride);
-                const float4 w = (c < nchunk) ? __ldg(xvl + c * (C / 2) + q) : make_float4(0.f, 0.f, 0.f, 0.f);
-                xl[t][2 * q] = make_float2(w.x, w.y);
-                xl[t][2 * q + 1] = make_float2(w.z, w.w);
-              }
             }
           }
         }
@@ -344,41 +330,7 @@ __global__ void __launch_bounds__(32 * (stream_warps(EL, SHORT, DF, R) + 1), 1)
       const int rrow = valid ? lr : base;
       const uint4* row = reinterpret_cast<const uint4*>(buf + s * stage_bytes + rrow * row_bytes);
       const uint4* row_lo = reinterpret_cast<const uint4*>(buf_lo + s * stage_bytes + rrow * row_bytes);
-      if constexpr (DF) {
-        // (g + g_lo)(x + x_lo) per complex entry, four real pair products
-        // into two compensated accumulators per chain (two chains)
-        dacc sr[2] = {{0.f, 0.f}, {0.f, 0.f}}, si[2] = {{0.f, 0.f}, {0.f, 0.f}};
-#pragma unroll
-        for (int t = 0; t < T; ++t) {
-          const int c = sub + lpr * t;
-          if (valid && c < nchunk) {
-            float2 g[C], gl[C];
-            CH::unpack(row[c], g);
-            CH::unpack(row_lo[c], gl);
-#pragma unroll
-            for (int q = 0; q < C; ++q) {
-              const dfl gr{g[q].x, gl[q].x}, gi{g[q].y, gl[q].y};
-              const dfl xre{xr[0][t][q].x, xl[t][q].x}, xim{xr[0][t][q].y, xl[t][q].y};
-              acc_mac(sr[q & 1], gr, xre);
-              acc_mac(sr[q & 1], df_neg(gi), xim);
-              acc_mac(si[q & 1], gr, xim);
-              acc_mac(si[q & 1], gi, xre);
-            }
-          }
-        }
-        dacc ar = acc_merge(sr[0], sr[1]), ai = acc_merge(si[0], si[1]);
-        for (int o = lpr / 2; o > 0; o >>= 1) {
-          const dacc br{__shfl_xor_sync(0xffffffffu, ar.s, o), __shfl_xor_sync(0xffffffffu, ar.c, o)};
-          const dacc bi{__shfl_xor_sync(0xffffffffu, ai.s, o), __shfl_xor_sync(0xffffffffu, ai.c, o)};
-          ar = acc_merge(ar, br);
-          ai = acc_merge(ai, bi);
-        }
-        if (valid && sub == 0) {
-          const dfl yr = acc_get(ar), yi = acc_get(ai);
-          ay[f] = make_float2(yr.hi, yi.hi);
-          a.y_lo[blockIdx.y * a.y_ldb + f] = make_float2(yr.lo, yi.lo);
-        }
-      } else if constexpr (F8) {
+      if constexpr (F8) {
         // e4m3 pairs (Re, Im) widen exactly to FP16 pairs (one cvt per
         // complex entry); g * (xr, xr) and g * (xi, xi) accumulate as FP16
         // pairs over the lane's T = 4 chunks of the row (eight independent
@@ -489,7 +441,7 @@ __global__ void __launch_bounds__(32 * (stream_warps(EL, SHORT, DF, R) + 1), 1)
   }
 }
 
-template <int EL, bool HILO, bool SHORT, bool DF = false, int R = 1>
+template <int EL, bool HILO, bool SHORT, int R = 1>
 cudaError_t launch_t(const StreamArgs& a, int num_sms, cudaStream_t st) {
   constexpr int C = Chunk<EL>::C;
   const int row_bytes = a.row_len * (16 / C);
@@ -498,14 +450,14 @@ cudaError_t launch_t(const StreamArgs& a, int num_sms, cudaStream_t st) {
   if (stage_rows >= 8) stage_rows -= stage_rows % 8;
   if (stage_rows < 1) stage_rows = 1;
   const size_t smem = 128 + static_cast<size_t>(kStages) * stage_rows * row_bytes * (HILO ? 2 : 1);
-  cudaError_t e = cudaFuncSetAttribute(k_stream_dot<EL, HILO, SHORT, DF, R>,
+  cudaError_t e = cudaFuncSetAttribute(k_stream_dot<EL, HILO, SHORT, R>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   long long grid = num_sms;
   if (grid > a.F) grid = a.F;
   if (grid < 1) grid = 1;
   const dim3 g(static_cast<unsigned>(grid), R == 1 ? static_cast<unsigned>(a.nb) : 1u);
-  k_stream_dot<EL, HILO, SHORT, DF, R><<<g, 32 * (stream_warps(EL, SHORT, DF, R) + 1), smem, st>>>(a, stage_rows);
+  k_stream_dot<EL, HILO, SHORT, R><<<g, 32 * (stream_warps(SHORT, R) + 1), smem, st>>>(a, stage_rows);
   return cudaGetLastError();
 }
 
@@ -534,7 +486,7 @@ cudaError_t launch_plain(const StreamArgs& a, int num_sms, cudaStream_t st) {
     h.nb = a.nb - b < kMostVectors ? a.nb - b : kMostVectors;
     h.x = a.x + b * a.x_ldb;
     h.y = a.y + b * a.y_ldb;
-    const cudaError_t e = launch_t<EL, HILO, true, false, kMostVectors>(h, num_sms, st);
+    const cudaError_t e = launch_t<EL, HILO, true, kMostVectors>(h, num_sms, st);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -552,10 +504,7 @@ cudaError_t launch_stream_dot(const StreamArgs& a, int num_sms, cudaStream_t st)
     case EL_FP8:
       return short_rows(a, 8) ? launch_t<EL_FP8, false, true>(a, num_sms, st)
                               : launch_t<EL_FP8, false, false>(a, num_sms, st);
-    case EL_FP32_HILO:
-      if (a.rows_lo == nullptr || a.x_lo == nullptr || a.y_lo == nullptr) return cudaErrorInvalidValue;
-      return short_rows(a, 2) ? launch_t<EL_FP32, true, true, true>(a, num_sms, st)
-                              : launch_t<EL_FP32, true, false, true>(a, num_sms, st);
+    case EL_FP32_HILO: return launch_stream_df(a, num_sms, st);
     default: return cudaErrorInvalidValue;
   }
 }

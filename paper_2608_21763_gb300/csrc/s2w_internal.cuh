@@ -221,6 +221,8 @@ cudaError_t launch_stream_dot(const StreamArgs& a, int num_sms, cudaStream_t st)
 // k_multi.cu: the same for 2 .. kStreamMulti ruptures and FP32 / BF16 /
 // BF16 hi/lo rows of more than 64 16-byte chunks (launch_stream_dot calls it).
 cudaError_t launch_stream_multi(const StreamArgs& a, int num_sms, cudaStream_t st);
+// k_dfdot.cu: the same for FP32 pairs (any nb; two ruptures per pass).
+cudaError_t launch_stream_df(const StreamArgs& a, int num_sms, cudaStream_t st);
 
 // k_tdot.cu, transposed: y[u][c] = sum_{f in unit u} conj(rows[f][c]) w_f,
 // unit u = chunk (u % nchunk) of Rc rows of group (u / nchunk) of G1 rows,
