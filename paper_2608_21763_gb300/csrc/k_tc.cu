@@ -112,13 +112,16 @@ __device__ __forceinline__ void tc_commit(uint64_t* bar) {
                : "memory");
 }
 
-__device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                            uint32_t accumulate) {
+// D (+)= A B^T with shared-memory descriptors {a_lo, hi}, {b_lo, hi}.
+__device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
+                                            uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+      "mov.b64 da, {%1, %3};\n\t"
+      "mov.b64 db, {%2, %3};\n\t"
+      "setp.ne.b32 p, %5, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}" ::"r"(d_tmem),
+      "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 
@@ -167,19 +170,32 @@ __device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v)[64]) {
 // 128-byte swizzle: rows of 128 bytes, 8-row core-matrix groups 1024 bytes
 // apart (stride byte offset), tile base 1024-byte aligned; advancing along K
 // inside the swizzle row is a plain byte offset of the start address.
-template <int BK>
-__device__ __forceinline__ uint64_t sdesc_sw(uint32_t saddr) {
-  // BK = 64: rows of 128 B, 128-byte swizzle; BK = 32: rows of 64 B, 64-byte swizzle
-  constexpr uint32_t sbo = 8 * BK * 2;
-  constexpr uint64_t layout = BK == 64 ? 2 : 4;
-  uint64_t d = 0;
-  d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);  // start address
-  d |= static_cast<uint64_t>(1) << 16;                  // leading byte offset (unused here)
-  d |= static_cast<uint64_t>(sbo >> 4) << 32;           // stride byte offset (8-row groups)
-  d |= static_cast<uint64_t>(1) << 46;                  // descriptor version (tcgen05)
-  d |= layout << 61;                                    // swizzle mode
-  return d;
+// The descriptor's two words: only the low one (the start address, in 16-byte
+// units) varies, by constants within a stage, so the issuing thread keeps a
+// stage's low word and adds to it.  Building each descriptor from its address
+// (with the ring position from a division) took about 200 cycles per MMA in
+// that one thread, which held the GEMMs of up to 128 columns, not the tensor
+// cores or HBM: 963 x 8,000 x 256 at 8 ruptures, stage 1 1.62 ms with the MMAs
+// against 1.23 without.
+__device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr) {
+  return ((saddr & 0x3FFFFu) >> 4) | (1u << 16);  // start address; leading byte offset (unused here)
 }
+// BK = 64: rows of 128 B, 128-byte swizzle; BK = 32: rows of 64 B, 64-byte swizzle
+template <int BK>
+__host__ __device__ constexpr uint32_t sdesc_hi() {
+  return static_cast<uint32_t>((8 * BK * 2) >> 4) |  // stride byte offset (8-row groups)
+         (1u << 14) |                                 // descriptor version (tcgen05)
+         (static_cast<uint32_t>(BK == 64 ? 2 : 4) << 29);  // swizzle mode
+}
+
+// Position in a ring of S slots: slot, and the parity of its current lap.
+struct RingPos {
+  int s = 0;
+  uint32_t ph = 0;
+  __device__ __forceinline__ void next(int S) {
+    if (++s == S) s = 0, ph ^= 1u;
+  }
+};
 
 // Instruction descriptor, kind::f16: BF16 A and B, FP32 D, both K-major.
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
@@ -406,15 +422,16 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* tmA, const CUten
   if (warp == 0) {
     if (lane == 0) {
       int it = 0;
+      RingPos rp;
       bool ok = true;
       for (long long u = cid; u < units && ok; u += ncl) {
         int l, mt, kc;
         unit_coords(u, l, mt, kc);
         const int kb0 = a.kb_off + kc * a.kblocks_per_chunk;
         const int kb1 = min(nk_total, kb0 + a.kblocks_per_chunk);
-        for (int kb = kb0; kb < kb1; ++kb, ++it) {
-          const int s = it % S;
-          if (it >= S && !mbar_wait_bounded(empty + s, ((it / S) - 1) & 1, a.status, DEV_ERR_TIMEOUT_EMPTY)) {
+        for (int kb = kb0; kb < kb1; ++kb, ++it, rp.next(S)) {
+          const int s = rp.s;
+          if (it >= S && !mbar_wait_bounded(empty + s, rp.ph ^ 1u, a.status, DEV_ERR_TIMEOUT_EMPTY)) {
             ok = false;
             break;
           }
@@ -451,8 +468,11 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* tmA, const CUten
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      int it = 0, acc_it = 0;
+      int acc_it = 0;
+      RingPos rp;
       bool ok = true;
+      constexpr uint32_t hi = sdesc_hi<BK>();
+      const uint32_t a0 = sdesc_lo(smem_u32(smem)), stage16 = static_cast<uint32_t>(stage_bytes) >> 4;
       for (long long u = cid; u < units && ok; u += ncl) {
         int l, mt, kc;
         unit_coords(u, l, mt, kc);
@@ -463,33 +483,40 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* tmA, const CUten
           break;
         }
         tc_fence_after();
-        for (int kb = kb0; kb < kb1; ++kb, ++it) {
-          const int s = it % S;
-          if (!mbar_wait_bounded(CONV ? aready + s : full + s, (it / S) & 1, a.status, DEV_ERR_TIMEOUT_FULL)) {
+        for (int kb = kb0; kb < kb1; ++kb, rp.next(S)) {
+          const int s = rp.s;
+          if (!mbar_wait_bounded(CONV ? aready + s : full + s, rp.ph, a.status, DEV_ERR_TIMEOUT_FULL)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t sa = smem_u32(smem + s * stage_bytes);
-          const uint32_t sb = sa + a_all;
+          const uint32_t al = a0 + static_cast<uint32_t>(s) * stage16;
+          const uint32_t bl = al + (a_all >> 4);
+          const uint32_t first = kb > kb0 ? 1u : 0u;  // 0: the unit's first MMA overwrites the accumulator
+          auto kblock = [&](auto nm_tag) {
+            constexpr int NM = decltype(nm_tag)::value;  // 256-column MMAs per K step
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {
+            for (int k = 0; k < BK / 16; ++k) {
 #pragma unroll
-            for (int j = 0; j < MT; ++j) {  // accumulator j at TMEM columns j N ..
-              const uint32_t aoff = j * a_tile + k * 32;
-              const uint64_t ad = sdesc_sw<BK>(sa + aoff);
-              for (int c = 0; c < n_mma; ++c) {
-                const uint32_t boff = c * n_mma_cols * BK * 2 + k * 32;
-                const uint64_t bd = sdesc_sw<BK>(sb + boff);
-                const uint32_t dcol = tmem + j * N + c * n_mma_cols;
-                tc_mma_bf16(dcol, ad, bd, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
-                if constexpr (SPLIT) {
-                  tc_mma_bf16(dcol, ad, sdesc_sw<BK>(sb + b_bytes + boff), idesc, 1u);
-                  tc_mma_bf16(dcol, sdesc_sw<BK>(sa + aoff + kA), bd, idesc, 1u);
+              for (int j = 0; j < MT; ++j) {  // accumulator j at TMEM columns j N ..
+                const uint32_t ad = al + ((j * a_tile + k * 32) >> 4);
+#pragma unroll
+                for (int c = 0; c < NM; ++c) {
+                  const uint32_t bd = bl + ((c * 256 * BK * 2 + k * 32) >> 4);
+                  const uint32_t dcol = tmem + j * N + c * 256;
+                  tc_mma_bf16(dcol, ad, bd, hi, idesc, k > 0 ? 1u : first);
+                  if constexpr (SPLIT) {
+                    tc_mma_bf16(dcol, ad, bd + (static_cast<uint32_t>(b_bytes) >> 4), hi, idesc, 1u);
+                    tc_mma_bf16(dcol, ad + (kA >> 4), bd, hi, idesc, 1u);
+                  }
                 }
               }
             }
-          }
+          };
+          if (n_mma == 1)
+            kblock(std::integral_constant<int, 1>{});
+          else
+            kblock(std::integral_constant<int, 2>{});
           tc_commit(empty + s);
         }
         if (!ok) break;
@@ -505,16 +532,16 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* tmA, const CUten
     // and r share the 128-byte swizzle phase, N / 2 being a multiple of 8,
     // so the bytes copy straight across), 16 bytes per thread and step
     const int t = threadIdx.x - 32 * kConvWarp0;
-    int it = 0;
+    RingPos rp;
     bool ok = true;
     for (long long u = cid; u < units && ok; u += ncl) {
       int l, mt, kc;
       unit_coords(u, l, mt, kc);
       const int kb0 = a.kb_off + kc * a.kblocks_per_chunk;
       const int kb1 = min(nk_total, kb0 + a.kblocks_per_chunk);
-      for (int kb = kb0; kb < kb1; ++kb, ++it) {
-        const int s = it % S;
-        if (!mbar_wait_bounded(full + s, (it / S) & 1, a.status, DEV_ERR_TIMEOUT_FULL)) {
+      for (int kb = kb0; kb < kb1; ++kb, rp.next(S)) {
+        const int s = rp.s;
+        if (!mbar_wait_bounded(full + s, rp.ph, a.status, DEV_ERR_TIMEOUT_FULL)) {
           ok = false;
           break;
         }
@@ -699,25 +726,29 @@ __device__ __forceinline__ void tc_commit2_mc(uint64_t* bar, uint16_t mask) {
       "h"(mask)
       : "memory");
 }
-__device__ __forceinline__ void tc_mma2_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                             uint32_t accumulate) {
+__device__ __forceinline__ void tc_mma2_bf16(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
+                                             uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+      "mov.b64 da, {%1, %3};\n\t"
+      "mov.b64 db, {%2, %3};\n\t"
+      "setp.ne.b32 p, %5, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p;\n\t}" ::"r"(d_tmem),
+      "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 
 // Same with 8-bit operands (kind::f8f6f4; both e4m3 with the f16 instruction
 // descriptor's zero type fields), K = 32 per instruction.
-__device__ __forceinline__ void tc_mma2_f8f8(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                             uint32_t accumulate) {
+__device__ __forceinline__ void tc_mma2_f8f8(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
+                                             uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+      "mov.b64 da, {%1, %3};\n\t"
+      "mov.b64 db, {%2, %3};\n\t"
+      "setp.ne.b32 p, %5, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], da, db, %4, p;\n\t}" ::"r"(d_tmem),
+      "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 
@@ -827,15 +858,16 @@ __device__ __forceinline__ void tc_gemm2_body(const CUtensorMap* tmA, const CUte
     if (lane == 0) {
       const uint32_t full0 = cluster_addr(full, 0);  // rank 0's full[0]
       int it = 0;
+      RingPos rp;
       bool ok = true;
       for (long long u = cid; u < units && ok; u += ncl) {
         int l, mt, nh, kc;
         unit_coords(u, l, mt, nh, kc);
         const int kb0 = a.kb_off + kc * a.kblocks_per_chunk;
         const int kb1 = min(nk_total, kb0 + a.kblocks_per_chunk);
-        for (int kb = kb0; kb < kb1; ++kb, ++it) {
-          const int s = it % S;
-          if (it >= S && !mbar_wait_bounded(empty + s, ((it / S) - 1) & 1, a.status, DEV_ERR_TIMEOUT_EMPTY)) {
+        for (int kb = kb0; kb < kb1; ++kb, ++it, rp.next(S)) {
+          const int s = rp.s;
+          if (it >= S && !mbar_wait_bounded(empty + s, rp.ph ^ 1u, a.status, DEV_ERR_TIMEOUT_EMPTY)) {
             ok = false;
             break;
           }
@@ -868,8 +900,12 @@ __device__ __forceinline__ void tc_gemm2_body(const CUtensorMap* tmA, const CUte
     }
   } else if (warp == 1) {
     if (lane == 0 && lead) {
-      int it = 0, acc_it = 0;
+      int acc_it = 0;
+      RingPos rp;
       bool ok = true;
+      constexpr uint32_t hi = sdesc_hi<BKB / 2>();
+      const uint32_t a0 = sdesc_lo(smem_u32(smem)), stage16 = static_cast<uint32_t>(stage_bytes) >> 4;
+      const uint32_t b_off = static_cast<uint32_t>(a_bytes) >> 4, blo_off = static_cast<uint32_t>(bh_bytes) >> 4;
       for (long long u = cid; u < units && ok; u += ncl) {
         int l, mt, nh, kc;
         unit_coords(u, l, mt, nh, kc);
@@ -882,36 +918,45 @@ __device__ __forceinline__ void tc_gemm2_body(const CUtensorMap* tmA, const CUte
           break;
         }
         tc_fence_after();
-        for (int kb = kb0; kb < kb1; ++kb, ++it) {
-          const int s = it % S;
-          const bool got = F8 ? mbar_wait_bounded_cl(aready + s, (it / S) & 1, a.status, DEV_ERR_TIMEOUT_FULL)
-                              : mbar_wait_bounded(full + s, (it / S) & 1, a.status, DEV_ERR_TIMEOUT_FULL);
+        const uint32_t dtm = tmem + static_cast<uint32_t>(as * NU);
+        for (int kb = kb0; kb < kb1; ++kb, rp.next(S)) {
+          const int s = rp.s;
+          const bool got = F8 ? mbar_wait_bounded_cl(aready + s, rp.ph, a.status, DEV_ERR_TIMEOUT_FULL)
+                              : mbar_wait_bounded(full + s, rp.ph, a.status, DEV_ERR_TIMEOUT_FULL);
           if (!got) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t sa = smem_u32(smem + s * stage_bytes);
-          const uint32_t sb = sa + a_bytes;
+          const uint32_t al = a0 + static_cast<uint32_t>(s) * stage16;
+          const uint32_t first = kb > kb0 ? 1u : 0u;  // 0: the unit's first MMA overwrites the accumulator
+          auto kblock = [&](auto nm_tag) {
+            constexpr int NM = decltype(nm_tag)::value;  // 256-column MMAs per K step
 #pragma unroll
-          for (int k = 0; k < BK / KI; ++k) {
-            const uint64_t ad = sdesc_sw<BKB / 2>(sa + k * 32);
-            for (int c = 0; c < n_mma; ++c) {
-              const uint32_t boff = c * hb + k * 32;
-              const uint64_t bd = sdesc_sw<BKB / 2>(sb + boff);
-              const uint32_t dcol = tmem + static_cast<uint32_t>(as * NU + c * n_mma_cols);
-              if constexpr (F8F8) {
-                tc_mma2_f8f8(dcol, ad, bd, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
-                if constexpr (BLO) tc_mma2_f8f8(dcol, ad, sdesc_sw<BKB / 2>(sb + bh_bytes + boff), idesc, 1u);
-              } else {
-                tc_mma2_bf16(dcol, ad, bd, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
-              }
-              if constexpr (SPLIT) {
-                tc_mma2_bf16(dcol, ad, sdesc_sw<BK>(sb + bh_bytes + boff), idesc, 1u);
-                tc_mma2_bf16(dcol, sdesc_sw<BK>(sa + kA + k * 32), bd, idesc, 1u);
+            for (int k = 0; k < BK / KI; ++k) {
+              const uint32_t ad = al + ((k * 32) >> 4);
+#pragma unroll
+              for (int c = 0; c < NM; ++c) {
+                const uint32_t bd = al + b_off + ((c * 128 * BKB + k * 32) >> 4);  // (c > 0: slices of 128 staged rows)
+                const uint32_t dcol = dtm + c * 256;
+                const uint32_t acc = k > 0 ? 1u : first;
+                if constexpr (F8F8) {
+                  tc_mma2_f8f8(dcol, ad, bd, hi, idesc, acc);
+                  if constexpr (BLO) tc_mma2_f8f8(dcol, ad, bd + blo_off, hi, idesc, 1u);
+                } else {
+                  tc_mma2_bf16(dcol, ad, bd, hi, idesc, acc);
+                }
+                if constexpr (SPLIT) {
+                  tc_mma2_bf16(dcol, ad, bd + blo_off, hi, idesc, 1u);
+                  tc_mma2_bf16(dcol, ad + (kA >> 4), bd, hi, idesc, 1u);
+                }
               }
             }
-          }
+          };
+          if (n_mma == 1)
+            kblock(std::integral_constant<int, 1>{});
+          else
+            kblock(std::integral_constant<int, 2>{});
           tc_commit2_mc(empty + s, 0x3);
         }
         if (!ok) break;
@@ -926,16 +971,16 @@ __device__ __forceinline__ void tc_gemm2_body(const CUtensorMap* tmA, const CUte
     // converter warps of both CTAs: thread t widens row t of this CTA's FP8 A tile
     const int t = threadIdx.x - 32 * kConvWarp0;
     const uint32_t aready0 = cluster_addr(aready, 0);
-    int it = 0;
+    RingPos rp;
     bool ok = true;
     for (long long u = cid; u < units && ok; u += ncl) {
       int l, mt, nh, kc;
       unit_coords(u, l, mt, nh, kc);
       const int kb0 = a.kb_off + kc * a.kblocks_per_chunk;
       const int kb1 = min(nk_total, kb0 + a.kblocks_per_chunk);
-      for (int kb = kb0; kb < kb1; ++kb, ++it) {
-        const int s = it % S;
-        if (!mbar_wait_bounded(full + s, (it / S) & 1, a.status, DEV_ERR_TIMEOUT_FULL)) {
+      for (int kb = kb0; kb < kb1; ++kb, rp.next(S)) {
+        const int s = rp.s;
+        if (!mbar_wait_bounded(full + s, rp.ph, a.status, DEV_ERR_TIMEOUT_FULL)) {
           ok = false;
           break;
         }
@@ -1307,15 +1352,16 @@ __global__ void __launch_bounds__(rt_threads(SPLIT), 1)
     // T slots in job order: tile, unit, k-block, half within the unit
     if (lane == 0) {
       int it = 0;
+      RingPos rp;
       bool ok = true;
       const uint32_t tfull0 = PAIR ? cluster_addr(tfull, 0) : 0u;
       for (long long t = cid; t < tiles && ok; t += ncl) {
         for (int u = 0; u < U && ok; ++u) {
           for (int kb = 0; kb < KB && ok; ++kb) {
-            for (int hh = 0; hh < H; ++hh, ++it) {
+            for (int hh = 0; hh < H; ++hh, ++it, rp.next(RT)) {
               const int h = hout ? u : hh;
-              const int s = it % RT;
-              if (it >= RT && !mbar_wait_bounded(tempty + s, ((it / RT) - 1) & 1, a.status, DEV_ERR_TIMEOUT_EMPTY)) {
+              const int s = rp.s;
+              if (it >= RT && !mbar_wait_bounded(tempty + s, rp.ph ^ 1u, a.status, DEV_ERR_TIMEOUT_EMPTY)) {
                 ok = false;
                 break;
               }
@@ -1351,7 +1397,11 @@ __global__ void __launch_bounds__(rt_threads(SPLIT), 1)
         else
           tc_commit(bar);
       };
-      int it = 0, tl = 0, un = 0;  // T slot, tile and accumulator unit counters
+      int tl = 0, un = 0;  // tile and accumulator unit counters
+      RingPos rp;          // T slot
+      constexpr uint32_t hi = sdesc_hi<BK>();
+      const uint32_t a0 = sdesc_lo(smem_u32(sA)), b0 = sdesc_lo(smem_u32(sT));
+      const uint32_t t_slot16 = static_cast<uint32_t>(t_slot) >> 4, t_part16 = static_cast<uint32_t>(t_part) >> 4;
       bool ok = true;
       for (long long t = cid; t < tiles && ok; t += ncl, ++tl) {
         for (int u = 0; u < U && ok; ++u, ++un) {
@@ -1369,27 +1419,27 @@ __global__ void __launch_bounds__(rt_threads(SPLIT), 1)
               ok = false;
               break;
             }
-            for (int hh = 0; hh < H; ++hh, ++it) {
-              const int s = it % RT;
-              if (!mbar_wait_bounded(tfull + s, (it / RT) & 1, a.status, DEV_ERR_TIMEOUT_FULL)) {
+            for (int hh = 0; hh < H; ++hh, rp.next(RT)) {
+              const int s = rp.s;
+              if (!mbar_wait_bounded(tfull + s, rp.ph, a.status, DEV_ERR_TIMEOUT_FULL)) {
                 ok = false;
                 break;
               }
               tc_fence_after();
-              const uint32_t ua = smem_u32(sA + sa * a_slot);
-              const uint32_t ub = smem_u32(sT + s * t_slot);
+              const uint32_t al = a0 + static_cast<uint32_t>(sa) * (a_slot >> 4);
+              const uint32_t bl = b0 + static_cast<uint32_t>(s) * t_slot16;
               const uint32_t d = dcol + static_cast<uint32_t>(hh * ncols);
 #pragma unroll
               for (int k = 0; k < BK / 16; ++k) {
-                const uint64_t ad = sdesc_sw<BK>(ua + k * 32);
-                const uint64_t bd = sdesc_sw<BK>(ub + k * 32);
+                const uint32_t ad = al + ((k * 32) >> 4), bd = bl + ((k * 32) >> 4);
+                const uint32_t acc = k > 0 ? 1u : (kb > 0 ? 1u : 0u);
                 if constexpr (PAIR)
-                  tc_mma2_bf16(d, ad, bd, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+                  tc_mma2_bf16(d, ad, bd, hi, idesc, acc);
                 else
-                  tc_mma_bf16(d, ad, bd, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+                  tc_mma_bf16(d, ad, bd, hi, idesc, acc);
                 if constexpr (SPLIT) {
-                  tc_mma_bf16(d, ad, sdesc_sw<BK>(ub + t_part + k * 32), idesc, 1u);
-                  tc_mma_bf16(d, sdesc_sw<BK>(ua + kAs + k * 32), bd, idesc, 1u);
+                  tc_mma_bf16(d, ad, bd + t_part16, hi, idesc, 1u);
+                  tc_mma_bf16(d, ad + (kAs >> 4), bd, hi, idesc, 1u);
                 }
               }
               commit(tempty + s);
