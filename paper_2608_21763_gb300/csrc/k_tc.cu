@@ -174,9 +174,12 @@ __device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v)[64]) {
 // units) varies, by constants within a stage, so the issuing thread keeps a
 // stage's low word and adds to it.  Building each descriptor from its address
 // (with the ring position from a division) took about 200 cycles per MMA in
-// that one thread, which held the GEMMs of up to 128 columns, not the tensor
-// cores or HBM: 963 x 8,000 x 256 at 8 ruptures, stage 1 1.62 ms with the MMAs
-// against 1.23 without.
+// that one thread, and held every GEMM here below the tensor cores and HBM
+// (963 x 8,000 x 256 at 8 ruptures: stage 1 1.62 ms, 1.23 with the MMAs left
+// out).  Stage 1 per launch, before and after: 963 x 20,000, 8 ruptures BF16,
+// 3.94 -> 3.05 ms (0.96 of the copy rate); 963 x 37,758, 256 ruptures BF16, 13.5
+// -> 11.8 (1.01 of the sustained BF16 rate); 963 x 50,000, 256 ruptures FP8 hi +
+// lo, 17.6 -> 15.9.
 __device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr) {
   return ((saddr & 0x3FFFFu) >> 4) | (1u << 16);  // start address; leading byte offset (unused here)
 }
