@@ -26,9 +26,11 @@
 //   warps 2-17 epilogue: tcgen05.ld of the accumulator (warp w reads TMEM
 //              lanes 32 (w % 4) .. +31, i.e. tile rows, and every fourth
 //              64-column chunk), scale, store.  Four warps per lane quadrant
-//              cut the time the MMAs wait for the accumulator to drain
-//              (with N = 512 it fills tensor memory, so it cannot be
-//              double-buffered); FP8 kernels keep two per quadrant.  The
+//              cut the time the MMAs wait for the accumulator to drain where
+//              one unit's accumulators fill more than half of tensor memory;
+//              smaller ones alternate between two sets (tc_acc_sets), so the
+//              drain overlaps the next unit's MMAs (split adjoint of 64
+//              ruptures: 0.52 ms of 6.1); FP8 kernels keep two per quadrant.  The
 //              two-SM FP8 x (hi + lo FP8) kernel at N = 512 instead splits
 //              the columns into two 256-column units (n_split) whose
 //              accumulators alternate, so the drain overlaps the MMAs.
@@ -190,6 +192,9 @@ __host__ __device__ constexpr uint32_t sdesc_hi() {
          (1u << 14) |                                 // descriptor version (tcgen05)
          (static_cast<uint32_t>(BK == 64 ? 2 : 4) << 29);  // swizzle mode
 }
+
+// Accumulator sets of `cols` columns that tensor memory (512) holds, at most two.
+__host__ __device__ constexpr int tc_acc_sets(int cols) { return 2 * cols <= 512 ? 2 : 1; }
 
 // Position in a ring of S slots: slot, and the parity of its current lap.
 struct RingPos {
@@ -384,8 +389,12 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* tmA, const CUten
   uint64_t* empty = full + S;
   uint64_t* aready = empty + S;  // F8 / BH: the stage completed (count 4 converter warps)
   uint64_t* acc_full = aready + (CONV ? S : 0);
-  uint64_t* acc_empty = acc_full + 1;
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(acc_empty + 1);
+  uint64_t* acc_empty = acc_full + 2;
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(acc_empty + 2);
+  // accumulators of a unit, and how many such sets tensor memory holds: with
+  // two, the epilogue drains one while the MMAs fill the other
+  const int AC = MT * N;
+  const int AS = tc_acc_sets(AC);
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int nk_total = (a.K + BK - 1) / BK;
@@ -402,8 +411,10 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* tmA, const CUten
       mbar_init(empty + s, 1);
       if (CONV) mbar_init(aready + s, 4);
     }
-    mbar_init(acc_full, 1);
-    mbar_init(acc_empty, kEpiWarps);
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(acc_full + s, 1);
+      mbar_init(acc_empty + s, kEpiWarps);
+    }
     fence_mbar_init();
   }
   if (warp == 1) {
@@ -481,11 +492,14 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* tmA, const CUten
         unit_coords(u, l, mt, kc);
         const int kb0 = a.kb_off + kc * a.kblocks_per_chunk;
         const int kb1 = min(nk_total, kb0 + a.kblocks_per_chunk);
-        if (acc_it > 0 && !mbar_wait_bounded(acc_empty, (acc_it - 1) & 1, a.status, DEV_ERR_TIMEOUT_MMA)) {
+        const int as = acc_it & (AS - 1);
+        if (acc_it >= AS && !mbar_wait_bounded(acc_empty + as, ((acc_it >> (AS - 1)) - 1) & 1, a.status,
+                                               DEV_ERR_TIMEOUT_MMA)) {
           ok = false;
           break;
         }
         tc_fence_after();
+        const uint32_t dtm = tmem + static_cast<uint32_t>(as * AC);
         for (int kb = kb0; kb < kb1; ++kb, rp.next(S)) {
           const int s = rp.s;
           if (!mbar_wait_bounded(CONV ? aready + s : full + s, rp.ph, a.status, DEV_ERR_TIMEOUT_FULL)) {
@@ -506,7 +520,7 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* tmA, const CUten
 #pragma unroll
                 for (int c = 0; c < NM; ++c) {
                   const uint32_t bd = bl + ((c * 256 * BK * 2 + k * 32) >> 4);
-                  const uint32_t dcol = tmem + j * N + c * 256;
+                  const uint32_t dcol = dtm + j * N + c * 256;
                   tc_mma_bf16(dcol, ad, bd, hi, idesc, k > 0 ? 1u : first);
                   if constexpr (SPLIT) {
                     tc_mma_bf16(dcol, ad, bd + (static_cast<uint32_t>(b_bytes) >> 4), hi, idesc, 1u);
@@ -523,11 +537,12 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* tmA, const CUten
           tc_commit(empty + s);
         }
         if (!ok) break;
-        tc_commit(acc_full);
+        tc_commit(acc_full + as);
         ++acc_it;
       }
-      // the epilogue consumes the last accumulator; wait for it before teardown
-      if (acc_it > 0) mbar_wait_bounded(acc_empty, (acc_it - 1) & 1, a.status, DEV_ERR_TIMEOUT_MMA);
+      // the epilogue consumes the last accumulators; wait for it before teardown
+      for (int k = (acc_it > AS ? acc_it - AS : 0); k < acc_it; ++k)
+        mbar_wait_bounded(acc_empty + (k & (AS - 1)), (k >> (AS - 1)) & 1, a.status, DEV_ERR_TIMEOUT_MMA);
     }
   } else if (CONV && warp >= kConvWarp0) {
     // converter warps.  F8: thread t widens row t of each FP8 A tile.  BH:
@@ -572,12 +587,13 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* tmA, const CUten
     for (long long u = cid; u < units; u += ncl) {
       int l, mt, kc;
       unit_coords(u, l, mt, kc);
-      if (!mbar_wait_bounded(acc_full, acc_it & 1, a.status, DEV_ERR_TIMEOUT_MMA)) break;
+      const int as = acc_it & (AS - 1);
+      if (!mbar_wait_bounded(acc_full + as, (acc_it >> (AS - 1)) & 1, a.status, DEV_ERR_TIMEOUT_MMA)) break;
       tc_fence_after();
 #pragma unroll 1
       for (int j = 0; j < MT; ++j) {
         const int row = (mt + j) * kBlockM + q * 32 + lane;
-        const uint32_t tbase = tmem + j * N + (static_cast<uint32_t>(q * 32) << 16);
+        const uint32_t tbase = tmem + as * AC + j * N + (static_cast<uint32_t>(q * 32) << 16);
         const bool live = row < a.M_total && mt + j < a.m_tiles;
         float scale = 1.f;
         if (a.row_scale != nullptr && live) scale = a.row_scale[static_cast<long long>(l) * a.nblk + row / 256];
@@ -589,7 +605,7 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* tmA, const CUten
       }  // M tiles of the unit
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(acc_empty);
+      if (lane == 0) mbar_arrive(acc_empty + as);
       ++acc_it;
     }
   }
@@ -801,7 +817,7 @@ __device__ __forceinline__ void tc_gemm2_body(const CUtensorMap* tmA, const CUte
   // MMAs of the next unit run while the epilogue drains the last one
   const int NS = (BLO && a.n_split == 2) ? 2 : 1;
   const int NU = N / NS;       // accumulator columns per unit
-  const int AS = NS;           // accumulators in tensor memory
+  const int AS = tc_acc_sets(NU);  // accumulators in tensor memory
   const int n_mma = NU > 256 ? NU / 256 : 1;
   const int n_mma_cols = NU > 256 ? 256 : NU;
   const int hrows = n_mma_cols / 2;  // B rows this CTA stages per MMA slice
@@ -814,7 +830,7 @@ __device__ __forceinline__ void tc_gemm2_body(const CUtensorMap* tmA, const CUte
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + S * stage_bytes);
   uint64_t* empty = full + S;
   uint64_t* aready = empty + S;  // F8, rank 0: both CTAs' A slots widened
-  constexpr int kAccBars = BLO ? 2 : 1;  // hi + lo B may alternate two accumulators
+  constexpr int kAccBars = 2;
   uint64_t* acc_full = aready + (F8 ? S : 0);
   uint64_t* acc_empty = acc_full + kAccBars;
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(acc_empty + kAccBars);
@@ -1768,7 +1784,7 @@ int tc_stages_for(int N, int a_lo, int b_lo, int fp8, int mt) {
 }
 
 size_t tc_smem_bytes(int N, int stages, int a_lo, int b_lo, int fp8, int mt) {
-  return 1024 + static_cast<size_t>(stages) * tc_stage_bytes(N, a_lo, b_lo, fp8, mt) + 8 * (3 * stages + 2) + 16;
+  return 1024 + static_cast<size_t>(stages) * tc_stage_bytes(N, a_lo, b_lo, fp8, mt) + 8 * (3 * stages + 4) + 16;
 }
 
 namespace {
@@ -1786,7 +1802,7 @@ int tc2_stage_bytes(int N, int split, int fp8) {
   return (kBlockM * bk * 2 + (N / 2) * bk * 2) * (1 + split) + (fp8 ? kBlockM * bk : 0);
 }
 size_t tc2_smem_bytes(int N, int stages, int split, int fp8) {
-  return 1024 + static_cast<size_t>(stages) * tc2_stage_bytes(N, split, fp8) + 8 * (3 * stages + 2) + 16;
+  return 1024 + static_cast<size_t>(stages) * tc2_stage_bytes(N, split, fp8) + 8 * (3 * stages + 4) + 16;
 }
 constexpr int kSmemOptIn = 227 * 1024;
 }  // namespace
@@ -1794,7 +1810,7 @@ constexpr int kSmemOptIn = 227 * 1024;
 int tc_stages_pair(int N, int split, int fp8) {
   // FP8 stages that carry the staging too may use all of the opt-in shared
   // memory (four 56 KB stages at N = 512)
-  const int budget = fp8 == 1 ? kSmemOptIn - 1024 - 8 * (3 * 8 + 2) - 16 : kSmemBudget;
+  const int budget = fp8 == 1 ? kSmemOptIn - 1024 - 8 * (3 * 8 + 4) - 16 : kSmemBudget;
   int s = budget / tc2_stage_bytes(N, split, fp8);
   if (s > 8) s = 8;
   return s;
@@ -1824,9 +1840,15 @@ cudaError_t launch_tc_one(const CUtensorMap& tmA, const CUtensorMap& tmB, const 
   return cudaGetLastError();
 }
 
-cudaError_t launch_tc_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const TcArgs& a, int num_sms,
+cudaError_t launch_tc_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const TcArgs& args, int num_sms,
                            cudaStream_t st, const CUtensorMap* tmA2, const CUtensorMap* tmB2, const float* col_scale,
                            int col_ld) {
+  TcArgs a = args;
+  {  // tensor memory: the unit's accumulators, twice when they fit
+    const int unit = a.m_pair ? 2 * a.N : (a.n_split == 2 ? a.N / 2 : a.N);
+    const int cols = unit * tc_acc_sets(unit);
+    a.tmem_cols = cols <= 32 ? 32 : (cols <= 64 ? 64 : (cols <= 128 ? 128 : (cols <= 256 ? 256 : 512)));
+  }
   const long long units = static_cast<long long>(a.Nb) * a.m_tiles * a.n_kchunks;
   if (units <= 0) return cudaSuccess;
   if (a.N < 16 || a.N > 512 || a.N % 16 != 0 || (a.N > 256 && a.N % 256 != 0) || a.stages < 2)

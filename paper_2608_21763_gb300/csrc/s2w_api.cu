@@ -205,12 +205,16 @@ int pointer_kind(const void* p, int device) {
   return 0;
 }
 
-// Tensor engine: whether GEMMs take the two-SM form by default (kPairAuto: for N = 512, where half
-// of B per CTA lets the ring take 64-element K blocks with 128-byte swizzle;
-// measured 0.86 against 0.75 of the sustained BF16 peak for the 256-rupture
-// stage 1.  At N = 128 the M-tile pairs of one CTA were faster, and so
-// were single CTAs for FP8 A: 0.63 against 0.50, the pair's cross-CTA
-// converter handshake sitting on every stage.)
+// Tensor engine: which GEMMs take the two-SM form by default (kPairAuto).  Half
+// of B per CTA lets the ring take 64-element K blocks at N = 512 (256 ruptures:
+// 1.91 against 2.33 ms of stage 1 at 963 x 6,000) and leaves room for two
+// accumulator sets at 144 .. 256 columns, where two M tiles of one CTA fill
+// tensor memory (128 ruptures BF16: 1.10 against 1.19 ms; hi/lo split of 80:
+// 2.11 against 2.17); at 16 .. 64 ruptures it is 1 - 3 % faster.  Not for FP8 A
+// widened in shared memory (the pair's converter handshake sits on every
+// stage: 0.63 against 0.50 of the peak), and not for short K (the tensor
+// adjoint's first GEMM, K = 2 No, is its epilogue: 0.64 against 0.69 ms).
+constexpr long long kPairMinK = 512;
 constexpr int kPairAuto = 2;
 constexpr int kDefaultPair = kPairAuto;
 // Largest stage-2 split-K chunk count (the tensor partials are sized for it,
@@ -232,20 +236,30 @@ constexpr long long kSplitChunkK = 2048;
 // 1.6e-5 at +9 %, of 2,048 9.8e-6 at +21 %).
 constexpr long long kSplitAdjChunkK = 4096;
 
-// Form of one tensor GEMM; sets the ring depth and TMEM columns of `a` and
+long long round_up(long long x, long long m) { return (x + m - 1) / m * m; }
+
+// MMA columns for Bs ruptures: a multiple of 16, or for BF16 of 32 from 128
+// columns up, where the two-SM form wants it (at most 16 columns of zeros, read
+// past the operand's rows as TMA fill; below, and with the split's three MMAs
+// per K step, the columns cost what the form gains: 100 ruptures hi/lo, 208
+// columns 2.38 ms, 224 2.43).
+int b_columns(int Bs, int split) {
+  const int N = static_cast<int>(round_up(2 * Bs, !split && 2 * Bs > 128 ? 32 : 16));
+  return N > 256 ? 512 : N;
+}
+
+// Form of one tensor GEMM; sets the ring depth of `a` and
 // returns the B tensor map's box rows.  With `pair` (1, or kPairAuto and
 // the shape it covers; and N % 32 == 0, at least two M tiles): two-SM MMAs,
 // a CTA pair per M = 256 tile staging half of B each.  Otherwise two M tiles
 // per unit sharing each B tile when the accumulators fit (N <= 256), for
 // non-FP8 A and at least two M tiles.  Every CTA loads its own tiles.
-int tc_shape(TcArgs& a, int N, int m_tiles, int split, int fp8, int pair) {
-  if (pair == kPairAuto) pair = N == 512 && !split && !fp8;
+int tc_shape(TcArgs& a, int N, int m_tiles, long long K, int split, int fp8, int pair) {
+  if (pair == kPairAuto) pair = !fp8 && K >= kPairMinK && (N != 512 || !split);
   a.cta2 = (pair && N % 32 == 0 && m_tiles >= 2) ? 1 : 0;
   a.m_pair = (!a.cta2 && N <= 256 && !fp8 && m_tiles >= 2) ? 1 : 0;
   const int mt = a.m_pair ? 2 : 1;
   a.stages = a.cta2 ? tc_stages_pair(N, split, fp8) : tc_stages_for(N, split, split, fp8, mt);
-  const int cols = mt * N;
-  a.tmem_cols = cols <= 32 ? 32 : (cols <= 64 ? 64 : (cols <= 128 ? 128 : (cols <= 256 ? 256 : 512)));
   const int slice = N > 256 ? 256 : N;
   return a.cta2 ? slice / 2 : slice;
 }
@@ -285,8 +299,6 @@ void set_s2_chunks(s2w_ctx* ctx, int want) {
 constexpr int kStreamGroup = 64;
 
 bool supported_nt(int Nt) { return Nt == 32 || Nt == 64 || Nt == 128 || Nt == 256 || Nt == 512; }
-
-long long round_up(long long x, long long m) { return (x + m - 1) / m * m; }
 
 cudaEvent_t take_event(s2w_ctx* c) {
   if (!c->ev_free.empty()) {
@@ -433,7 +445,7 @@ int tc_gemm_epi0(s2w_ctx* ctx, const void* A, const void* A_lo, long long M, lon
   CUtensorMap ta, tb, ta2, tb2;
   const int mt = static_cast<int>((M + 127) / 128);
   TcArgs a{};
-  const int brows = tc_shape(a, N, mt, sp, 0, ctx->tc_pair);
+  const int brows = tc_shape(a, N, mt, K, sp, 0, ctx->tc_pair);
   const int bk = tc_block_k(N, sp, a.cta2);
   CK(tc_encode_3d(&ta, A, K, M, ctx->Nb, K, 128, bk));
   CK(tc_encode_3d(&tb, Bop, K, n_alloc, ctx->Nb, K, brows, bk));
@@ -482,8 +494,7 @@ int adjoint_tensor(s2w_ctx* ctx, const float* r_d, int B, float* g_d, cudaStream
   const int dt_t = ctx->opts.dt_mode == S2W_DT_NONE ? S2W_DT_NONE : kDtTranspose;
   for (int b0 = 0; b0 < B; b0 += ctx->tc_bsub) {
     const int Bs = std::min(ctx->tc_bsub, B - b0);
-    int N1 = static_cast<int>(round_up(2 * Bs, 16));
-    if (N1 > 256) N1 = 512;
+    const int N1 = b_columns(Bs, sp);
     {
       StageTimer t(ctx, 6, st);
       CK(launch_rfft_pack(r_d + static_cast<long long>(b0) * No * Nt, Bs * No, static_cast<int>(Nt), ctx->tw, No,
@@ -560,7 +571,7 @@ int waveforms_tensor(s2w_ctx* ctx, const float* slip_d, int B, float* q_d, cudaS
     const bool f8 = ctx->opts.prec_g == S2W_PREC_FP8_E4M3;
     // FP8 x FP8 stage 1 (two-SM tiles: N % 32, at least two M tiles)
     const bool f8f8 = f8 && ctx->tc_f8act && m1 >= 2;
-    int N1 = static_cast<int>(round_up(2 * Bs, f8f8 ? 32 : 16));
+    int N1 = f8 ? static_cast<int>(round_up(2 * Bs, f8f8 ? 32 : 16)) : b_columns(Bs, sp);
     if (N1 > 256) N1 = 512;
     const int* lens = ctx->cur_lens ? ctx->cur_lens + b0 : nullptr;
     if (!f8) {  // BF16 operand, written by the transform itself (padding columns stay zero)
@@ -608,7 +619,6 @@ int waveforms_tensor(s2w_ctx* ctx, const float* slip_d, int B, float* q_d, cudaS
       a.cta2 = 1;
       a.stages = tc_stages_pair(nsp ? N1 / 2 : N1, 0, lo ? (nsp ? 4 : 3) : 2);
       a.n_split = nsp ? 2 : 1;
-      a.tmem_cols = N1 <= 32 ? 32 : (N1 <= 64 ? 64 : (N1 <= 128 ? 128 : (N1 <= 256 ? 256 : 512)));
       a.a_fp8 = 1;
       a.row_scale = ctx->G_scale;
       a.nblk = ctx->nblk;
@@ -622,7 +632,7 @@ int waveforms_tensor(s2w_ctx* ctx, const float* slip_d, int B, float* q_d, cudaS
       StageTimer t(ctx, 1, st);
       CUtensorMap ta, tb, ta2, tb2;
       TcArgs a{};
-      const int brows = tc_shape(a, N1, m1, sp, f8 ? 1 : 0, ctx->tc_pair);
+      const int brows = tc_shape(a, N1, m1, K1, sp, f8 ? 1 : 0, ctx->tc_pair);
       const int bk = tc_block_k(N1, sp, a.cta2);
       if (f8)  // one byte per K element: row pitch 2 Ns_pad bytes
         CK(tc_encode_3d_u8(&ta, ctx->G, K1, Ng, Nb, 128, bk));
@@ -692,9 +702,9 @@ int waveforms_tensor(s2w_ctx* ctx, const float* slip_d, int B, float* q_d, cudaS
       const int m2 = (Bs + 127) / 128;
       TcArgs a{};
       // the half-stored operand runs on one CTA per tile (or M-tile pair)
-      int brows = tc_shape(a, ctx->tc_n2, m2, sp, 0, ctx->tc_p2h ? 0 : ctx->tc_pair);
+      int brows = tc_shape(a, ctx->tc_n2, m2, K2, sp, 0, ctx->tc_p2h ? 0 : ctx->tc_pair);
       // the chunk length tc_kbpc counts K blocks of the single-CTA size
-      if (tc_block_k(ctx->tc_n2, sp, a.cta2) != tc_block_k(ctx->tc_n2, sp)) brows = tc_shape(a, ctx->tc_n2, m2, sp, 0, 0);
+      if (tc_block_k(ctx->tc_n2, sp, a.cta2) != tc_block_k(ctx->tc_n2, sp)) brows = tc_shape(a, ctx->tc_n2, m2, K2, sp, 0, 0);
       const int bk = tc_block_k(ctx->tc_n2, sp, a.cta2);
       const int p2rows = ctx->tc_p2h ? ctx->tc_n2 / 2 : ctx->tc_n2;
       a.b_half = ctx->tc_p2h ? 1 : 0;

@@ -260,7 +260,7 @@ struct TcArgs {
                           //   kb_off + kc kblocks_per_chunk ...)
   int acc_out;            // epi 0, FP32 out: add into out instead of storing (K ranges in turn)
   int stages;             // shared-memory ring depth
-  int tmem_cols;          // power of two >= max(32, N)
+  int tmem_cols;          // set by launch_tc_gemm: the unit's accumulator columns, twice when they fit
   int epi;                // 0: out[l*ld_l + t*ld_t + row]; 1: out[((l*n_kchunks + kc)*M_total + row)*T + t]
   int T;                  // complex output columns (N / 2 live)
   float2* out;
