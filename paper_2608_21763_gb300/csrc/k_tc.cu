@@ -145,6 +145,23 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   for (int k = 0; k < 16; ++k) v[k] = __uint_as_float(r[k]);
 }
 
+// Same for 32 columns.
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
+  uint32_t r[32];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, "
+      "%24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr)
+      : "memory");
+#pragma unroll
+  for (int k = 0; k < 32; ++k) v[k] = __uint_as_float(r[k]);
+}
+
 // Same for 64 columns in one load (one wait per 64 accumulators).
 __device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v)[64]) {
   uint32_t r[64];
@@ -1245,26 +1262,33 @@ __global__ void k_pack_a(const float2* __restrict__ src, int Nb, int rows, long 
 // spectra split into hi + lo on the way).  T streams through a ring by TMA
 // (it stays in L2); the accumulator rows go back out as BF16 velocity
 // spectra in the stage-2 operand layout.
-// Warps: 0 TMA (T), 1 TMEM + MMA, then 4 RT_EPW epilogue warps (RT_EPW per
-// TMEM lane quadrant, each taking every RT_EPW-th 64-column chunk of an
-// accumulator unit), then the 8 fill warps.  The split kernel keeps one
-// epilogue warp per quadrant (its fill warps need the registers).
+// Warps, in warpgroups that share out the registers (setmaxnreg): 0 TMA (T),
+// 1 TMEM + MMA, 2 and 3 idle; then 4 EPW epilogue warps (EPW per TMEM lane
+// quadrant, each taking every EPW-th 32-column chunk of an accumulator); then
+// the 8 fill warps, which hold the whole next k-block of theirs in registers:
+// its loads are in flight while the MMAs still use the slot, a whole tile
+// (128 KB) per SM.  With half a k-block in flight (and none in the split
+// kernel) the fill's latency, and through it the stores that it competes
+// with, set the time: 256 ruptures x 16,000 points x 256 steps 1.95 ms with or
+// without the MMAs, 1.02 without stores.
 // ---------------------------------------------------------------------------
 constexpr int kRtFillWarps = 8;
 __host__ __device__ constexpr int rt_epw(bool split) { return split ? 1 : 2; }
-__host__ __device__ constexpr int rt_threads(bool split) { return 32 * (2 + 4 * rt_epw(split) + kRtFillWarps); }
+__host__ __device__ constexpr int rt_threads(bool split) { return 32 * (4 + 4 * rt_epw(split) + kRtFillWarps); }
+// Registers of the three parts: BF16 128 x 40 + 256 x 56 + 256 x 160 <= 640 x
+// 96; split 128 x 40 + 128 x 104 + 256 x 184 = 512 x 128
+constexpr int kRtRegsIssue = 40;
+__host__ __device__ constexpr int rt_regs_epi(bool split) { return split ? 104 : 56; }
+__host__ __device__ constexpr int rt_regs_fill(bool split) { return split ? 184 : 160; }
 
 // Schedule.  A tile's K = 2 Nt output columns are at most two 256-column MMA
-// halves.  BF16 runs the halves outer: each half is one accumulator unit of
-// 256 columns, tensor memory holds two units, and the epilogue drains one
-// unit while the MMAs fill the other (a whole 512-column tile would fill
-// tensor memory and make the next tile's MMAs wait for its drain).  The M
-// tile then stays whole in a ring of RA = 8 k-block slots (K / 64 <= 8) until
-// the second half has used it.  Split mode at Nt = 256 cannot hold its
-// doubled M tile whole: it runs the K blocks outer and both halves inner in
-// one 512-column unit, so each k-block slot is freed once both halves have
-// used it.  With a single half (Nt <= 128) both orders coincide and two
-// units of K columns fit.
+// halves, each an accumulator of its own; tensor memory holds two, so the
+// epilogue drains one while the MMAs fill the other.  The k-blocks go in
+// groups of at most RA = 8, the slots of the A ring: within a group the halves
+// are outer, and the last half frees the slots.  BF16 has one group (K / 64 <=
+// 8: the tile stays whole in the ring); the split's doubled slots hold half a
+// tile at Nt = 256, so it takes two groups, and the first half's accumulator
+// is complete, and drained, while the second half's last group runs.
 // SPLIT: the FP32 seafloor spectra are split by the fill warps into hi + lo
 // BF16 parts, T comes as hi + lo (both from the FP64 matrix), three MMAs per
 // K step (hi hi, hi lo, lo hi), and the epilogue writes hi + lo velocity
@@ -1285,7 +1309,8 @@ __global__ void __launch_bounds__(rt_threads(SPLIT), 1)
   static_assert(!(SPLIT && PAIR), "two-SM retransform: BF16 only");
   constexpr int BK = SPLIT ? 32 : 64;        // K elements per k-block
   constexpr int EPW = rt_epw(SPLIT);
-  constexpr int kFill0 = 2 + 4 * EPW;        // first fill warp
+  constexpr int kEpi0 = 4;                   // first epilogue warp
+  constexpr int kFill0 = kEpi0 + 4 * EPW;    // first fill warp
   constexpr int kAs = kBlockM * BK * 2;      // one BF16 part of an M-tile k-block
   constexpr int a_slot = kAs * (SPLIT ? 2 : 1);
   constexpr int kBins = BK / 2;              // complex bins per k-block
@@ -1296,11 +1321,9 @@ __global__ void __launch_bounds__(rt_threads(SPLIT), 1)
   const int KB = K / BK;          // k-blocks per tile
   const int n_half = K > 256 ? 2 : 1;   // MMA column halves (256 output columns each)
   const int ncols = K > 256 ? 256 : K;
-  const bool hout = !SPLIT || n_half == 1;  // halves outer (see the schedule above)
-  const int U = hout ? n_half : 1;          // accumulator units per tile
-  const int H = hout ? 1 : n_half;          // halves per unit
-  const int ucols = H * ncols;              // accumulator columns per unit
-  const int AS = 2 * ucols <= 512 ? 2 : 1;  // accumulator units in tensor memory
+  const int U = n_half;           // accumulators (halves) per tile
+  const int KG = KB < kRtFillWarps ? KB : kRtFillWarps;  // k-blocks per group
+  const int AS = 2;               // accumulators in tensor memory
   const int trows = PAIR ? ncols / 2 : ncols;  // T rows this CTA stages per half
   const int t_part = trows * BK * 2;
   const int t_slot = t_part * (SPLIT ? 2 : 1);
@@ -1334,7 +1357,7 @@ __global__ void __launch_bounds__(rt_threads(SPLIT), 1)
     i0 = (static_cast<int>(u % mgroups) * (PAIR ? 2 : 1) + static_cast<int>(crank)) * kBlockM;
   };
   const uint32_t idesc = idesc_bf16(PAIR ? 2 * kBlockM : kBlockM, ncols);
-  const int acols = AS * ucols;
+  const int acols = AS * ncols;
   const uint32_t tmem_cols = acols <= 64 ? 64 : (acols <= 128 ? 128 : (acols <= 256 ? 256 : 512));
 
   if (threadIdx.x == 0) {
@@ -1367,18 +1390,19 @@ __global__ void __launch_bounds__(rt_threads(SPLIT), 1)
   tc_fence_after();
   const uint32_t tmem = *tmem_holder;
 
+  if (warp < kEpi0) {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRtRegsIssue));
   if (warp == 0) {
-    // T slots in job order: tile, unit, k-block, half within the unit
+    // T slots in job order: tile, group of k-blocks, half, k-block
     if (lane == 0) {
       int it = 0;
       RingPos rp;
       bool ok = true;
       const uint32_t tfull0 = PAIR ? cluster_addr(tfull, 0) : 0u;
       for (long long t = cid; t < tiles && ok; t += ncl) {
-        for (int u = 0; u < U && ok; ++u) {
-          for (int kb = 0; kb < KB && ok; ++kb) {
-            for (int hh = 0; hh < H; ++hh, ++it, rp.next(RT)) {
-              const int h = hout ? u : hh;
+        for (int k0 = 0; k0 < KB && ok; k0 += KG) {
+          for (int h = 0; h < U && ok; ++h) {
+            for (int kb = k0; kb < k0 + KG; ++kb, ++it, rp.next(RT)) {
               const int s = rp.s;
               if (it >= RT && !mbar_wait_bounded(tempty + s, rp.ph ^ 1u, a.status, DEV_ERR_TIMEOUT_EMPTY)) {
                 ok = false;
@@ -1416,38 +1440,32 @@ __global__ void __launch_bounds__(rt_threads(SPLIT), 1)
         else
           tc_commit(bar);
       };
-      int tl = 0, un = 0;  // tile and accumulator unit counters
-      RingPos rp;          // T slot
+      int tl = 0;  // tiles done
+      RingPos rp;  // T slot
       constexpr uint32_t hi = sdesc_hi<BK>();
       const uint32_t a0 = sdesc_lo(smem_u32(sA)), b0 = sdesc_lo(smem_u32(sT));
       const uint32_t t_slot16 = static_cast<uint32_t>(t_slot) >> 4, t_part16 = static_cast<uint32_t>(t_part) >> 4;
       bool ok = true;
       for (long long t = cid; t < tiles && ok; t += ncl, ++tl) {
-        for (int u = 0; u < U && ok; ++u, ++un) {
-          const int as = un % AS;
-          if (un >= AS && !wait_x(acc_empty + as, ((un / AS) - 1) & 1, DEV_ERR_TIMEOUT_MMA)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t dcol = tmem + static_cast<uint32_t>(as * ucols);
-          for (int kb = 0; kb < KB && ok; ++kb) {
-            const long long n = static_cast<long long>(tl) * KB + kb;
-            const int sa = static_cast<int>(n % RA);
-            if (u == 0 && !wait_x(afull + sa, static_cast<int>((n / RA) & 1), DEV_ERR_TIMEOUT_FULL)) {
+        for (int k0 = 0; k0 < KB && ok; k0 += KG) {
+          for (int u = 0; u < U && ok; ++u) {
+            const int un = tl * U + u, as = un % AS;
+            if (k0 == 0 && un >= AS && !wait_x(acc_empty + as, ((un / AS) - 1) & 1, DEV_ERR_TIMEOUT_MMA)) {
               ok = false;
               break;
             }
-            for (int hh = 0; hh < H; ++hh, rp.next(RT)) {
-              const int s = rp.s;
-              if (!mbar_wait_bounded(tfull + s, rp.ph, a.status, DEV_ERR_TIMEOUT_FULL)) {
+            tc_fence_after();
+            const uint32_t d = tmem + static_cast<uint32_t>(as * ncols);
+            for (int kb = k0; kb < k0 + KG; ++kb, rp.next(RT)) {
+              const int n = tl * KB + kb, sa = n % RA, s = rp.s;
+              if ((u == 0 && !wait_x(afull + sa, static_cast<uint32_t>(n / RA) & 1u, DEV_ERR_TIMEOUT_FULL)) ||
+                  !mbar_wait_bounded(tfull + s, rp.ph, a.status, DEV_ERR_TIMEOUT_FULL)) {
                 ok = false;
                 break;
               }
               tc_fence_after();
               const uint32_t al = a0 + static_cast<uint32_t>(sa) * (a_slot >> 4);
               const uint32_t bl = b0 + static_cast<uint32_t>(s) * t_slot16;
-              const uint32_t d = dcol + static_cast<uint32_t>(hh * ncols);
 #pragma unroll
               for (int k = 0; k < BK / 16; ++k) {
                 const uint32_t ad = al + ((k * 32) >> 4), bd = bl + ((k * 32) >> 4);
@@ -1462,21 +1480,22 @@ __global__ void __launch_bounds__(rt_threads(SPLIT), 1)
                 }
               }
               commit(tempty + s);
+              if (u == U - 1) commit(afree + sa);  // the last half has used this k-block
             }
-            if (!ok) break;
-            if (u == U - 1) commit(afree + sa);  // the last unit has used this k-block
+            if (ok && k0 + KG >= KB) commit(acc_full + as);
           }
-          if (!ok) break;
-          commit(acc_full + as);
         }
       }
+      const int un = tl * U;  // accumulators (started, if a wait gave up)
       // the epilogue's releases of the last units (from both CTAs) have landed
       for (int k = (un > AS ? un - AS : 0); k < un; ++k) wait_x(acc_empty + k % AS, (k / AS) & 1, DEV_ERR_TIMEOUT_MMA);
     }
+  }
   } else if (warp < kFill0) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(rt_regs_epi(SPLIT)));
     // epilogue: accumulator row = signal, columns = output degrees of freedom
     const int q = warp & 3;
-    const int g = (warp - 2) >> 2;  // column group of the quadrant
+    const int g = (warp - kEpi0) >> 2;  // column group of the quadrant
     const uint32_t acc_empty0 = PAIR ? cluster_addr(acc_empty, 0) : 0u;
     int un = 0;
     bool ok = true;
@@ -1502,23 +1521,28 @@ __global__ void __launch_bounds__(rt_threads(SPLIT), 1)
           break;
         }
         tc_fence_after();
-        const uint32_t tbase = tmem + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(as * ucols);
-        const int cb = hout ? u * ncols : 0;  // first output column of the unit
+        const uint32_t tbase = tmem + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(as * ncols);
         // K = 2 Nt is a multiple of 64 for every supported Nt (32..256)
-        for (int c0 = 64 * g; c0 < ucols; c0 += 64 * EPW) {
-          float v[64];
-          tmem_ld64(tbase + c0, v);
+        constexpr int CW = SPLIT ? 32 : 16;  // columns per load
+        for (int c0 = CW * g; c0 < ncols; c0 += CW * EPW) {
+          float v[CW];
+          if constexpr (SPLIT)
+            tmem_ld32(tbase + c0, v);
+          else
+            tmem_ld16(tbase + c0, v);
           if (i >= a.Ng) continue;
-          const int oc = cb + c0;
+          const int l0 = (u * ncols + c0) / 2;  // first bin of the chunk
+          long long off = static_cast<long long>(l0) * a.vld_l;
+          if (l0 == 0) {  // K slots 0 and 1: Re bins 0 and Nt
+            put(0, v[0], 0.f);
+            put(static_cast<long long>(Nt) * a.vld_l, v[1], 0.f);
+          } else {
+            put(off, v[0], v[1]);
+          }
 #pragma unroll
-          for (int k = 0; k < 32; ++k) {
-            const int l = oc / 2 + k;
-            if (l == 0) {
-              put(0, v[0], 0.f);
-              put(static_cast<long long>(Nt) * a.vld_l, v[1], 0.f);
-            } else {
-              put(static_cast<long long>(l) * a.vld_l, v[2 * k], v[2 * k + 1]);
-            }
+          for (int k = 1; k < CW / 2; ++k) {
+            off += a.vld_l;
+            put(off, v[2 * k], v[2 * k + 1]);
           }
         }
         tc_fence_before();
@@ -1531,151 +1555,94 @@ __global__ void __launch_bounds__(rt_threads(SPLIT), 1)
         }
       }
     }
-  } else if constexpr (!SPLIT) {
-    // fill warps (BF16): warp f fills k-blocks f, f + 8, ... of every tile
-    // (k-block kb holds bins 32 kb .. 32 kb + 31 for 128 signals; K slot 1
-    // of bin 0 carries Re(bin Nt)), two batches of 16 bins each with 64
-    // loads in flight per lane.  The first batch is loaded before the wait
-    // for the slot, so its HBM latency overlaps the MMAs that still read the
-    // slot; 16-byte chunks are stored in the TMA 128-byte swizzle pattern
-    // (chunk ^ (row & 7)).
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(rt_regs_fill(SPLIT)));
+    // fill warps: warp f fills k-blocks f, f + 8, ... of every tile (k-block kb
+    // holds bins kBins kb .. for 128 signals; K slot 1 of bin 0 carries Re(bin
+    // Nt)).  A k-block is loaded whole into registers as soon as the warp's
+    // one before is stored, so its HBM latency overlaps the MMAs that still
+    // read the slot; 16-byte chunks are stored in the TMA swizzle pattern
+    // (BF16: chunk ^ (row & 7) of 128-byte rows; split: chunk ^ ((row >> 1) &
+    // 3) of 64-byte rows, hi and lo parts).
+    using Raw = std::conditional_t<SPLIT, float2, unsigned>;
     const int f = warp - kFill0;
     const uint32_t afull0 = PAIR ? cluster_addr(afull, 0) : 0u;
-    int tl = 0;
-    bool ok = true;
-    for (long long t = cid; t < tiles && ok; t += ncl, ++tl) {
+    Raw raw[kBins][4];
+    Raw rawn[4];  // bin Nt (warp 0, k-block 0)
+    auto load = [&](long long t, int kb) {
       int b, i0;
       unit_tile(t, b, i0);
-      const unsigned* mbb = reinterpret_cast<const unsigned*>(a.mhat_bf) + static_cast<long long>(b) * a.ld_b;
-      for (int kb = f; kb < KB && ok; kb += kRtFillWarps) {
-        const long long n = static_cast<long long>(tl) * KB + kb;
-        const int sa = static_cast<int>(n % RA);
-        unsigned raw[16][4];
-        auto load = [&](int hh) {
+      const Raw* m;
+      if constexpr (SPLIT)
+        m = a.mhat32 + static_cast<long long>(b) * a.ld_b + i0 + lane;
+      else
+        m = reinterpret_cast<const unsigned*>(a.mhat_bf) + static_cast<long long>(b) * a.ld_b + i0 + lane;
+      const int left = a.Ng - i0 - lane;  // signals 32 g < left of this lane are live
+      const Raw* p = m + static_cast<long long>(kb * kBins) * a.ld_l;
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const long long lo = static_cast<long long>(kb * kBins + 16 * hh + j) * a.ld_l;
+      for (int j = 0; j < kBins; ++j, p += a.ld_l) {
 #pragma unroll
-            for (int g = 0; g < 4; ++g) {
-              const int i = i0 + 32 * g + lane;
-              raw[j][g] = i < a.Ng ? __ldg(mbb + lo + i) : 0u;
-            }
-          }
-        };
-        unsigned char* slot = sA + sa * a_slot;
-        auto store = [&](int hh) {
+        for (int g = 0; g < 4; ++g) raw[j][g] = 32 * g < left ? __ldg(p + 32 * g) : Raw{};
+      }
+      if (kb == 0) {
+        p = m + static_cast<long long>(Nt) * a.ld_l;
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
+        for (int g = 0; g < 4; ++g) rawn[g] = 32 * g < left ? __ldg(p + 32 * g) : Raw{};
+      }
+    };
+    long long t = cid;
+    int kb = f;
+    if (f < KB && t < tiles) load(t, kb);
+    for (int tl = 0; f < KB && t < tiles;) {
+      const int n = tl * KB + kb, sa = n % RA;
+      if (n >= RA && !mbar_wait_bounded(afree + sa, (static_cast<uint32_t>(n / RA) - 1u) & 1u, a.status,
+                                        DEV_ERR_TIMEOUT_EMPTY))
+        break;
+      unsigned char* slot = sA + sa * a_slot;
+      if (kb == 0) {
 #pragma unroll
-            for (int g = 0; g < 4; ++g) {
-              const int row = 32 * g + lane;
-              *reinterpret_cast<uint4*>(slot + row * 128 + (((4 * hh + c) ^ (row & 7)) << 4)) =
-                  make_uint4(raw[4 * c][g], raw[4 * c + 1][g], raw[4 * c + 2][g], raw[4 * c + 3][g]);
-            }
-          }
-        };
-        load(0);
-        if (kb == 0) {
-#pragma unroll
-          for (int g = 0; g < 4; ++g) {
-            const int i = i0 + 32 * g + lane;
-            const unsigned rn = i < a.Ng ? __ldg(mbb + static_cast<long long>(Nt) * a.ld_l + i) : 0u;
-            raw[0][g] = (raw[0][g] & 0xffffu) | (rn << 16);  // K slot 1: Re(bin Nt)
-          }
-        }
-        if (n >= RA &&
-            !mbar_wait_bounded(afree + sa, static_cast<int>(((n / RA) - 1) & 1), a.status, DEV_ERR_TIMEOUT_EMPTY)) {
-          ok = false;
-          break;
-        }
-        store(0);
-#pragma unroll
-        for (int hh = 1; hh < kBins / 16; ++hh) {
-          load(hh);
-          store(hh);
-        }
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) {
-          if constexpr (PAIR)
-            mbar_arrive_cluster(afull0 + 8u * static_cast<uint32_t>(sa));
+        for (int g = 0; g < 4; ++g) {  // K slot 1: Re(bin Nt)
+          if constexpr (SPLIT)
+            raw[0][g].y = rawn[g].x;
           else
-            mbar_arrive(afull + sa);
+            raw[0][g] = (raw[0][g] & 0xffffu) | (rawn[g] << 16);
         }
       }
-    }
-  } else {
-    // fill warps (split): warp f fills k-blocks f, f + 8, ... of every tile
-    // (k-block kb holds bins kBins kb .. kBins kb + kBins - 1 for 128 signals;
-    // K slot 1 of bin 0 carries Re(bin Nt)); all of a tile's loads are in
-    // flight together; 16-byte chunks are stored in the TMA swizzle pattern
-    const int f = warp - kFill0;
-    int tl = 0;
-    bool ok = true;
-    for (long long t = cid; t < tiles && ok; t += ncl, ++tl) {
-      int b, i0;
-      unit_tile(t, b, i0);
-      for (int kb = f; kb < KB && ok; kb += kRtFillWarps) {
-        const long long n = static_cast<long long>(tl) * KB + kb;
-        const int sa = static_cast<int>(n % RA);
-        if (n >= RA &&
-            !mbar_wait_bounded(afree + sa, static_cast<int>(((n / RA) - 1) & 1), a.status, DEV_ERR_TIMEOUT_EMPTY)) {
-          ok = false;
-          break;
-        }
-        unsigned char* slot = sA + sa * a_slot;
-        auto chunk_off = [&](int row, int chunk) {  // 16-byte chunk `chunk` of K-major row `row` (64-byte swizzle)
-          return row * 64 + ((chunk ^ ((row >> 1) & 3)) << 4);
-        };
-        const float2* mb = a.mhat32 + static_cast<long long>(b) * a.ld_b;
-        float rawn[4] = {0.f, 0.f, 0.f, 0.f};
-        if (kb == 0) {
 #pragma unroll
-          for (int g = 0; g < 4; ++g) {
-            const int i = i0 + 32 * g + lane;
-            rawn[g] = i < a.Ng ? __ldg(mb + static_cast<long long>(Nt) * a.ld_l + i).x : 0.f;
-          }
-        }
+      for (int c = 0; c < kBins / 4; ++c) {
 #pragma unroll
-        for (int hh = 0; hh < kBins / 8; ++hh) {  // 8 bins per batch, 32 float2 loads in flight
-          float2 raw[8][4];
+        for (int g = 0; g < 4; ++g) {
+          const int row = 32 * g + lane;
+          if constexpr (SPLIT) {
+            unsigned hw[4], lw[4];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const long long lo = static_cast<long long>(kb * kBins + 8 * hh + j) * a.ld_l;
-#pragma unroll
-            for (int g = 0; g < 4; ++g) {
-              const int i = i0 + 32 * g + lane;
-              raw[j][g] = i < a.Ng ? __ldg(mb + lo + i) : make_float2(0.f, 0.f);
+            for (int e = 0; e < 4; ++e) {
+              const float2 x = raw[4 * c + e][g];
+              const __nv_bfloat162 h2 = __floats2bfloat162_rn(x.x, x.y);
+              const __nv_bfloat162 l2 = __floats2bfloat162_rn(x.x - __low2float(h2), x.y - __high2float(h2));
+              hw[e] = *reinterpret_cast<const unsigned*>(&h2);
+              lw[e] = *reinterpret_cast<const unsigned*>(&l2);
             }
-          }
-          if (kb == 0 && hh == 0) {
-#pragma unroll
-            for (int g = 0; g < 4; ++g) raw[0][g].y = rawn[g];  // K slot 1: Re(bin Nt)
-          }
-#pragma unroll
-          for (int c = 0; c < 2; ++c) {  // chunk 2 hh + c = bins 8 hh + 4 c .. + 3
-#pragma unroll
-            for (int g = 0; g < 4; ++g) {
-              const int row = 32 * g + lane;
-              unsigned hw[4], lw[4];
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const float2 x = raw[4 * c + e][g];
-                const __nv_bfloat162 h2 = __floats2bfloat162_rn(x.x, x.y);
-                const __nv_bfloat162 l2 = __floats2bfloat162_rn(x.x - __low2float(h2), x.y - __high2float(h2));
-                hw[e] = *reinterpret_cast<const unsigned*>(&h2);
-                lw[e] = *reinterpret_cast<const unsigned*>(&l2);
-              }
-              const int off = chunk_off(row, 2 * hh + c);
-              *reinterpret_cast<uint4*>(slot + off) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-              *reinterpret_cast<uint4*>(slot + kAs + off) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
-            }
+            const int off = row * 64 + ((c ^ ((row >> 1) & 3)) << 4);
+            *reinterpret_cast<uint4*>(slot + off) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+            *reinterpret_cast<uint4*>(slot + kAs + off) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+          } else {
+            *reinterpret_cast<uint4*>(slot + row * 128 + ((c ^ (row & 7)) << 4)) =
+                make_uint4(raw[4 * c][g], raw[4 * c + 1][g], raw[4 * c + 2][g], raw[4 * c + 3][g]);
           }
         }
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(afull + sa);
       }
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) {
+        if constexpr (PAIR)
+          mbar_arrive_cluster(afull0 + 8u * static_cast<uint32_t>(sa));
+        else
+          mbar_arrive(afull + sa);
+      }
+      kb += kRtFillWarps;
+      if (kb >= KB) kb = f, t += ncl, ++tl;
+      if (t < tiles) load(t, kb);
     }
   }
   tc_fence_before();
