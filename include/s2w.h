@@ -139,8 +139,9 @@ typedef struct {
                       two-SM MMAs: a pair of CTAs computes one 256-row tile
                       with each CTA staging half of the B tile.  S2W_PAIR_OFF
                       keeps one CTA per 128-row tile; S2W_PAIR_AUTO (0,
-                      default) takes the two-SM form for stage 1 and the
-                      adjoint's long GEMM wherever the shape allows.
+                      default) takes the two-SM form for stage 1, the
+                      adjoint's long GEMM and the BF16 retransform where it
+                      is the faster one.
                       The BF16 stage-2 GEMM, whose adjoint operand is stored
                       once (the embedding's second rows are built in shared
                       memory), runs on one CTA per tile in every mode; the

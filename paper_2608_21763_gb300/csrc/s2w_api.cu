@@ -210,12 +210,18 @@ int pointer_kind(const void* p, int device) {
 // 1.91 against 2.33 ms of stage 1 at 963 x 6,000) and leaves room for two
 // accumulator sets at 144 .. 256 columns, where two M tiles of one CTA fill
 // tensor memory (128 ruptures BF16: 1.10 against 1.19 ms; hi/lo split of 80:
-// 2.11 against 2.17); at 16 .. 64 ruptures it is 1 - 3 % faster.  Not for FP8 A
+// 2.11 against 2.17); at 16 .. 64 ruptures it is 1 - 8 % faster.  Not for FP8 A
 // widened in shared memory (the pair's converter handshake sits on every
-// stage: 0.63 against 0.50 of the peak), and not for short K (the tensor
-// adjoint's first GEMM, K = 2 No, is its epilogue: 0.64 against 0.69 ms).
-constexpr long long kPairMinK = 512;
+// stage: 0.63 against 0.50 of the peak), and not for short K, where a unit is
+// mostly its epilogue (BF16, 64 ruptures, 8,000 points: K = 512 0.39 against
+// 0.43 ms, K = 800 equal, K = 1,200 0.86 against 0.82; the tensor adjoint's
+// first GEMM, K = 2 No, 0.64 against 0.69).
+constexpr long long kPairMinK = 768;
 constexpr int kPairAuto = 2;
+// The BF16 retransform on two-SM tiles: when asked for, and by default where its
+// output takes two 256-column halves (37,758 points x 256 ruptures x 256 steps
+// 4.06 -> 3.81 ms; 30,000 x 256 x 128, one half, 1.61 against 1.63).
+bool rt_pair(int pub, int Nt) { return pub == S2W_PAIR_ON || (pub == S2W_PAIR_AUTO && Nt == 256); }
 constexpr int kDefaultPair = kPairAuto;
 // Largest stage-2 split-K chunk count (the tensor partials are sized for it,
 // so s2w_autotune and opts.tc_s2_chunks can pick any count up to it).
@@ -255,7 +261,7 @@ int b_columns(int Bs, int split) {
 // per unit sharing each B tile when the accumulators fit (N <= 256), for
 // non-FP8 A and at least two M tiles.  Every CTA loads its own tiles.
 int tc_shape(TcArgs& a, int N, int m_tiles, long long K, int split, int fp8, int pair) {
-  if (pair == kPairAuto) pair = !fp8 && K >= kPairMinK && (N != 512 || !split);
+  if (pair == kPairAuto) pair = !fp8 && (K >= kPairMinK || N == 512);
   a.cta2 = (pair && N % 32 == 0 && m_tiles >= 2) ? 1 : 0;
   a.m_pair = (!a.cta2 && N <= 256 && !fp8 && m_tiles >= 2) ? 1 : 0;
   const int mt = a.m_pair ? 2 : 1;
@@ -953,9 +959,7 @@ int s2w_create(int Ns, int Ng, int No, int Nt, const s2w_opts* opts, s2w_ctx** o
     ctx->tc_bsub = static_cast<int>(std::min<long long>(B, bsub_want));
     ctx->tc_bsub_max = ctx->tc_bsub;
     ctx->tc_pair = o.tc_pair == S2W_PAIR_ON ? 1 : (o.tc_pair == S2W_PAIR_OFF ? 0 : kDefaultPair);
-    // the two-SM retransform measured slower (9.0 against 8.4 ms per 256-rupture
-    // batch): only when asked for
-    ctx->tc_rtpair = o.tc_pair == S2W_PAIR_ON;
+    ctx->tc_rtpair = rt_pair(o.tc_pair, Nt);
     ctx->tc_f8act = o.tc_fp8_act != 0;
     ctx->tc_f8lo = o.tc_fp8_act == 2;
     // FP8 B rows come in multiples of 32 (N % 32 for the two-SM tiles)
@@ -1851,11 +1855,11 @@ bool tune_cache_write(const std::string& path, const std::string& key, int bsub,
 // GEMM-form knob of the tensor engine: the public S2W_PAIR_* value and the
 // internal tc_pair code it selects.
 int pair_code(int pub) { return pub == S2W_PAIR_ON ? 1 : (pub == S2W_PAIR_OFF ? 0 : kDefaultPair); }
-// The GEMM form of a public pair value: S2W_PAIR_ON also runs the BF16
-// retransform GEMM on two-SM tiles, as when the caller sets it.
+// The GEMM form of a public pair value, the BF16 retransform's included, as
+// when the caller sets it.
 void apply_pair_mode(s2w_ctx* ctx, int pub) {
   ctx->tc_pair = pair_code(pub);
-  ctx->tc_rtpair = pub == S2W_PAIR_ON;
+  ctx->tc_rtpair = rt_pair(pub, ctx->Nt);
 }
 
 }  // namespace
