@@ -213,6 +213,15 @@ __host__ __device__ constexpr uint32_t sdesc_hi() {
 // Accumulator sets of `cols` columns that tensor memory (512) holds, at most two.
 __host__ __device__ constexpr int tc_acc_sets(int cols) { return 2 * cols <= 512 ? 2 : 1; }
 
+// Rows of A that a stage of the half-stored-B GEMM keeps when the ruptures are
+// fewer than a tile's 128: the MMAs read on past them, into whatever follows
+// in shared memory (the launch adds the missing rows past the ring), and those
+// accumulator rows are not stored.  A stage of 8 ruptures and 64 observations
+// is 17 KB instead of 32, so the ring keeps 12 instead of 6 in flight, of
+// which only the 8 KB of adjoint spectra come from HBM.
+__host__ __device__ constexpr int tc_half_rows(int M) { return M >= kBlockM ? kBlockM : (M + 7) / 8 * 8; }
+constexpr int kHalfStages = 24;  // most ring stages of that GEMM
+
 // Position in a ring of S slots: slot, and the parity of its current lap.
 struct RingPos {
   int s = 0;
@@ -399,12 +408,14 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* tmA, const CUten
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
   const int N = a.N;
   const int b_bytes = N * BK * 2;
-  constexpr int a_all = a_tile * MT;                   // A (+ A_lo) bytes per stage, all M tiles
+  // A (+ A_lo) bytes per stage, all M tiles; a half-stored B with fewer than
+  // 128 rows of A keeps only the live rows (tc_half_rows)
+  const int a_all = BH && MT == 1 ? tc_half_rows(a.M_total) * BK * 2 : a_tile * MT;
   const int stage_bytes = a_all + b_bytes * (SPLIT ? 2 : 1) + kStg;
   const int S = a.stages;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + S * stage_bytes);
   uint64_t* empty = full + S;
-  uint64_t* aready = empty + S;  // F8 / BH: the stage completed (count 4 converter warps)
+  uint64_t* aready = empty + S;  // F8: the stage completed by the 4 converter warps; BH: by its one
   uint64_t* acc_full = aready + (CONV ? S : 0);
   uint64_t* acc_empty = acc_full + 2;
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(acc_empty + 2);
@@ -426,7 +437,7 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* tmA, const CUten
     for (int s = 0; s < S; ++s) {
       mbar_init(full + s, 1);
       mbar_init(empty + s, 1);
-      if (CONV) mbar_init(aready + s, 4);
+      if (CONV) mbar_init(aready + s, BH ? 1 : 4);
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(acc_full + s, 1);
@@ -525,7 +536,7 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* tmA, const CUten
           }
           tc_fence_after();
           const uint32_t al = a0 + static_cast<uint32_t>(s) * stage16;
-          const uint32_t bl = al + (a_all >> 4);
+          const uint32_t bl = al + (static_cast<uint32_t>(a_all) >> 4);
           const uint32_t first = kb > kb0 ? 1u : 0u;  // 0: the unit's first MMA overwrites the accumulator
           auto kblock = [&](auto nm_tag) {
             constexpr int NM = decltype(nm_tag)::value;  // 256-column MMAs per K step
@@ -565,8 +576,13 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* tmA, const CUten
     // converter warps.  F8: thread t widens row t of each FP8 A tile.  BH:
     // the B tile's second half, row by row from the first (rows N / 2 + r
     // and r share the 128-byte swizzle phase, N / 2 being a multiple of 8,
-    // so the bytes copy straight across), 16 bytes per thread and step
+    // so the bytes copy straight across), 16 bytes per lane and step.  Each
+    // warp owns every fourth ring slot whole (a slot, not a turn: its full
+    // barrier's phases are then seen in order): the four work on four stages
+    // at once, where a quarter of each in turn paid the wait, the
+    // shared-memory latency and the fence once per stage and warp
     const int t = threadIdx.x - 32 * kConvWarp0;
+    const int cw = t >> 5;
     RingPos rp;
     bool ok = true;
     for (long long u = cid; u < units && ok; u += ncl) {
@@ -576,6 +592,7 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* tmA, const CUten
       const int kb1 = min(nk_total, kb0 + a.kblocks_per_chunk);
       for (int kb = kb0; kb < kb1; ++kb, rp.next(S)) {
         const int s = rp.s;
+        if (BH && (s & 3) != cw) continue;
         if (!mbar_wait_bounded(full + s, rp.ph, a.status, DEV_ERR_TIMEOUT_FULL)) {
           ok = false;
           break;
@@ -586,9 +603,14 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* tmA, const CUten
         } else {
           const uint4* src = reinterpret_cast<const uint4*>(sa + a_all);
           uint4* dst = reinterpret_cast<uint4*>(sa + a_all + b_bytes / 2);
-          for (int i = t; i < b_bytes / 32; i += 128) {
-            const uint4 w = src[i];
-            dst[i] = make_uint4(rot_pair_bf16(w.x), rot_pair_bf16(w.y), rot_pair_bf16(w.z), rot_pair_bf16(w.w));
+          for (int i = lane; i < b_bytes / 32; i += 128) {  // N % 32 == 0: 4 N words, whole batches
+            uint4 w[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) w[k] = src[i + 32 * k];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              dst[i + 32 * k] = make_uint4(rot_pair_bf16(w[k].x), rot_pair_bf16(w[k].y), rot_pair_bf16(w[k].z),
+                                           rot_pair_bf16(w[k].w));
           }
         }
         fence_proxy_async_smem();
@@ -1830,7 +1852,14 @@ cudaError_t launch_tc_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const
         tc_block_k(a.N, 0) != 64)
       return cudaErrorInvalidValue;
     const int mt = a.m_pair ? 2 : 1;
-    const size_t smem = tc_smem_bytes(a.N, a.stages, 0, 0, 0, mt);
+    size_t smem = tc_smem_bytes(a.N, a.stages, 0, 0, 0, mt);
+    if (mt == 1) {
+      const int rows = tc_half_rows(a.M_total);
+      const int stage = (rows + a.N) * 128, pad = (kBlockM - rows) * 128;
+      const int s = (kSmemOptIn - 1024 - 8 * (3 * kHalfStages + 4) - 16 - pad) / stage;
+      a.stages = s < kHalfStages ? s : kHalfStages;
+      smem = 1024 + static_cast<size_t>(a.stages) * stage + 8 * (3 * a.stages + 4) + 16 + pad;
+    }
     if (smem > 227 * 1024) return cudaErrorInvalidValue;
     const long long pu = static_cast<long long>(a.Nb) * ((a.m_tiles + mt - 1) / mt) * a.n_kchunks;
     const unsigned grid = static_cast<unsigned>(pu < num_sms ? pu : num_sms);

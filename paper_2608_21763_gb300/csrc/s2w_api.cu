@@ -714,7 +714,8 @@ int waveforms_tensor(s2w_ctx* ctx, const float* slip_d, int B, float* q_d, cudaS
       const int bk = tc_block_k(ctx->tc_n2, sp, a.cta2);
       const int p2rows = ctx->tc_p2h ? ctx->tc_n2 / 2 : ctx->tc_n2;
       a.b_half = ctx->tc_p2h ? 1 : 0;
-      CK(tc_encode_3d(&ta, ctx->tc_vhat, K2, ctx->tc_bsub, Nb, K2, 128, bk));
+      const int arows = ctx->tc_p2h && !a.m_pair && Bs < 128 ? static_cast<int>(round_up(Bs, 8)) : 128;
+      CK(tc_encode_3d(&ta, ctx->tc_vhat, K2, ctx->tc_bsub, Nb, K2, arows, bk));
       CK(tc_encode_3d(&tb, ctx->tc_p2, K2, p2rows, Nb, K2, ctx->tc_p2h ? p2rows : brows, bk));
       if (sp) {
         CK(tc_encode_3d(&ta2, ctx->tc_vhat_lo, K2, ctx->tc_bsub, Nb, K2, 128, bk));
