@@ -60,6 +60,7 @@ __global__ void __launch_bounds__(kDfThreads) k_df_rfft_rows(const float* __rest
                                                              const float4* __restrict__ tw, float2* X, float2* X_lo,
                                                              long long ld_l, long long rows_a, long long ld_a,
                                                              const int* __restrict__ lens) {
+  grid_dependency();
   constexpr int N = 32 * P, NB = N + 1;
   extern __shared__ __align__(16) unsigned char smraw[];
   float4* tws = reinterpret_cast<float4*>(smraw);
@@ -109,6 +110,7 @@ __global__ void __launch_bounds__(kDfThreads) k_df_retransform(const float2* __r
                                                                float2* vhat, float2* vhat_lo, long long ld_v,
                                                                float* seafloor, long long mhat_ld_b,
                                                                long long vhat_ld_b) {
+  grid_dependency();
   constexpr int N = 32 * P, NB = N + 1;
   mhat += blockIdx.y * mhat_ld_b;
   mhat_lo += blockIdx.y * mhat_ld_b;
@@ -187,6 +189,7 @@ __global__ void __launch_bounds__(kDfThreads) k_df_reduce_irfft(const float2* __
                                                                 const float2* __restrict__ part_lo, int No, int nseg,
                                                                 long long s_b, long long s_l, long long s_s,
                                                                 const float4* __restrict__ tw, float* q, int n_keep) {
+  grid_dependency();
   constexpr int N = 32 * P;
   extern __shared__ __align__(16) unsigned char smraw[];
   float4* tws = reinterpret_cast<float4*>(smraw);
@@ -258,8 +261,8 @@ cudaError_t launch_df_rfft_rows(const float* x, long long rows, int n_in, int Nt
     const size_t sm = smem_df<P>(kCols, kWarps);
     const cudaError_t e = allow_smem(k_df_rfft_rows<P>, sm);
     if (e != cudaSuccess) return e;
-    k_df_rfft_rows<P><<<df_grid((rows + kCols - 1) / kCols), kDfThreads, sm, st>>>(x, rows, n_in, tw, X, X_lo, ld_l,
-                                                                                    rows_a, ld_a, lens);
+    launch_next(k_df_rfft_rows<P>, df_grid((rows + kCols - 1) / kCols), kDfThreads, sm, st, x, rows, n_in, tw, X,
+                X_lo, ld_l, rows_a, ld_a, lens);
   });
   return cudaGetLastError();
 }
@@ -277,8 +280,8 @@ cudaError_t launch_df_retransform(const float2* mhat, const float2* mhat_lo, lon
     const size_t sm = smem_df<P>(kCols, kWarps);
     const cudaError_t e = allow_smem(k_df_retransform<P>, sm);
     if (e != cudaSuccess) return e;
-    k_df_retransform<P><<<grid, kDfThreads, sm, st>>>(mhat, mhat_lo, Ng, ld_m, tw, ih, il, dt_mode, vhat, vhat_lo,
-                                                      ld_v, seafloor, mhat_ld_b, vhat_ld_b);
+    launch_next(k_df_retransform<P>, grid, kDfThreads, sm, st, mhat, mhat_lo, Ng, ld_m, tw, ih, il, dt_mode, vhat,
+                vhat_lo, ld_v, seafloor, mhat_ld_b, vhat_ld_b);
   });
   return cudaGetLastError();
 }
@@ -293,8 +296,8 @@ cudaError_t launch_df_reduce_irfft(const float2* part, const float2* part_lo, in
     const size_t sm = smem_df<P>(1, 1);
     const cudaError_t e = allow_smem(k_df_reduce_irfft<P>, sm);
     if (e != cudaSuccess) return e;
-    k_df_reduce_irfft<P><<<static_cast<unsigned>(n), kDfThreads, sm, st>>>(part, part_lo, No, nseg, s_b, s_l, s_s, tw,
-                                                                           q, n_keep);
+    launch_next(k_df_reduce_irfft<P>, static_cast<unsigned>(n), kDfThreads, sm, st, part, part_lo, No, nseg, s_b,
+                s_l, s_s, tw, q, n_keep);
   });
   return cudaGetLastError();
 }

@@ -77,6 +77,7 @@ template <int R, bool SHORT, int LPR>
 __global__ void __launch_bounds__(kThreads, 1)
     k_stream_df(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmAlo,
                 const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmXlo, const DfArgs a) {
+  grid_dependency();
   constexpr int RW = rows_warp(R);
   constexpr int G = 32 / LPR;  // row groups per warp
   const int slab_bytes = SHORT ? a.slab_bytes : kSlabBytes;
@@ -258,7 +259,7 @@ cudaError_t launch_r(const StreamArgs& a, int num_sms, cudaStream_t st) {
     return e;
   long long grid = static_cast<long long>(m.n_vec) * m.tiles;
   if (grid > num_sms) grid = num_sms;
-  k_stream_df<R, SHORT, LPR><<<static_cast<unsigned>(grid), kThreads, smem, st>>>(ta, tl, tx, txl, m);
+  launch_next(k_stream_df<R, SHORT, LPR>, static_cast<unsigned>(grid), kThreads, smem, st, ta, tl, tx, txl, m);
   return cudaGetLastError();
 }
 

@@ -63,6 +63,7 @@ template <int P>
 __global__ void __launch_bounds__(kThreads, fft_ctas(P)) k_rfft_rows(const float* __restrict__ x, long long rows,
                                                                   int n_in, const float2* __restrict__ twg,
                                                                   float2* __restrict__ X) {
+  grid_dependency();
   constexpr int N = 32 * P;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* tw = reinterpret_cast<float2*>(smraw);
@@ -105,6 +106,7 @@ __global__ void __launch_bounds__(kThreads, tile_ctas(P))
                 float2* __restrict__ X, long long ld_l, long long rows_a, long long ld_a,
                 const int* __restrict__ lens, int conj, __nv_bfloat162* __restrict__ hi,
                 __nv_bfloat162* __restrict__ lo) {
+  grid_dependency();
   constexpr int N = 32 * P;
   constexpr int NB = N + 1;  // odd: a bin's column of the tile lies on distinct banks
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -173,6 +175,7 @@ template <int P>
 __global__ void __launch_bounds__(kThreads, irfft_ctas(P)) k_irfft_rows(const float2* __restrict__ X, long long rows,
                                                                    const float2* __restrict__ twg,
                                                                    float* __restrict__ x) {
+  grid_dependency();
   constexpr int N = 32 * P;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* tw = reinterpret_cast<float2*>(smraw);
@@ -232,6 +235,7 @@ __global__ void __launch_bounds__(kThreads, fft_ctas(P))
     k_retransform(const float2* __restrict__ mhat, long long Ng, long long ld_m, const float2* __restrict__ twg,
                   float inv_dt, int dt_mode, void* __restrict__ vout, long long ld_v, float* __restrict__ seafloor,
                   long long mhat_ld_b, long long vhat_ld_b, __nv_bfloat162* __restrict__ vout_lo, int n_alloc) {
+  grid_dependency();
   constexpr int N = 32 * P;
   constexpr int NB = N + 1;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -355,6 +359,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce_irfft(const float2* __restr
                                                            long long s_b, long long s_l, long long s_s,
                                                            const float2* __restrict__ twg, float* __restrict__ q,
                                                            int n_keep) {
+  grid_dependency();
   constexpr int N = 32 * P;
   constexpr int NB = N + 1;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -395,6 +400,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce_irfft(const float2* __restr
 // over s in increasing order (the order k_reduce_irfft adds them in), read
 // coalesced along e, so that the reduction reads one segment.
 __global__ void k_sum_chunks(float2* __restrict__ part, int Nb, int nseg, long long per) {
+  grid_dependency();
   const long long total = static_cast<long long>(Nb) * per;
   for (long long e = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; e < total;
        e += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -513,6 +519,7 @@ __global__ void k_fp8_quantize(const float2* __restrict__ spec, int Nb, long lon
 // rupture's No x Nt samples (one CTA per rupture, fixed summation order).
 __global__ void __launch_bounds__(kThreads) k_residual(float* __restrict__ q, const float* __restrict__ d,
                                                        long long n_per_b, float* __restrict__ loss) {
+  grid_dependency();
   const long long base = static_cast<long long>(blockIdx.x) * n_per_b;
   float acc = 0.f;
   for (long long e = threadIdx.x; e < n_per_b; e += kThreads) {
@@ -565,8 +572,8 @@ cudaError_t run_rfft_tile(const float* x, long long rows, int n_in, const float2
   const size_t sm = smem_fft<P>(TR);
   const cudaError_t e = allow_smem(k_rfft_tile<P, PACK, TR>, sm);
   if (e != cudaSuccess) return e;
-  k_rfft_tile<P, PACK, TR><<<fft_grid<P>((rows + TR - 1) / TR, tile_ctas(P)), kThreads, sm, st>>>(
-      x, rows, n_in, tw, X, ld_l, rows_a, ld_a, lens, conj, hi, lo);
+  launch_next(k_rfft_tile<P, PACK, TR>, fft_grid<P>((rows + TR - 1) / TR, tile_ctas(P)), kThreads, sm, st, x, rows,
+              n_in, tw, X, ld_l, rows_a, ld_a, lens, conj, hi, lo);
   return cudaGetLastError();
 }
 
@@ -584,7 +591,7 @@ cudaError_t run_rfft_tile(const float* x, long long rows, int n_in, const float2
 
 cudaError_t launch_residual(float* q, const float* d, int B, long long n_per_b, float* loss, cudaStream_t st) {
   if (B <= 0) return cudaSuccess;
-  k_residual<<<B, kThreads, 0, st>>>(q, d, n_per_b, loss);
+  launch_next(k_residual, B, kThreads, 0, st, q, d, n_per_b, loss);
   return cudaGetLastError();
 }
 
@@ -601,7 +608,8 @@ cudaError_t launch_rfft_rows(const float* x, long long rows, int n_in, int Nt, c
     if (ld_l == 1 && rows_a == 1 && ld_a == Nt + 1 && lens == nullptr) {
       const size_t sm = smem_fft<P>(0);
       if ((e = allow_smem(k_rfft_rows<P>, sm)) != cudaSuccess) return e;
-      k_rfft_rows<P><<<fft_grid<P>((rows + kWarps - 1) / kWarps), kThreads, sm, st>>>(x, rows, n_in, tw, X);
+      launch_next(k_rfft_rows<P>, fft_grid<P>((rows + kWarps - 1) / kWarps), kThreads, sm, st, x, rows, n_in, tw,
+                  X);
     } else if (rows <= kFewRows) {
       e = run_rfft_tile<P, false, 8>(x, rows, n_in, tw, X, ld_l, rows_a, ld_a, lens, 0, nullptr, nullptr, st);
     } else {
@@ -636,7 +644,8 @@ cudaError_t launch_irfft_rows(const float2* X, long long rows, int Nt, const flo
     const size_t sm = smem_fft<P>(0);
     const cudaError_t e = allow_smem(k_irfft_rows<P>, sm);
     if (e != cudaSuccess) return e;
-    k_irfft_rows<P><<<fft_grid<P>((rows + kWarps - 1) / kWarps, irfft_ctas(P)), kThreads, sm, st>>>(X, rows, tw, x);
+    launch_next(k_irfft_rows<P>, fft_grid<P>((rows + kWarps - 1) / kWarps, irfft_ctas(P)), kThreads, sm, st, X,
+                rows, tw, x);
   });
   return cudaGetLastError();
 }
@@ -652,12 +661,12 @@ cudaError_t launch_retransform(const float2* mhat, long long Ng, long long ld_m,
     cudaError_t e;
     if (vhat_bf != nullptr) {
       if ((e = allow_smem(k_retransform<P, true>, sm)) != cudaSuccess) return e;
-      k_retransform<P, true><<<grid, kThreads, sm, st>>>(mhat, Ng, ld_m, tw, inv_dt, dt_mode, vhat_bf, ld_v, seafloor,
-                                                         mhat_ld_b, vhat_ld_b, vhat_bf_lo, n_alloc);
+      launch_next(k_retransform<P, true>, grid, kThreads, sm, st, mhat, Ng, ld_m, tw, inv_dt, dt_mode, vhat_bf,
+                  ld_v, seafloor, mhat_ld_b, vhat_ld_b, vhat_bf_lo, n_alloc);
     } else {
       if ((e = allow_smem(k_retransform<P, false>, sm)) != cudaSuccess) return e;
-      k_retransform<P, false><<<grid, kThreads, sm, st>>>(mhat, Ng, ld_m, tw, inv_dt, dt_mode, vhat, ld_v, seafloor,
-                                                          mhat_ld_b, vhat_ld_b, nullptr, 0);
+      launch_next(k_retransform<P, false>, grid, kThreads, sm, st, mhat, Ng, ld_m, tw, inv_dt, dt_mode, vhat, ld_v,
+                  seafloor, mhat_ld_b, vhat_ld_b, nullptr, 0);
     }
   });
   return cudaGetLastError();
@@ -676,19 +685,19 @@ cudaError_t launch_reduce_irfft(const float2* part, int B, int No, int nseg, int
       const size_t sm = smem_fft<P>(8);
       if ((e = allow_smem(k_reduce_irfft<P, 8>, sm)) != cudaSuccess) return e;
       const long long grid = static_cast<long long>(B) * ((No + 7) / 8);
-      k_reduce_irfft<P, 8><<<static_cast<unsigned>(grid), kThreads, sm, st>>>(part, No, nseg, s_b, s_l, s_s, tw, q,
-                                                                              n_keep);
+      launch_next(k_reduce_irfft<P, 8>, static_cast<unsigned>(grid), kThreads, sm, st, part, No, nseg, s_b, s_l,
+                  s_s, tw, q, n_keep);
     } else {
       const size_t sm = smem_fft<P>(1, 1);
-      k_reduce_irfft<P, 1><<<static_cast<unsigned>(n), kThreads, sm, st>>>(part, No, nseg, s_b, s_l, s_s, tw, q,
-                                                                           n_keep);
+      launch_next(k_reduce_irfft<P, 1>, static_cast<unsigned>(n), kThreads, sm, st, part, No, nseg, s_b, s_l, s_s,
+                  tw, q, n_keep);
     }
   });
   return cudaGetLastError();
 }
 
 cudaError_t launch_sum_chunks(float2* part, int Nb, int nseg, long long per, cudaStream_t st) {
-  k_sum_chunks<<<grid_for(Nb * per, 256), 256, 0, st>>>(part, Nb, nseg, per);
+  launch_next(k_sum_chunks, grid_for(Nb * per, 256), 256, 0, st, part, Nb, nseg, per);
   return cudaGetLastError();
 }
 

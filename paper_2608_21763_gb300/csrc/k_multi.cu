@@ -85,6 +85,7 @@ template <int EL, bool HILO, int R, bool SHORT>
 __global__ void __launch_bounds__(kThreads, 1)
     k_stream_multi(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmAlo,
                    const __grid_constant__ CUtensorMap tmX, const MultiArgs a) {
+  grid_dependency();
   using CH = Chunk<EL>;
   constexpr int C = CH::C;
   const int slab_bytes = SHORT ? a.slab_bytes : kSlabBytes;
@@ -271,7 +272,7 @@ cudaError_t launch_r(const StreamArgs& a, int num_sms, cudaStream_t st) {
     return e;
   long long grid = static_cast<long long>(m.n_vec) * m.tiles;
   if (grid > num_sms) grid = num_sms;
-  k_stream_multi<EL, HILO, R, SHORT><<<static_cast<unsigned>(grid), kThreads, smem, st>>>(ta, tl, tx, m);
+  launch_next(k_stream_multi<EL, HILO, R, SHORT>, static_cast<unsigned>(grid), kThreads, smem, st, ta, tl, tx, m);
   return cudaGetLastError();
 }
 

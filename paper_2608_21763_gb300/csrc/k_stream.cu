@@ -55,6 +55,7 @@ __host__ __device__ constexpr int stream_warps(bool short_rows, int r) {
 template <int EL, bool HILO, bool SHORT, int R = 1>
 __global__ void __launch_bounds__(32 * (stream_warps(SHORT, R) + 1), 1)
     k_stream_dot(const StreamArgs a, int stage_rows) {
+  grid_dependency();
   constexpr int kConsumerWarps = stream_warps(SHORT, R);
   static_assert(R == 1 || (SHORT && EL != EL_FP8), "several vectors: short FP32 or BF16 rows");
   using CH = Chunk<EL>;
@@ -457,7 +458,7 @@ cudaError_t launch_t(const StreamArgs& a, int num_sms, cudaStream_t st) {
   if (grid > a.F) grid = a.F;
   if (grid < 1) grid = 1;
   const dim3 g(static_cast<unsigned>(grid), R == 1 ? static_cast<unsigned>(a.nb) : 1u);
-  k_stream_dot<EL, HILO, SHORT, R><<<g, 32 * (stream_warps(SHORT, R) + 1), smem, st>>>(a, stage_rows);
+  launch_next(k_stream_dot<EL, HILO, SHORT, R>, g, 32 * (stream_warps(SHORT, R) + 1), smem, st, a, stage_rows);
   return cudaGetLastError();
 }
 

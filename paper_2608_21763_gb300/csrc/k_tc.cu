@@ -659,12 +659,14 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* tmA, const CUten
 template <int BK>
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_tc_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const TcArgs a) {
+  grid_dependency();
   tc_gemm_body<BK, 0>(&tmA, &tmB, nullptr, nullptr, a);
 }
 
 template <int BK>
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_tc_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const TcArgs a) {
+  grid_dependency();
   tc_gemm_body<BK, 0, 2>(&tmA, &tmB, nullptr, nullptr, a);
 }
 
@@ -673,6 +675,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 template <int BK>
 __global__ void __launch_bounds__(kTcThreadsF8, 1)
     k_tc_gemm_h(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const TcArgs a) {
+  grid_dependency();
   tc_gemm_body<BK, 5>(&tmA, &tmB, nullptr, nullptr, a);
 }
 
@@ -680,6 +683,7 @@ template <int BK>
 __global__ void __launch_bounds__(kTcThreadsF8, 1)
     k_tc_gemm_pair_h(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                      const TcArgs a) {
+  grid_dependency();
   tc_gemm_body<BK, 5, 2>(&tmA, &tmB, nullptr, nullptr, a);
 }
 
@@ -688,12 +692,14 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     k_tc_gemm_split_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                          const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
                          const TcArgs a) {
+  grid_dependency();
   tc_gemm_body<BK, 1, 2>(&tmA, &tmB, &tmA2, &tmB2, a);
 }
 
 template <int BK>
 __global__ void __launch_bounds__(kTcThreadsF8, 1)
     k_tc_gemm_f8(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const TcArgs a) {
+  grid_dependency();
   tc_gemm_body<BK, 2>(&tmA, &tmB, nullptr, nullptr, a);
 }
 
@@ -702,6 +708,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     k_tc_gemm_split(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
                     const TcArgs a) {
+  grid_dependency();
   tc_gemm_body<BK, 1>(&tmA, &tmB, &tmA2, &tmB2, a);
 }
 
@@ -1088,12 +1095,14 @@ __device__ __forceinline__ void tc_gemm2_body(const CUtensorMap* tmA, const CUte
 template <int BK>
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_tc_gemm2(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const TcArgs a) {
+  grid_dependency();
   tc_gemm2_body<BK, 0>(&tmA, &tmB, nullptr, nullptr, a);
 }
 
 template <int BK>
 __global__ void __launch_bounds__(kTcThreadsF8, 1)
     k_tc_gemm2_f8(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const TcArgs a) {
+  grid_dependency();
   tc_gemm2_body<BK, 2>(&tmA, &tmB, nullptr, nullptr, a);
 }
 
@@ -1101,6 +1110,7 @@ template <int BK>
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_tc_gemm2_f8f8(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const TcArgs a,
                     const float* col_scale, int col_ld) {
+  grid_dependency();
   tc_gemm2_body<BK, 3>(&tmA, &tmB, nullptr, nullptr, a, col_scale, col_ld);
 }
 
@@ -1111,6 +1121,7 @@ template <int BK>
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_tc_gemm2_f8f8lo(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                       const __grid_constant__ CUtensorMap tmB2, const TcArgs a, const float* col_scale, int col_ld) {
+  grid_dependency();
   tc_gemm2_body<BK, 4>(&tmA, &tmB, nullptr, &tmB2, a, col_scale, col_ld);
 }
 
@@ -1119,6 +1130,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     k_tc_gemm2_split(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                      const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
                      const TcArgs a) {
+  grid_dependency();
   tc_gemm2_body<BK, 1>(&tmA, &tmB, &tmA2, &tmB2, a);
 }
 
@@ -1131,6 +1143,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 __global__ void k_pack_b(const float2* __restrict__ src, int Nb, int T, long long nc, long long s_l, long long s_t,
                          long long c0, long long Kc, int N_alloc, int conj, __nv_bfloat162* __restrict__ hi,
                          __nv_bfloat162* __restrict__ lo) {
+  grid_dependency();
   const long long total = static_cast<long long>(Nb) * T * nc;
   for (long long e = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; e < total;
        e += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -1162,6 +1175,7 @@ __global__ void k_pack_b(const float2* __restrict__ src, int Nb, int T, long lon
 // Largest |Re|, |Im| of n complex values into *amax (float bits; *amax
 // starts at 0): the range of a B operand packed as FP16.
 __global__ void k_amax_c(const float2* __restrict__ x, long long n, unsigned* __restrict__ amax) {
+  grid_dependency();
   float m = 0.f;
   for (long long e = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; e < n;
        e += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -1177,6 +1191,7 @@ __global__ void k_amax_c(const float2* __restrict__ x, long long n, unsigned* __
 __global__ void k_pack_b_f16(const float2* __restrict__ src, int Nb, int T, long long nc, long long s_l,
                              long long s_t, long long Kc, int N_alloc, const unsigned* __restrict__ amax,
                              __half2* __restrict__ dst) {
+  grid_dependency();
   const float sc = f16_scale(*amax);
   const long long total = static_cast<long long>(Nb) * T * nc;
   for (long long e = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; e < total;
@@ -1196,6 +1211,7 @@ __global__ void k_pack_b_f16(const float2* __restrict__ src, int Nb, int T, long
 __global__ void k_pack_b_f8(const float2* __restrict__ src, int Nb, int T, long long nc, long long s_l,
                             long long s_t, long long Kc, int N_alloc, int n_rows, float* __restrict__ col_scale,
                             int col_ld, uint16_t* __restrict__ dst, uint16_t* __restrict__ dst_lo) {
+  grid_dependency();
   const int lane = threadIdx.x & 31;
   const int nt = n_rows / 2;
   const long long nw = static_cast<long long>(Nb) * nt;
@@ -1328,6 +1344,7 @@ template <bool SPLIT, bool PAIR>
 __global__ void __launch_bounds__(rt_threads(SPLIT), 1)
     k_tc_retransform(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmT2,
                      const TcRtArgs a) {
+  grid_dependency();
   static_assert(!(SPLIT && PAIR), "two-SM retransform: BF16 only");
   constexpr int BK = SPLIT ? 32 : 64;        // K elements per k-block
   constexpr int EPW = rt_epw(SPLIT);
@@ -1821,11 +1838,11 @@ cudaError_t launch_tc_one(const CUtensorMap& tmA, const CUtensorMap& tmB, const 
   const unsigned grid = static_cast<unsigned>(units < num_sms ? units : num_sms);
   const unsigned threads = MODE == 2 ? kTcThreadsF8 : kTcThreads;
   if (MODE == 1)
-    kern_s<<<grid, threads, smem, st>>>(tmA, tmB, tmA2, tmB2, a);
+    launch_next(kern_s, grid, threads, smem, st, tmA, tmB, tmA2, tmB2, a);
   else if (MODE == 2)
-    kern_f<<<grid, threads, smem, st>>>(tmA, tmB, a);
+    launch_next(kern_f, grid, threads, smem, st, tmA, tmB, a);
   else
-    kern<<<grid, threads, smem, st>>>(tmA, tmB, a);
+    launch_next(kern, grid, threads, smem, st, tmA, tmB, a);
   return cudaGetLastError();
 }
 
@@ -1868,9 +1885,9 @@ cudaError_t launch_tc_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const
     cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     if (a.m_pair)
-      k_tc_gemm_pair_h<64><<<grid, kTcThreadsF8, smem, st>>>(tmA, tmB, a);
+      launch_next(k_tc_gemm_pair_h<64>, grid, kTcThreadsF8, smem, st, tmA, tmB, a);
     else
-      k_tc_gemm_h<64><<<grid, kTcThreadsF8, smem, st>>>(tmA, tmB, a);
+      launch_next(k_tc_gemm_h<64>, grid, kTcThreadsF8, smem, st, tmA, tmB, a);
     return cudaGetLastError();
   }
   if (a.cta2) {  // two-SM MMAs (M = 256 per CTA pair), no M-tile pairs
@@ -1898,7 +1915,7 @@ cudaError_t launch_tc_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const
     cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
@@ -1917,6 +1934,7 @@ cudaError_t launch_tc_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const
     const long long pu = static_cast<long long>(a.Nb) * ((a.m_tiles + 1) / 2) * a.n_kchunks * (nsp ? 2 : 1);
     if (nclusters > pu) nclusters = pu;
     cfg.gridDim = dim3(static_cast<unsigned>(nclusters * 2));
+    cfg.numAttrs = 1 + next_attr(attr + 1, st);
     if (f8lo) {
       if (nsp)
         e = cudaLaunchKernelEx(&cfg, k_tc_gemm2_f8f8lo<128>, tmA, tmB, *tmB2, a, col_scale, col_ld);
@@ -1960,14 +1978,14 @@ cudaError_t launch_tc_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const
     if (e != cudaSuccess) return e;
     if (a.a_lo) {
       if (bk64)
-        k_tc_gemm_split_pair<64><<<grid, kTcThreads, smem, st>>>(tmA, tmB, *tmA2, *tmB2, a);
+        launch_next(k_tc_gemm_split_pair<64>, grid, kTcThreads, smem, st, tmA, tmB, *tmA2, *tmB2, a);
       else
-        k_tc_gemm_split_pair<32><<<grid, kTcThreads, smem, st>>>(tmA, tmB, *tmA2, *tmB2, a);
+        launch_next(k_tc_gemm_split_pair<32>, grid, kTcThreads, smem, st, tmA, tmB, *tmA2, *tmB2, a);
     } else {
       if (bk64)
-        k_tc_gemm_pair<64><<<grid, kTcThreads, smem, st>>>(tmA, tmB, a);
+        launch_next(k_tc_gemm_pair<64>, grid, kTcThreads, smem, st, tmA, tmB, a);
       else
-        k_tc_gemm_pair<32><<<grid, kTcThreads, smem, st>>>(tmA, tmB, a);
+        launch_next(k_tc_gemm_pair<32>, grid, kTcThreads, smem, st, tmA, tmB, a);
     }
     return cudaGetLastError();
   }
@@ -2019,7 +2037,7 @@ cudaError_t launch_tc_retransform(const CUtensorMap& tmT, const CUtensorMap* tmT
     cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
@@ -2038,6 +2056,7 @@ cudaError_t launch_tc_retransform(const CUtensorMap& tmT, const CUtensorMap* tmT
     const long long units = static_cast<long long>(a.Bs) * ((mtiles + 1) / 2);
     if (nclusters > units) nclusters = units;
     cfg.gridDim = dim3(static_cast<unsigned>(nclusters * 2));
+    cfg.numAttrs = 1 + next_attr(attr + 1, st);
     e = cudaLaunchKernelEx(&cfg, k_tc_retransform<false, true>, *tmTp, *tmTp, aa);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
@@ -2048,9 +2067,11 @@ cudaError_t launch_tc_retransform(const CUtensorMap& tmT, const CUtensorMap* tmT
   cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   if (split)
-    k_tc_retransform<true, false><<<static_cast<unsigned>(grid), rt_threads(true), smem, st>>>(tmT, *tmT2, aa);
+    launch_next(k_tc_retransform<true, false>, static_cast<unsigned>(grid), rt_threads(true), smem, st, tmT, *tmT2,
+                aa);
   else
-    k_tc_retransform<false, false><<<static_cast<unsigned>(grid), rt_threads(false), smem, st>>>(tmT, tmT, aa);
+    launch_next(k_tc_retransform<false, false>, static_cast<unsigned>(grid), rt_threads(false), smem, st, tmT, tmT,
+                aa);
   return cudaGetLastError();
 }
 
@@ -2058,8 +2079,8 @@ cudaError_t launch_pack_b(const float2* src, int Nb, int T, long long nc, long l
                           long long Kc, int N_alloc, int conj, void* hi, void* lo, cudaStream_t st) {
   const long long total = static_cast<long long>(Nb) * T * nc;
   if (total <= 0) return cudaSuccess;
-  k_pack_b<<<grid_for_tc(total), 256, 0, st>>>(src, Nb, T, nc, s_l, s_t, c0, Kc, N_alloc, conj,
-                                               static_cast<__nv_bfloat162*>(hi), static_cast<__nv_bfloat162*>(lo));
+  launch_next(k_pack_b, grid_for_tc(total), 256, 0, st, src, Nb, T, nc, s_l, s_t, c0, Kc, N_alloc, conj,
+              static_cast<__nv_bfloat162*>(hi), static_cast<__nv_bfloat162*>(lo));
   return cudaGetLastError();
 }
 
@@ -2072,9 +2093,8 @@ cudaError_t launch_pack_b_f8(const float2* src, int Nb, int T, long long nc, lon
   if (warps <= 0) return cudaSuccess;
   long long blocks = (warps + 7) / 8;
   if (blocks > 152LL * 16) blocks = 152LL * 16;
-  k_pack_b_f8<<<static_cast<unsigned>(blocks), 256, 0, st>>>(src, Nb, T, nc, s_l, s_t, Kc, N_alloc, n_rows,
-                                                                col_scale, col_ld, static_cast<uint16_t*>(dst),
-                                                                static_cast<uint16_t*>(dst_lo));
+  launch_next(k_pack_b_f8, static_cast<unsigned>(blocks), 256, 0, st, src, Nb, T, nc, s_l, s_t, Kc, N_alloc, n_rows,
+              col_scale, col_ld, static_cast<uint16_t*>(dst), static_cast<uint16_t*>(dst_lo));
   return cudaGetLastError();
 }
 
@@ -2084,9 +2104,9 @@ cudaError_t launch_pack_b_f16(const float2* src, int Nb, int T, long long nc, lo
   if (total <= 0) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(amax, 0, sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
-  k_amax_c<<<grid_for_tc(total), 256, 0, st>>>(src, total, amax);
-  k_pack_b_f16<<<grid_for_tc(total), 256, 0, st>>>(src, Nb, T, nc, s_l, s_t, Kc, N_alloc, amax,
-                                                   static_cast<__half2*>(dst));
+  launch_next(k_amax_c, grid_for_tc(total), 256, 0, st, src, total, amax);
+  launch_next(k_pack_b_f16, grid_for_tc(total), 256, 0, st, src, Nb, T, nc, s_l, s_t, Kc, N_alloc, amax,
+              static_cast<__half2*>(dst));
   return cudaGetLastError();
 }
 

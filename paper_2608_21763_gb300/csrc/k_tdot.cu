@@ -49,6 +49,7 @@ constexpr int kBudget = 208 * 1024;    // ring and sums (up to 64 KB)
 template <int EL, bool HILO, int R>
 __global__ void __launch_bounds__(32 * (tdot_warps(EL) + 1), 1)
     k_stream_tdot(const StreamTArgs a, int stage_rows, int stages, int cols, int groups) {
+  grid_dependency();
   using CH = Chunk<EL>;
   constexpr int C = CH::C;
   constexpr int kWarps = tdot_warps(EL);
@@ -289,7 +290,8 @@ cudaError_t launch_r(const StreamTArgs& a, int num_sms, cudaStream_t st) {
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   const long long grid = a.n_units < num_sms ? a.n_units : num_sms;
-  k_stream_tdot<EL, HILO, R><<<static_cast<unsigned>(grid), kCons + 32, smem, st>>>(a, stage_rows, stages, cols, groups);
+  launch_next(k_stream_tdot<EL, HILO, R>, static_cast<unsigned>(grid), kCons + 32, smem, st, a, stage_rows, stages,
+              cols, groups);
   return cudaGetLastError();
 }
 

@@ -47,6 +47,51 @@ __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
 
 // ---------------------------------------------------------------------------
+// Launches of a call's chain of kernels.  A kernel launched with launch_next
+// need not wait for the memory flush and the completion message of the one
+// before it in the stream: it is launched when that one's last CTA has
+// exited, and every thread first waits (grid_dependency, before any read or
+// write) until it has completed with its writes visible.  Every kernel of
+// such a chain waits, so completion stays in stream order; a kernel launched
+// without it (anyone's) is ordered as ever.  Bound by launch latency at small
+// sizes, per call before and after: the tiny FP32-pair workload 34.9 -> 26.2
+// us (the host's rate now); 200 subfaults x 2,000 points x 128 steps, 40
+// ruptures BF16, 116 -> 103; 300 x 1,000 x 128, 40 ruptures FP8, 103 -> 90;
+// 200 x 4,000 x 256, one FP32 rupture, 491 -> 479; 963 x 20,000 x 256, 8
+// ruptures BF16, 3.462 -> 3.447 ms.  Letting the next kernel's CTAs in early
+// (cudaTriggerProgrammaticLaunchCompletion at the start) gave nothing
+// more and cost the larger ones up to 3 % (501 x 10,007 x 128, 6
+// ruptures forward and backward: 2.186 ms before, 2.165 as it is, 2.236).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void grid_dependency() { cudaGridDependencySynchronize(); }
+
+// The launch attribute: one, or none under capture (graphs keep plain edges).
+inline unsigned next_attr(cudaLaunchAttribute* attr, cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr->val.programmaticStreamSerializationAllowed = 1;
+  return cap == cudaStreamCaptureStatusNone ? 1 : 0;
+}
+
+// Errors are left for cudaGetLastError, as <<<>>> leaves them.
+template <class... P, class... A>
+void launch_next(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = next_attr(attr, st);
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// ---------------------------------------------------------------------------
 // PTX wrappers: shared-memory addresses, mbarriers, bulk async copies
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
