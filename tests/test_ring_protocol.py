@@ -177,3 +177,55 @@ def test_converter_stage_ring(S, seed):
             state[s] = (n, "converted" if len(converted[n]) == CONV else "converting")
             aready[s].arrive()
             conv[a] += 1
+
+
+@pytest.mark.parametrize("S", [2, 3, 5, 6, 12])
+@pytest.mark.parametrize("seed", range(20))
+def test_converter_warps_that_own_ring_slots(S, seed):
+    """The same ring where each of 4 converter warps completes whole stages,
+    those of the slots s with s % 4 its own (stage 2's B): the copies of
+    several stages are in flight and land in any order, aready[s] counts one
+    arrival, and no stage is converted before it has landed or read before
+    it is converted.  (Warps that took every fourth stage instead of every
+    fourth slot would meet a slot's full barrier a phase early: with S = 3 or
+    5 the parity wait then passes on the use before.)"""
+    import random
+    rnd = random.Random(2000 + seed)
+    NK, CONV = 41, 4
+    full, aready, empty = ([Barrier(1) for _ in range(S)] for _ in range(3))
+    state = [(None, "read")] * S       # (use n, 'loading' | 'loaded' | 'converted' | 'read')
+    prod, mma, conv = 0, 0, [0] * CONV
+    steps = 0
+    while mma < NK:
+        steps += 1
+        assert steps < 200000, "no progress"
+        a = rnd.choice(["prod", "land", "mma"] + list(range(CONV)))
+        if a == "prod" and prod < NK:
+            s = prod % S
+            if prod >= S and not empty[s].ready(((prod // S) - 1) & 1):
+                continue
+            assert state[s][1] == "read", (prod, state[s])
+            state[s] = (prod, "loading")
+            prod += 1
+        elif a == "land":
+            flying = [s for s in range(S) if state[s][1] == "loading"]
+            if flying:
+                s = rnd.choice(flying)
+                state[s] = (state[s][0], "loaded")
+                full[s].arrive()
+        elif a == "mma":
+            s = mma % S
+            if aready[s].ready((mma // S) & 1):
+                assert state[s] == (mma, "converted"), (mma, state[s])
+                state[s] = (mma, "read")
+                empty[s].arrive()
+                mma += 1
+        elif isinstance(a, int):
+            while conv[a] < NK and (conv[a] % S) % CONV != a:
+                conv[a] += 1
+            if conv[a] < NK and full[conv[a] % S].ready((conv[a] // S) & 1):
+                s = conv[a] % S
+                assert state[s] == (conv[a], "loaded"), (a, conv[a], state[s])
+                state[s] = (conv[a], "converted")
+                aready[s].arrive()
+                conv[a] += 1
