@@ -518,7 +518,8 @@ def run_ours(args, rank, world, local_rank):
     else:
         alg = stage1_algorithmic_bytes(wl, args.prec_g, 1, args.single_pass)
         achieved = alg / per_launch_s / 1e9
-        roof = {"kernel": "k_stream_dot (stage-1 per-bin contraction)", "bound": "hbm",
+        kname = "k_stream_df" if args.prec_g == "fp32_hilo" else "k_stream_dot"
+        roof = {"kernel": kname + " (stage-1 per-bin contraction)", "bound": "hbm",
                 "achieved": round(achieved, 1), "peak": pk["hbm_gbs"], "unit": "GB/s",
                 "frac": round(achieved / pk["hbm_gbs"], 4), "peak_source": pk_kind,
                 "traffic": None if args.single_pass else measured_traffic(wl, args.prec_g),
