@@ -222,6 +222,8 @@ __global__ void __launch_bounds__(32 * (tdot_warps(EL) + 1), 1)
       if (++s == stages) s = 0, ph ^= 1;
     }
     float2* y = a.y + u * a.row_len;
+    const int nc = static_cast<int>(  // columns that are not padding
+        max(0LL, min(static_cast<long long>(a.row_len), a.cols - (g % a.wa) * a.row_len)));
     flush(groups > 1);
     if (groups == 1) {
       if (!ok) return;
@@ -230,9 +232,14 @@ __global__ void __launch_bounds__(32 * (tdot_warps(EL) + 1), 1)
         for (int b = 0; b < R; ++b)
           if (b < a.nb)
 #pragma unroll
-            for (int q = 0; q < C; q += 2)
-              *reinterpret_cast<float4*>(y + b * a.y_ldb + c0 * C + q) =
-                  make_float4(acc[b][q].x, acc[b][q].y, acc[b][q + 1].x, acc[b][q + 1].y);
+            for (int q = 0; q < C; q += 2) {
+              float2* yc = y + b * a.y_ldb + c0 * C + q;
+              if (c0 * C + q + 1 < nc)
+                *reinterpret_cast<float4*>(yc) =
+                    make_float4(acc[b][q].x, acc[b][q].y, acc[b][q + 1].x, acc[b][q + 1].y);
+              else if (c0 * C + q < nc)
+                *yc = acc[b][q];
+            }
       }
       continue;
     }
@@ -242,6 +249,7 @@ __global__ void __launch_bounds__(32 * (tdot_warps(EL) + 1), 1)
     const float2* all = reinterpret_cast<const float2*>(part - threadIdx.x);
     for (int e = threadIdx.x; e < live; e += kCons) {
       const int b = e / a.row_len, col = e - b * a.row_len;
+      if (col >= nc) continue;
       const int at = 2 * ((b * (C / 2) + col % C / 2) * kCons + col / C) + (col & 1);
       float2 p[4];  // four partial sums: shorter chains, less rounding
 #pragma unroll

@@ -1604,6 +1604,7 @@ int s2w_adjoint(s2w_ctx* ctx, const float* r, int B, float* grad_s, void* stream
       a.w_base = static_cast<long long>(b) * No;
       a.wa = ctx->nseg;
       a.wb = static_cast<long long>(B) * No;
+      a.cols = Ng;
       a.nb = nb;
       a.w_ldb = No;
       a.y = ctx->ws_vhat;
@@ -1632,6 +1633,7 @@ int s2w_adjoint(s2w_ctx* ctx, const float* r, int B, float* grad_s, void* stream
       a.w_base = 0;
       a.wa = 1;
       a.wb = Ng;
+      a.cols = Ns;
       a.scale = ctx->G_scale;
       a.nblk = ctx->nblk;
       a.nb = nb;

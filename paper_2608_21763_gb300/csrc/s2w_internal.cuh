@@ -272,7 +272,10 @@ cudaError_t launch_stream_df(const StreamArgs& a, int num_sms, cudaStream_t st);
 // k_tdot.cu, transposed: y[u][c] = sum_{f in unit u} conj(rows[f][c]) w_f,
 // unit u = chunk (u % nchunk) of Rc rows of group (u / nchunk) of G1 rows,
 // w_f = w[w_base + (g / wa) * wb + (f - g G1)], g = f / G1 (times the FP8
-// scale[g * nblk + (f - g G1) / 256] for FP8 rows).
+// scale[g * nblk + (f - g G1) / 256] for FP8 rows).  The rows of wa groups
+// in turn hold `cols` entries, then padding: only those columns are written
+// (a weight that is not finite would leave NaN in the others, where the
+// forward pass wants zeros).
 struct StreamTArgs {
   const void* rows;
   const void* rows_lo;
@@ -283,6 +286,7 @@ struct StreamTArgs {
   int Rc, nchunk;
   const float2* w;
   long long w_base, wa, wb;
+  long long cols;
   const float* scale;
   int nblk;
   float2* y;
