@@ -8,28 +8,37 @@
 // by TMA: the tile's rows (512 bytes of each, 32 chunks of 16) and the same
 // columns of the R vectors, which come from L2 after their first use.  Warp w
 // owns eight of the rows, lane l chunk l of each slab, and the FP32
-// accumulators of all 8 x R products stay in registers over the whole row;
-// at the end one butterfly reduce-scatter over the lanes sums them.
+// accumulators of all 8 x R products stay in registers over the whole row, or
+// half of a long one; then one butterfly reduce-scatter over the lanes sums
+// them.
 //
 // What bounds it: 4 FMAs per stored entry and rupture.  At eight ruptures an
 // FP32 entry costs 32 FMAs for 8 bytes; scalar FFMAs with three register
 // operands run at 25 TFMA/s here, so the FMAs take as long as the bytes at
-// the copy rate at about six ruptures, and eight take 1.2x the time of one
-// (963 x 8,000 x 64 x 256: 2.46 ms for one, 2.50 for two, 2.54 for four, 2.96
-// for eight, 19.5 ms eight times over; 480 x 37,758 x 32 x 256, eight
-// ruptures: 46.0 -> 8.0 ms; 333 x 4,999 x 17 x 512 with seafloor output, five:
-// 6.66 -> 1.42 ms).  Rows are cut into K slabs (not whole rows per warp)
-// because eight warps with eight whole rows each would need 0.5 MB of shared
-// memory, and eight rows per warp because each vector entry read from shared
-// memory must serve several rows.  Packed FP32 products (35 TFMA/s) were
-// slower here: they want the vectors twice (rotated), in registers or in
-// shared-memory reads, at two warps per scheduler (8.8 ms; also twelve warps
-// with four or six rows each, 8.3 - 9.3 ms).
+// the copy rate at about six ruptures.  Rows are cut into K slabs (not whole
+// rows per warp) because eight warps with eight whole rows each would need
+// 0.5 MB of shared memory, and eight rows per warp because each vector entry
+// read from shared memory must serve several rows.  Packed FP32 products (35
+// TFMA/s) on (re, im) pairs were slower here: they want the vectors twice
+// (rotated), in registers or in shared-memory reads, at two warps per
+// scheduler (also twelve warps with four or six rows each).
 //
 // Each lane sums its chunks l, l + 32, ... in column order into one
-// accumulator per component, then the lanes are added over xor 16, 8, 4, 2, 1:
-// the order of k_stream_dot, so a rupture's result is the same bits alone or
-// in a batch.
+// accumulator per component, then the lanes are added over xor 16, 8, 4, 2, 1;
+// a row of more than two slabs goes in two blocks (chain_slabs), each reduced
+// by itself, then added: k_stream_dot's order, so a rupture's result is the
+// same bits alone or in a batch.  The two blocks round like two accumulators
+// per component, for which there are no registers (128 hold one each).  They
+// cost eight ruptures a second reduction, about 500 instructions per 64 rows
+// and lane; dealing each lane its rows in an order that the reduction wants
+// takes the selections out of it.  Stage 1 of 963 x 8,000 x 64 x 256: one
+// rupture 2.25 ms, two 2.28, four 2.39, six 2.34, eight 2.78 (2.61 in one
+// block; 18.0 eight times over).  Whole calls, operators read once per
+// rupture, then one block, then as it is: 480 x 37,758 x 32 x 256, eight
+// ruptures, 46.0 -> 7.94 -> 8.65 ms; 333 x 4,999 x 17 x 512 with seafloor
+// output, five, 6.66 -> 1.37 -> 1.52 ms.  Other ways to the same rounding, at
+// the first of these: two accumulators with four rows per warp 10.4 ms, the
+// first block's sums kept in tensor memory 8.7 - 9.4.
 #include <cuda.h>
 
 #include <type_traits>
@@ -55,6 +64,7 @@ constexpr int kBudget = 208 * 1024;   // ring bytes
 struct MultiArgs {
   int n_vec, rows_per_vec, tiles, mrows;  // tiles of mrows rows per vector group
   int slabs, stages;
+  int block;        // slabs of the first block (chain_slabs), all of them in rows that are not cut
   int slab_bytes;   // of each row per stage: kSlabBytes, or the whole of a shorter row
   int nb;
   int x_vec_first;  // the vector map's dimensions are (entry, vector, rupture), else (entry, rupture, vector)
@@ -152,78 +162,90 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int vec = static_cast<int>(u / a.tiles), tile = static_cast<int>(u % a.tiles);
     const int nr = min(a.mrows, a.rows_per_vec - tile * a.mrows);
     // a full tile gives each warp eight adjacent rows (64-byte stores), a
-    // partial one deals its rows out over the warps
+    // partial one deals its rows out over the warps.  The lanes of a full
+    // tile's warp take their eight rows in an order of their own, so that
+    // the reduction's first three steps need no selection
     const bool whole = nr == kWarps * RW;
     const int r_w = whole ? RW : 1, r_i = whole ? 1 : kWarps;
     const int row0 = warp * r_w;
-    float acc[RW * R * 2];
+    const int deal = !SHORT && whole ? lane >> 2 : 0;  // slot i of the lane is row i ^ deal of the warp's
+    constexpr int PL = RW * R / 16;  // sums of a lane
+    float sum[PL];
+    for (int k0 = 0, k1 = a.block; k0 < a.slabs; k0 = k1, k1 = a.slabs) {
+      float acc[RW * R * 2];
 #pragma unroll
-    for (int k = 0; k < RW * R * 2; ++k) acc[k] = 0.f;
-    for (int k = 0; k < a.slabs; ++k) {
-      if (!mbar_wait_bounded(full + s, ph, a.status, DEV_ERR_TIMEOUT_FULL, a.wait_ns)) return;
-      const unsigned char* st = ring + s * stage_bytes;
-      const uint4* rows = reinterpret_cast<const uint4*>(st) + lane;
-      const uint4* rows_lo = reinterpret_cast<const uint4*>(st + a_bytes) + lane;
-      const float4* xs = reinterpret_cast<const float4*>(st + a_bytes * (HILO ? 2 : 1)) + lane * (C / 2);
-      auto slab = [&](auto whole_tag) {
-        constexpr bool WHOLE = decltype(whole_tag)::value;
+      for (int k = 0; k < RW * R * 2; ++k) acc[k] = 0.f;
+      for (int k = k0; k < k1; ++k) {
+        if (!mbar_wait_bounded(full + s, ph, a.status, DEV_ERR_TIMEOUT_FULL, a.wait_ns)) return;
+        const unsigned char* st = ring + s * stage_bytes;
+        const uint4* rows = reinterpret_cast<const uint4*>(st) + lane;
+        const uint4* rows_lo = reinterpret_cast<const uint4*>(st + a_bytes) + lane;
+        const float4* xs = reinterpret_cast<const float4*>(st + a_bytes * (HILO ? 2 : 1)) + lane * (C / 2);
+        auto slab = [&](auto whole_tag) {
+          constexpr bool WHOLE = decltype(whole_tag)::value;
 #pragma unroll
-        for (int h = 0; h < C / 2; ++h) {  // two entries of the lane's chunk at a time
-          float4 x[R];
+          for (int h = 0; h < C / 2; ++h) {  // two entries of the lane's chunk at a time
+            float4 x[R];
 #pragma unroll
-          for (int b = 0; b < R; ++b) x[b] = xs[b * pitch * (C / 2) + h];
+            for (int b = 0; b < R; ++b) x[b] = xs[b * pitch * (C / 2) + h];
 #pragma unroll
-          for (int i = 0; i < RW; ++i) {
-            const int row = WHOLE ? row0 + i : row0 + kWarps * i;
-            if (!WHOLE && row >= nr) continue;
-            float2 g[C];
-            CH::unpack(rows[row * pitch], g);
-            if (HILO) {
-              float2 gl[C];
-              CH::unpack(rows_lo[row * pitch], gl);
+            for (int i = 0; i < RW; ++i) {
+              const int row = WHOLE ? row0 + (i ^ deal) : row0 + kWarps * i;
+              if (!WHOLE && row >= nr) continue;
+              float2 g[C];
+              CH::unpack(rows[row * pitch], g);
+              if (HILO) {
+                float2 gl[C];
+                CH::unpack(rows_lo[row * pitch], gl);
 #pragma unroll
-              for (int q = 0; q < C; ++q) g[q] = cadd(g[q], gl[q]);
-            }
-            const float2 g0 = g[2 * h], g1 = g[2 * h + 1];
+                for (int q = 0; q < C; ++q) g[q] = cadd(g[q], gl[q]);
+              }
+              const float2 g0 = g[2 * h], g1 = g[2 * h + 1];
 #pragma unroll
-            for (int b = 0; b < R; ++b) {
-              cmac(g0, make_float2(x[b].x, x[b].y), acc[(i * R + b) * 2], acc[(i * R + b) * 2 + 1]);
-              cmac(g1, make_float2(x[b].z, x[b].w), acc[(i * R + b) * 2], acc[(i * R + b) * 2 + 1]);
+              for (int b = 0; b < R; ++b) {
+                cmac(g0, make_float2(x[b].x, x[b].y), acc[(i * R + b) * 2], acc[(i * R + b) * 2 + 1]);
+                cmac(g1, make_float2(x[b].z, x[b].w), acc[(i * R + b) * 2], acc[(i * R + b) * 2 + 1]);
+              }
             }
           }
+        };
+        if (!SHORT || lane < pitch) {  // (a row shorter than a slab leaves lanes without a chunk)
+          if (whole)
+            slab(std::true_type{});
+          else
+            slab(std::false_type{});
         }
-      };
-      if (!SHORT || lane < pitch) {  // (a row shorter than a slab leaves lanes without a chunk)
-        if (whole)
-          slab(std::true_type{});
-        else
-          slab(std::false_type{});
+        __syncwarp();
+        if (lane == 0) mbar_arrive(empty + s);
+        if (++s == S) s = 0, ph ^= 1;
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(empty + s);
-      if (++s == S) s = 0, ph ^= 1;
-    }
-    // reduce-scatter over the lanes: after the step with lane bit o a lane
-    // keeps the half of its values that the bit selects, summed with its
-    // partner's; value index ((row * R) + b) * 2 + component
+      // reduce-scatter over the lanes: after the step with lane bit o a lane
+      // keeps the half of its values that the bit selects, summed with its
+      // partner's; value index ((row * R) + b) * 2 + component
 #pragma unroll
-    for (int o = 16, n = RW * R; o > 0; o >>= 1, n >>= 1) {
-      const bool up = (lane & o) != 0;
+      for (int o = 16, n = RW * R; o > 0; o >>= 1, n >>= 1) {
+        const bool up = (lane & o) != 0;
+        if (!SHORT && o > 2 && whole) {  // the rows are dealt so that the first half is the lane's own
 #pragma unroll
-      for (int k = 0; k < RW * R; ++k) {
-        if (k < n) {
-          const float keep = up ? acc[k + n] : acc[k];
-          const float send = up ? acc[k] : acc[k + n];
-          acc[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+          for (int k = 0; k < n; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k + n], o);
+        } else {
+#pragma unroll
+          for (int k = 0; k < n; ++k) {
+            const float keep = up ? acc[k + n] : acc[k];
+            const float send = up ? acc[k] : acc[k + n];
+            acc[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+          }
         }
       }
+#pragma unroll
+      for (int j = 0; j < PL; ++j) sum[j] = k0 == 0 ? acc[j] : sum[j] + acc[j];
     }
     float2* y = a.y + static_cast<long long>(vec) * a.rows_per_vec + tile * a.mrows;
 #pragma unroll
-    for (int j = 0; j < RW * R / 16; ++j) {
-      const int v = lane * (RW * R / 16) + j;  // (each step's bit selects a half: lane major)
+    for (int j = 0; j < PL; ++j) {
+      const int v = lane * PL + j;  // (each step's bit selects a half: lane major)
       const int row = row0 + v / (2 * R) * r_i, b = v / 2 % R;
-      if (row < nr && b < a.nb) reinterpret_cast<float*>(y + b * a.y_ldb + row)[v & 1] = acc[j];
+      if (row < nr && b < a.nb) reinterpret_cast<float*>(y + b * a.y_ldb + row)[v & 1] = sum[j];
     }
   }
 }
@@ -241,6 +263,7 @@ cudaError_t launch_r(const StreamArgs& a, int num_sms, cudaStream_t st) {
   m.mrows = a.rows_per_vec >= tile_rows ? tile_rows : static_cast<int>((a.rows_per_vec + 7) / 8 * 8);
   m.tiles = (m.rows_per_vec + m.mrows - 1) / m.mrows;
   m.slabs = static_cast<int>((row_bytes + kSlabBytes - 1) / kSlabBytes);
+  m.block = chain_slabs(m.slabs) > 0 ? chain_slabs(m.slabs) : m.slabs;
   const int stage = (m.mrows * m.slab_bytes * (HILO ? 2 : 1) + R * x_bytes + 127) & ~127;
   m.stages = kBudget / stage < kMaxStages ? kBudget / stage : kMaxStages;
   m.nb = a.nb;

@@ -52,7 +52,14 @@ __host__ __device__ constexpr int stream_warps(bool short_rows, int r) {
 // each lane's slices of all R held in registers, so a batch reads the
 // operator once per R ruptures.  Otherwise a batch takes one grid slice (y)
 // per rupture.
-template <int EL, bool HILO, bool SHORT, int R = 1>
+// BLK: slabs in the first block of a long FP32 / BF16 row (chain_slabs), so
+// the row has 2 BLK or 2 BLK + 1 of them.  A kernel for each count keeps the
+// blocks' border and the empty slabs of shorter rows out of the row loop,
+// which is bound by its instructions below about 500 entries: stage 1, one
+// rupture, 190 x 20,000 x 256 FP32 2.01 ms in one kernel for all lengths, 1.12
+// here; 300 x 12,000 1.44 -> 1.08; 300 x 8,000 BF16 0.71 -> 0.53; 963 x 8,000 FP32
+// 2.30 -> 2.25 (its bytes), BF16 1.16 -> 1.15.
+template <int EL, bool HILO, bool SHORT, int R = 1, int BLK = 0>
 __global__ void __launch_bounds__(32 * (stream_warps(SHORT, R) + 1), 1)
     k_stream_dot(const StreamArgs a, int stage_rows) {
   grid_dependency();
@@ -61,7 +68,8 @@ __global__ void __launch_bounds__(32 * (stream_warps(SHORT, R) + 1), 1)
   using CH = Chunk<EL>;
   constexpr int C = CH::C;
   // chunk slots per lane: a short row gives each lane at most four chunks
-  constexpr int T = SHORT ? 4 : kMaxRowLen / (32 * C);
+  constexpr int kMostSlabs = kMaxRowLen / (32 * C);
+  constexpr int T = SHORT ? 4 : (BLK > 0 && 2 * BLK + 1 < kMostSlabs ? 2 * BLK + 1 : kMostSlabs);
   extern __shared__ __align__(128) unsigned char sm[];
   uint64_t* full = reinterpret_cast<uint64_t*>(sm);
   uint64_t* empty = full + kStages;
@@ -376,11 +384,13 @@ __global__ void __launch_bounds__(32 * (stream_warps(SHORT, R) + 1), 1)
         }
       } else {
         // The order of k_stream_multi (chunk c on lane c mod 32, one chain per
-        // component and lane, then the lanes added over xor 16, 8, .. 1), so
+        // component and lane, then the lanes added over xor 16, 8, .. 1; a long
+        // row's blocks of slabs each by itself, then one after the other), so
         // that a rupture's result does not depend on the batch.  A short row's
         // lane holds four of those lanes' chunks: with 16 lanes per row the
         // chunks t and t + 2 are one chain, with fewer all four are apart.
         constexpr int H = SHORT ? 2 : 1;  // chains per lane and component
+        float first_a = 0.f, first_i = 0.f;  // a long row's first block (R = 1)
         float xa[H][R], xi[H][R], sa[H][R], si[H][R];
 #pragma unroll
         for (int h = 0; h < H; ++h)
@@ -389,6 +399,10 @@ __global__ void __launch_bounds__(32 * (stream_warps(SHORT, R) + 1), 1)
 #pragma unroll
         for (int t = 0; t < T; ++t) {
           const int c = sub + lpr * t;
+          if (!SHORT && t == BLK) {
+            first_a = xa[0][0], first_i = xi[0][0];
+            xa[0][0] = xi[0][0] = 0.f;
+          }
           if (SHORT && t == 2 && lpr < 16) {
 #pragma unroll
             for (int h = 0; h < H; ++h)
@@ -399,7 +413,7 @@ __global__ void __launch_bounds__(32 * (stream_warps(SHORT, R) + 1), 1)
                 xa[h][b] = xi[h][b] = 0.f;
               }
           }
-          if (valid && c < nchunk) {
+          if ((!SHORT || valid) && (t < 2 * BLK - 1 || c < nchunk)) {
             float2 g[C];
             CH::unpack(row[c], g);
             if (HILO) {
@@ -423,17 +437,29 @@ __global__ void __launch_bounds__(32 * (stream_warps(SHORT, R) + 1), 1)
           ar[b] = SHORT ? (sa[0][b] + xa[0][b]) + (sa[H - 1][b] + xa[H - 1][b]) : xa[0][b];
           ai[b] = SHORT ? (si[0][b] + xi[0][b]) + (si[H - 1][b] + xi[H - 1][b]) : xi[0][b];
         }
-        for (int o = lpr / 2; o > 0; o >>= 1) {
+        if constexpr (SHORT) {
+          for (int o = lpr / 2; o > 0; o >>= 1) {
 #pragma unroll
-          for (int b = 0; b < R; ++b) {
-            ar[b] += __shfl_xor_sync(0xffffffffu, ar[b], o);
-            ai[b] += __shfl_xor_sync(0xffffffffu, ai[b], o);
+            for (int b = 0; b < R; ++b) {
+              ar[b] += __shfl_xor_sync(0xffffffffu, ar[b], o);
+              ai[b] += __shfl_xor_sync(0xffffffffu, ai[b], o);
+            }
           }
-        }
-        if (valid && sub == 0) {
+          if (valid && sub == 0) {
 #pragma unroll
-          for (int b = 0; b < R; ++b)
-            if (R == 1 || b < a.nb) ay[b * a.y_ldb + f] = make_float2(ar[b], ai[b]);
+            for (int b = 0; b < R; ++b)
+              if (R == 1 || b < a.nb) ay[b * a.y_ldb + f] = make_float2(ar[b], ai[b]);
+          }
+        } else {
+          // reduce-scatter: lane bit 16 selects the block, bit 8 the component
+          const bool last = (lane & 16) != 0, im = (lane & 8) != 0;
+          float re = (last ? ar[0] : first_a) + __shfl_xor_sync(0xffffffffu, last ? first_a : ar[0], 16);
+          float iv = (last ? ai[0] : first_i) + __shfl_xor_sync(0xffffffffu, last ? first_i : ai[0], 16);
+          float v = (im ? iv : re) + __shfl_xor_sync(0xffffffffu, im ? re : iv, 8);
+#pragma unroll
+          for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          v += __shfl_xor_sync(0xffffffffu, v, 16);  // the two blocks
+          if ((lane & ~8) == 0) reinterpret_cast<float*>(ay + f)[lane >> 3] = v;
         }
       }
     }
@@ -442,7 +468,7 @@ __global__ void __launch_bounds__(32 * (stream_warps(SHORT, R) + 1), 1)
   }
 }
 
-template <int EL, bool HILO, bool SHORT, int R = 1>
+template <int EL, bool HILO, bool SHORT, int R = 1, int BLK = 0>
 cudaError_t launch_t(const StreamArgs& a, int num_sms, cudaStream_t st) {
   constexpr int C = Chunk<EL>::C;
   const int row_bytes = a.row_len * (16 / C);
@@ -451,14 +477,14 @@ cudaError_t launch_t(const StreamArgs& a, int num_sms, cudaStream_t st) {
   if (stage_rows >= 8) stage_rows -= stage_rows % 8;
   if (stage_rows < 1) stage_rows = 1;
   const size_t smem = 128 + static_cast<size_t>(kStages) * stage_rows * row_bytes * (HILO ? 2 : 1);
-  cudaError_t e = cudaFuncSetAttribute(k_stream_dot<EL, HILO, SHORT, R>,
+  cudaError_t e = cudaFuncSetAttribute(k_stream_dot<EL, HILO, SHORT, R, BLK>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   long long grid = num_sms;
   if (grid > a.F) grid = a.F;
   if (grid < 1) grid = 1;
   const dim3 g(static_cast<unsigned>(grid), R == 1 ? static_cast<unsigned>(a.nb) : 1u);
-  launch_next(k_stream_dot<EL, HILO, SHORT, R>, g, 32 * (stream_warps(SHORT, R) + 1), smem, st, a, stage_rows);
+  launch_next(k_stream_dot<EL, HILO, SHORT, R, BLK>, g, 32 * (stream_warps(SHORT, R) + 1), smem, st, a, stage_rows);
   return cudaGetLastError();
 }
 
@@ -471,12 +497,19 @@ bool short_rows(const StreamArgs& a, int C) { return a.row_len / C <= 64; }
 namespace {
 // Rows of at most this many chunks stay on the lane groups in a batch.
 constexpr int kShortestChunks = 16;
+// Long rows of one rupture, by the slabs of their first block.
+template <int EL, bool HILO, int BLK = 1>
+cudaError_t launch_long(const StreamArgs& a, int num_sms, cudaStream_t st) {
+  constexpr int C = Chunk<EL>::C, most = chain_slabs(kMaxRowLen / (32 * C));
+  if constexpr (BLK < most)
+    if (chain_slabs((a.row_len / C + 31) / 32) > BLK) return launch_long<EL, HILO, BLK + 1>(a, num_sms, st);
+  return launch_t<EL, HILO, false, 1, BLK>(a, num_sms, st);
+}
 // One launch for a.nb ruptures of FP32 / BF16 storage (nb <= kStreamMulti).
 template <int EL, bool HILO>
 cudaError_t launch_plain(const StreamArgs& a, int num_sms, cudaStream_t st) {
   if (a.nb == 1)
-    return short_rows(a, Chunk<EL>::C) ? launch_t<EL, HILO, true>(a, num_sms, st)
-                                       : launch_t<EL, HILO, false>(a, num_sms, st);
+    return short_rows(a, Chunk<EL>::C) ? launch_t<EL, HILO, true>(a, num_sms, st) : launch_long<EL, HILO>(a, num_sms, st);
   // A batch: k_stream_multi, whose warps take eight rows at about the same
   // cost however short they are; the shortest rows in lane groups here, at
   // most kMostVectors at a time (a lane holds its slices of every vector)

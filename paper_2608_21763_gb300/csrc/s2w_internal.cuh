@@ -263,6 +263,14 @@ struct StreamArgs {
 constexpr int kStreamMulti = 8;
 cudaError_t launch_stream_dot(const StreamArgs& a, int num_sms, cudaStream_t st);
 
+// Rows of 16-byte chunks are dealt over 32 lanes in slabs of 32 chunks.  A
+// row longer than two slabs is summed in two blocks, the first of
+// chain_slabs(slabs) slabs (0: not cut): one accumulation per lane over the
+// whole row rounds 1.05 (three slabs) to 1.28 times (sixteen) as much as two
+// of half its products each (of random sign), the two blocks 1.00 with an even
+// count of slabs and 1.02 (three) to 1.00 (fifteen) with an odd one.
+__host__ __device__ constexpr int chain_slabs(int slabs) { return slabs > 2 ? slabs / 2 : 0; }
+
 // k_multi.cu: the same for 2 .. kStreamMulti ruptures and FP32 / BF16 /
 // BF16 hi/lo rows of more than 64 16-byte chunks (launch_stream_dot calls it).
 cudaError_t launch_stream_multi(const StreamArgs& a, int num_sms, cudaStream_t st);
