@@ -51,6 +51,7 @@ struct s2w_ctx {
   float* ws_slip = nullptr;
   float2* ws_shat = nullptr;
   int multi = 1;               // ruptures per streaming launch: ws_mhat, ws_vhat hold this many
+  int multi_adj = 1;           // the same for the adjoint: ws_gpart holds this many (0: no adjoint)
   float2* ws_mhat = nullptr;   // [multi][Nb][Ng]
   float2* ws_vhat = nullptr;   // [multi][Nb][nseg * RL]
   float2* ws_part = nullptr;
@@ -60,7 +61,7 @@ struct s2w_ctx {
   float* ws_resid = nullptr;   // misfit gradient: q then r = q - d, [b][No][Nt]
   float* ws_d = nullptr;       // misfit gradient: staged targets, [b][No][Nt]
   float* ws_loss = nullptr;    // misfit gradient: per-rupture loss
-  float2* ws_gpart = nullptr;  // adjoint: stage-1 chunk partials [multi][l][chunk][Ns_pad]
+  float2* ws_gpart = nullptr;  // adjoint: stage-1 chunk partials [multi_adj][l][chunk][Ns_pad]
   int adj_rc = 512;            // adjoint: grid rows per stage-1 chunk
   int adj_nchunk = 1;
   int* d_status = nullptr;
@@ -1064,20 +1065,31 @@ int s2w_create(int Ns, int Ng, int No, int Nt, const s2w_opts* opts, s2w_ctx** o
     }
   }
   // Seafloor and velocity spectra and the adjoint's partials of the streaming
-  // kernels, last: room for kStreamMulti ruptures per launch when that takes
-  // at most 1/8 of the memory still free, for fewer (at least the one that
-  // every call needs) otherwise.  Results do not depend on the count.
+  // kernels, last: one set per rupture of a pass, for as many ruptures as the
+  // kernels that this context can run share a pass of the operator for.
+  // ENGINE_TENSOR streams only where it has no other way (seafloor output,
+  // the adjoint without its operands) and keeps one; FP32 pairs take two and
+  // have no adjoint, nor has the single-pass variant; FP8 rows are shared by
+  // the adjoint alone, four ruptures; with the adjoint's tensor operands only
+  // batches below the threshold stream it.  The sets past the first take at
+  // most 1/16 of the operators' bytes (or 1 GiB) and 1/8 of the memory still
+  // free.  Results do not depend on the count.
   {
     const size_t mh = sizeof(float2) * Nb * Ng, vh = sizeof(float2) * Nb * ctx->nseg * ctx->RL;
     const size_t gp = sizeof(float2) * Nb * ctx->adj_nchunk * ctx->Ns_pad;
+    const bool adjoint = !ctx->df && !ctx->single_pass;
+    const int want = o.engine == S2W_ENGINE_TENSOR ? 1 : (ctx->df ? 2 : (o.prec_g == S2W_PREC_FP8_E4M3 ? 4 : kStreamMulti));
     size_t free_b = 0, total_b = 0;
-    int m = static_cast<int>(std::min<long long>(B, kStreamMulti));
+    int m = static_cast<int>(std::min<long long>(B, want));
     if (m > 1 && (e = cudaMemGetInfo(&free_b, &total_b)) != cudaSuccess) return bad(e, "free memory");
-    while (m > 1 && static_cast<size_t>(m) * ((mh + vh) * (ctx->df ? 2 : 1) + gp) > free_b / 8) m /= 2;
+    const size_t most = std::min(free_b / 8, std::max<size_t>(1ull << 30, (ctx->g_bytes + ctx->p_bytes) / 16));
+    const size_t set = (mh + vh) * (ctx->df ? 2 : 1) + (adjoint && !ctx->tc_adj ? gp : 0);
+    while (m > 1 && static_cast<size_t>(m - 1) * set > most) m /= 2;
     ctx->multi = m;
+    ctx->multi_adj = !adjoint ? 0 : (ctx->tc_adj ? 1 : m);
     if ((e = dalloc(&ctx->ws_mhat, m * mh)) != cudaSuccess) return bad(e, "seafloor spectra");
     if ((e = dalloc(&ctx->ws_vhat, m * vh)) != cudaSuccess) return bad(e, "velocity spectra");
-    if ((e = dalloc(&ctx->ws_gpart, m * gp)) != cudaSuccess) return bad(e, "adjoint partials");
+    if (adjoint && (e = dalloc(&ctx->ws_gpart, ctx->multi_adj * gp)) != cudaSuccess) return bad(e, "adjoint partials");
     if (ctx->df) {
       if ((e = dalloc(&ctx->ws_mhat_lo, m * mh)) != cudaSuccess) return bad(e, "seafloor spectra lo");
       if ((e = dalloc(&ctx->ws_vhat_lo, m * vh)) != cudaSuccess) return bad(e, "velocity spectra lo");
@@ -1587,9 +1599,9 @@ int s2w_adjoint(s2w_ctx* ctx, const float* r, int B, float* grad_s, void* stream
   const int dt_t = ctx->opts.dt_mode == S2W_DT_NONE ? S2W_DT_NONE : kDtTranspose;
   const long long vcols = static_cast<long long>(ctx->nseg) * ctx->RL;
   const long long mhat_b = Nb * Ng, vhat_b = Nb * vcols, gpart_b = Nb * ctx->adj_nchunk * Ns_pad;  // per rupture
-  const int npass = (B + ctx->multi - 1) / ctx->multi;
+  const int npass = (B + ctx->multi_adj - 1) / ctx->multi_adj;
   for (int p = 0, b = 0, nb = 0; p < npass; ++p, b += nb) {
-    nb = (B - b + npass - p - 1) / (npass - p);  // equal passes of at most ctx->multi ruptures
+    nb = (B - b + npass - p - 1) / (npass - p);  // equal passes of at most ctx->multi_adj ruptures
     {  // stage-2 adjoint: what_l[i] = sum_o conj(Phat_l[o][i]) rhat_l[o]
       StageTimer t(ctx, 3, st);
       StreamTArgs a{};
