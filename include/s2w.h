@@ -349,8 +349,8 @@ typedef struct {
  * stage-2 K chunk count (how the grid is split between the persistent
  * CTAs; with the BF16 hi/lo split, only counts at or above the default,
  * since each chunk is one FP32 accumulation and a longer one costs that
- * precision accuracy), and the batch size from which AUTO uses the tensor engine instead
- * of streaming the spectra once per rupture.  The choices are kept in the
+ * precision accuracy), and the batch size from which AUTO uses the tensor engine:
+ * the smallest that it takes less time for than the streaming kernels do.  The choices are kept in the
  * context (and written to opts.tune_cache when one is set); an entry already
  * in that cache is applied without timing.  Options the caller fixed
  * (tc_bsub, tc_pair other than AUTO, tc_s2_chunks) are not searched.

@@ -1924,8 +1924,10 @@ int s2w_autotune(s2w_ctx* ctx, int B, s2w_tuning* out, void* stream) {
   CK(cudaEventCreate(&e1));
   // dummy inputs: the slip workspace (any values; the timings do not depend on them)
   auto timed = [&](int nb, int engine, float* ms) -> int {
-    const int saved = ctx->opts.engine;
+    // (a context with the tensor engine on takes it from tc_min_batch up)
+    const int saved = ctx->opts.engine, saved_min = ctx->tc_min_batch;
     ctx->opts.engine = engine;
+    ctx->tc_min_batch = engine == S2W_ENGINE_STREAM ? nb + 1 : 1;
     int rc = s2w_waveforms(ctx, ctx->ws_slip, nb, ctx->ws_q, nullptr, st);  // warm-up
     float best = 1e30f;
     for (int rep = 0; rep < 2 && rc == S2W_OK; ++rep) {
@@ -1938,6 +1940,7 @@ int s2w_autotune(s2w_ctx* ctx, int B, s2w_tuning* out, void* stream) {
       best = std::min(best, m);
     }
     ctx->opts.engine = saved;
+    ctx->tc_min_batch = saved_min;
     *ms = best;
     return rc;
   };
@@ -2002,13 +2005,17 @@ int s2w_autotune(s2w_ctx* ctx, int B, s2w_tuning* out, void* stream) {
       set_s2_chunks(ctx, best_c);
     }
     r.tc_s2_chunks = ctx->tc_nkc;
-    // 3. the smallest batch whose tensor pass beats that many stream passes of one rupture
+    // 3. the smallest batch that the tensor engine takes less time for than
+    // the stream engine, whose ruptures share passes of the operators
     const int sizes[7] = {1, 2, 4, 8, 16, 32, 64};
     int min_b = 0;
     for (int k = 0; k < 7 && rc == S2W_OK; ++k) {
       if (sizes[k] > B || sizes[k] > ctx->tc_bsub) break;
       rc = timed(sizes[k], S2W_ENGINE_TENSOR, &r.ms_tensor_batch[k]);
-      if (rc == S2W_OK && min_b == 0 && r.ms_tensor_batch[k] < sizes[k] * r.ms_stream_per_rupture) min_b = sizes[k];
+      if (rc != S2W_OK || min_b != 0) continue;
+      float ms_stream = r.ms_stream_per_rupture;
+      if (sizes[k] > 1) rc = timed(sizes[k], S2W_ENGINE_STREAM, &ms_stream);
+      if (rc == S2W_OK && r.ms_tensor_batch[k] < ms_stream) min_b = sizes[k];
     }
     if (min_b == 0) min_b = r.ms_tensor_batch[0] > 0.f ? ctx->tc_bsub + 1 : ctx->tc_min_batch;
     ctx->tc_min_batch = min_b;
