@@ -180,7 +180,8 @@ typedef struct {
                       (default).  s2w_autotune reads its choices from it
                       when the file holds an entry for this problem (Ns,
                       Ng, No, Nt, the batch, both precisions, the FP8
-                      activation and adjoint options and the GPU model) and
+                      activation and adjoint options, the GPU model, and
+                      a revision of the kernels it was timed on) and
                       otherwise measures and writes one.  The string is read
                       during s2w_create and s2w_autotune only. */
   int fault;        /* test hook, an s2w_fault (default S2W_FAULT_NONE).  When

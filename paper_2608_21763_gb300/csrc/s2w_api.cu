@@ -1804,6 +1804,10 @@ namespace {
 //   s2w-tune-1 <key> bsub=<n> pair=<n> s2c=<n> minb=<n>
 // with <key> naming everything the choices depend on.  A later entry for the
 // same key replaces the earlier one.
+// kTuneRev: raised when a choice means other kernels, or kernels of another
+// cost, than before (2: the two-SM rules of S2W_PAIR_AUTO, ruptures sharing
+// stream passes), so that entries timed on the earlier ones are timed again.
+constexpr int kTuneRev = 2;
 std::string tune_key(const s2w_ctx* ctx, int B) {
   cudaDeviceProp pr;
   char name[256] = "unknown";
@@ -1813,9 +1817,9 @@ std::string tune_key(const s2w_ctx* ctx, int B) {
       if (*c == ' ' || *c == '\t') *c = '_';
   }
   char k[512];
-  std::snprintf(k, sizeof(k), "Ns=%d,Ng=%d,No=%d,Nt=%d,B=%d,pg=%d,pp=%d,f8a=%d,adj=%d,bmax=%d,sms=%d,gpu=%s", ctx->Ns,
-                ctx->Ng, ctx->No, ctx->Nt, B, ctx->opts.prec_g, ctx->opts.prec_p, ctx->opts.tc_fp8_act,
-                ctx->opts.tc_adjoint, ctx->tc_bsub_max, ctx->num_sms, name);
+  std::snprintf(k, sizeof(k), "Ns=%d,Ng=%d,No=%d,Nt=%d,B=%d,pg=%d,pp=%d,f8a=%d,adj=%d,bmax=%d,sms=%d,gpu=%s,rev=%d",
+                ctx->Ns, ctx->Ng, ctx->No, ctx->Nt, B, ctx->opts.prec_g, ctx->opts.prec_p, ctx->opts.tc_fp8_act,
+                ctx->opts.tc_adjoint, ctx->tc_bsub_max, ctx->num_sms, name, kTuneRev);
   return k;
 }
 

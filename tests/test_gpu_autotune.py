@@ -23,3 +23,20 @@ def test_threshold_compares_the_engines_on_the_same_batch():
     t = ctx.autotune(32)
     print(t)
     assert 4 < t["tc_min_batch"] <= 16
+
+
+def test_cache_entries_of_earlier_kernels_are_timed_again(tmp_path):
+    """An entry without the revision of the kernels that it was timed on is
+    not applied; it stays in the file, and the new entry is."""
+    import re
+
+    cache = tmp_path / "tune.txt"
+    kw = dict(prec_g="bf16", prec_p="bf16", max_batch=8, tune_cache=str(cache))
+    assert not random_context(24, 700, 6, 64, **kw).autotune(8)["from_cache"]
+    line = cache.read_text()
+    earlier = re.sub(r",rev=\d+", "", line)
+    cache.write_text(earlier)
+    ctx = random_context(24, 700, 6, 64, **kw)
+    assert not ctx.autotune(8)["from_cache"]
+    assert earlier in cache.read_text() and cache.read_text().count("\n") == 2
+    assert ctx.autotune(8)["from_cache"]
