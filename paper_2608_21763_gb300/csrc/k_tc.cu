@@ -1935,6 +1935,7 @@ cudaError_t launch_tc_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const
     if (nclusters > pu) nclusters = pu;
     cfg.gridDim = dim3(static_cast<unsigned>(nclusters * 2));
     cfg.numAttrs = 1 + next_attr(attr + 1, st);
+    ++g_chain_launches;
     if (f8lo) {
       if (nsp)
         e = cudaLaunchKernelEx(&cfg, k_tc_gemm2_f8f8lo<128>, tmA, tmB, *tmB2, a, col_scale, col_ld);
@@ -2057,6 +2058,7 @@ cudaError_t launch_tc_retransform(const CUtensorMap& tmT, const CUtensorMap* tmT
     if (nclusters > units) nclusters = units;
     cfg.gridDim = dim3(static_cast<unsigned>(nclusters * 2));
     cfg.numAttrs = 1 + next_attr(attr + 1, st);
+    ++g_chain_launches;
     e = cudaLaunchKernelEx(&cfg, k_tc_retransform<false, true>, *tmTp, *tmTp, aa);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();

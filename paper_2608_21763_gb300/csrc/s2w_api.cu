@@ -322,14 +322,14 @@ cudaEvent_t take_event(s2w_ctx* c) {
 }
 
 // Brackets one stage launch with CUDA events on its stream when the profiler
-// is on; counts `n` kernel launches either way.
+// is on; counts the kernels launched meanwhile either way.
 struct StageTimer {
   s2w_ctx* c;
   int stage;
   cudaStream_t st;
   cudaEvent_t a = nullptr, b = nullptr;
-  StageTimer(s2w_ctx* c_, int stage_, cudaStream_t st_, int n = 1) : c(c_), stage(stage_), st(st_) {
-    c->launches += n;
+  long long l0 = g_chain_launches;
+  StageTimer(s2w_ctx* c_, int stage_, cudaStream_t st_) : c(c_), stage(stage_), st(st_) {
     if (c->prof_on) {
       a = take_event(c);
       b = take_event(c);
@@ -337,6 +337,7 @@ struct StageTimer {
     }
   }
   ~StageTimer() {
+    c->launches += g_chain_launches - l0;
     if (a && b) {
       cudaEventRecord(b, st);
       c->pending.push_back({stage, a, b});
@@ -591,7 +592,7 @@ int waveforms_tensor(s2w_ctx* ctx, const float* slip_d, int B, float* q_d, cudaS
                           static_cast<int>(Nt), ctx->tw, ctx->ws_shat, Bs * Ns_pad, Ns, Ns_pad, st, lens));
     }
     if (f8) {
-      StageTimer t(ctx, 6, st, f8f8 ? 1 : 2);
+      StageTimer t(ctx, 6, st);
       if (f8f8)  // e4m3 operand (+ lo parts), one power-of-two scale per (bin, rupture)
         CK(launch_pack_b_f8(ctx->ws_shat, static_cast<int>(Nb), Bs, Ns_pad, static_cast<long long>(Bs) * Ns_pad,
                             Ns_pad, Ns_pad, ctx->tc_n1max, N1, ctx->tc_colscale, ctx->tc_n1max / 2, ctx->tc_bp1,
@@ -1399,7 +1400,7 @@ int s2w_waveforms(s2w_ctx* ctx, const float* slip, int B, float* q, float* seafl
   if (use_tc && ks == 0 && kq == 0 && B > ctx->tc_bsub) return waveforms_tensor_host(ctx, slip, B, q, st);
   const float* slip_d = slip;
   if (ks == 0) {
-    StageTimer t(ctx, 5, st, 0);
+    StageTimer t(ctx, 5, st);
     CK(cudaMemcpyAsync(ctx->ws_slip, slip, sizeof(float) * B * Ns * Nt, cudaMemcpyHostToDevice, st));
     slip_d = ctx->ws_slip;
   }
@@ -1408,7 +1409,7 @@ int s2w_waveforms(s2w_ctx* ctx, const float* slip, int B, float* q, float* seafl
     int rc = waveforms_tensor(ctx, slip_d, B, q_d, st);
     if (rc != S2W_OK) return rc;
     if (kq == 0) {
-      StageTimer t(ctx, 5, st, 0);
+      StageTimer t(ctx, 5, st);
       CK(cudaMemcpyAsync(q, q_d, sizeof(float) * B * No * Nt, cudaMemcpyDeviceToHost, st));
       CK(cudaStreamSynchronize(st));
     }
@@ -1465,7 +1466,7 @@ int s2w_waveforms(s2w_ctx* ctx, const float* slip, int B, float* q, float* seafl
       }
       // K3
       if (ctx->single_pass) {  // mhat goes to stage 2 as it is, in the segment layout
-        StageTimer t(ctx, 2, st, 0);
+        StageTimer t(ctx, 2, st);
         CK(cudaMemcpy2DAsync(ctx->ws_vhat, sizeof(float2) * vcols, ctx->ws_mhat, sizeof(float2) * Ng,
                              sizeof(float2) * Ng, nb * Nb, cudaMemcpyDeviceToDevice, st));
       } else {
@@ -1529,7 +1530,7 @@ int s2w_waveforms(s2w_ctx* ctx, const float* slip, int B, float* q, float* seafl
     }
   }
   if (kq == 0) {
-    StageTimer t(ctx, 5, st, 0);
+    StageTimer t(ctx, 5, st);
     CK(cudaMemcpyAsync(q, q_d, sizeof(float) * B * No * Nt, cudaMemcpyDeviceToHost, st));
   }
   if (kq == 0 || (seafloor && kf == 0)) CK(cudaStreamSynchronize(st));
@@ -1576,7 +1577,7 @@ int s2w_adjoint(s2w_ctx* ctx, const float* r, int B, float* grad_s, void* stream
   const long long Ns = ctx->Ns, Ng = ctx->Ng, No = ctx->No, Nt = ctx->Nt, Nb = ctx->Nb, Ns_pad = ctx->Ns_pad;
   const float* r_d = r;
   if (kr == 0) {
-    StageTimer t(ctx, 5, st, 0);
+    StageTimer t(ctx, 5, st);
     CK(cudaMemcpyAsync(ctx->ws_q, r, sizeof(float) * B * No * Nt, cudaMemcpyHostToDevice, st));
     r_d = ctx->ws_q;
   }
@@ -1585,7 +1586,7 @@ int s2w_adjoint(s2w_ctx* ctx, const float* r, int B, float* grad_s, void* stream
     const int rc = adjoint_tensor(ctx, r_d, B, g_d, st);
     if (rc != S2W_OK) return rc;
     if (kg == 0) {
-      StageTimer t(ctx, 5, st, 0);
+      StageTimer t(ctx, 5, st);
       CK(cudaMemcpyAsync(grad_s, g_d, sizeof(float) * B * Ns * Nt, cudaMemcpyDeviceToHost, st));
       CK(cudaStreamSynchronize(st));
     }
@@ -1663,7 +1664,7 @@ int s2w_adjoint(s2w_ctx* ctx, const float* r, int B, float* grad_s, void* stream
     }
   }
   if (kg == 0) {
-    StageTimer t(ctx, 5, st, 0);
+    StageTimer t(ctx, 5, st);
     CK(cudaMemcpyAsync(grad_s, g_d, sizeof(float) * B * Ns * Nt, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
   }
@@ -1690,7 +1691,7 @@ int s2w_misfit_gradient(s2w_ctx* ctx, const float* slip, const float* d, int B, 
   if (rc != S2W_OK) return rc;
   const float* d_d = d;
   if (kd == 0) {
-    StageTimer t(ctx, 5, st, 0);
+    StageTimer t(ctx, 5, st);
     CK(cudaMemcpyAsync(ctx->ws_d, d, sizeof(float) * B * n_per_b, cudaMemcpyHostToDevice, st));
     d_d = ctx->ws_d;
   }
@@ -1791,7 +1792,8 @@ int s2w_waveforms_graph(s2w_ctx* ctx, const float* slip, int B, float* q, void* 
     ge = &ctx->graphs.back();
   }
   ge->last_use = ++ctx->graph_clock;
-  StageTimer t(ctx, 7, st, static_cast<int>(ge->launches));
+  StageTimer t(ctx, 7, st);
+  ctx->launches += ge->launches;
   CK(cudaGraphLaunch(ge->exec, st));
   return S2W_OK;
 }

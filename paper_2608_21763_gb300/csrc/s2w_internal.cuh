@@ -77,6 +77,10 @@ inline unsigned next_attr(cudaLaunchAttribute* attr, cudaStream_t st) {
   return cap == cudaStreamCaptureStatusNone ? 1 : 0;
 }
 
+// Kernels of such chains launched by this thread: a stage may take several
+// launches (passes of a few ruptures, ranges of K), so they are counted here.
+inline thread_local long long g_chain_launches = 0;
+
 // Errors are left for cudaGetLastError, as <<<>>> leaves them.
 template <class... P, class... A>
 void launch_next(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, const A&... args) {
@@ -88,6 +92,7 @@ void launch_next(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem,
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = next_attr(attr, st);
+  ++g_chain_launches;
   cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
