@@ -153,10 +153,11 @@ def _stream(stream, *arrays):
         return getattr(stream, "cuda_stream", stream)
     for a in arrays:
         if a is not None and not isinstance(a, np.ndarray) and getattr(a, "is_cuda", False):
-            # the handle alone: a torch.cuda.Stream object of it takes 2 us of
-            # a small call's 26
+            # the handle alone, where torch gives it (the name is not public):
+            # a torch.cuda.Stream object of it takes 2 us of a small call's 26
             import torch
-            return torch._C._cuda_getCurrentRawStream(a.get_device())
+            raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+            return raw(a.get_device()) if raw else torch.cuda.current_stream(a.device).cuda_stream
     return None
 
 
