@@ -69,9 +69,8 @@ struct Chunk<EL_FP8> {
 // Complex products on packed FP32 pairs: a stream of scalar FFMAs with three
 // register operands reaches 25.3 TFMA/s on this GPU (register reads), packed
 // ones 35.0 of 37.  y + g x in two instructions, from x prepared as (re, im)
-// and (-im, re): g.re times the one, then g.im times the other.  The same
-// FMAs in scalar form: cmac.
-__device__ __forceinline__ float4 cprep(float2 x) { return make_float4(x.x, x.y, -x.y, x.x); }
+// and (-im, re): g.re times the one, then g.im times the other (conj(g) x: the
+// second (im, -re)).  The FMAs of g x in scalar form: cmac.
 __device__ __forceinline__ float2 cmac2_re(float2 g, float4 x, float2 y) {
   return __ffma2_rn(make_float2(g.x, g.x), make_float2(x.x, x.y), y);
 }

@@ -99,24 +99,6 @@ __device__ __forceinline__ void acc_add(dacc& a, dfl v) {
   a.c += t.lo + v.lo;
 }
 
-// a += x * y
-__device__ __forceinline__ void acc_mac(dacc& a, dfl x, dfl y) {
-  const dfl p = two_prod(x.hi, y.hi);
-  const float cross = fmaf(x.hi, y.lo, fmaf(x.lo, y.hi, p.lo));
-  const dfl t = two_sum(a.s, p.hi);
-  a.s = t.hi;
-  a.c += t.lo + cross;
-}
-
-// a += x * y for an FP32 x (exact input samples)
-__device__ __forceinline__ void acc_mac_f(dacc& a, float x, dfl y) {
-  const dfl p = two_prod(x, y.hi);
-  const float cross = fmaf(x, y.lo, p.lo);
-  const dfl t = two_sum(a.s, p.hi);
-  a.s = t.hi;
-  a.c += t.lo + cross;
-}
-
 // a + b of two partial accumulators
 __device__ __forceinline__ dacc acc_merge(dacc a, dacc b) {
   const dfl t = two_sum(a.s, b.s);

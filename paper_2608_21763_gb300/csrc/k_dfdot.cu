@@ -58,7 +58,8 @@ __device__ __forceinline__ void tma_words(void* sdst, const CUtensorMap* tm, int
 }
 
 // (s, c) += (g + gl) (x + xl) for two real products at once (x: two values):
-// df.cuh's acc_mac on packed pairs; a - b is fma(b, -1, a).
+// TwoProduct, the two cross terms and TwoSum of df.cuh on packed pairs; a - b
+// is fma(b, -1, a).
 __device__ __forceinline__ void pmac(float2& s, float2& c, float g, float gl, float2 x, float2 xl) {
   const float2 m1 = make_float2(-1.f, -1.f), g2 = make_float2(g, g);
   const float2 p = __fmul2_rn(g2, x);

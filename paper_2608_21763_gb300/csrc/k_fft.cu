@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(kThreads, fft_ctas(P)) k_rfft_rows(const float
 // rows (with a warp per row storing one 8-byte entry per bin, 963 x 256 rows
 // of 256 samples took 0.58 ms, 0.24 now; with the packing 0.87 -> 0.25).  Bin l of row `row`, with a = row / rows_a and c = row %
 // rows_a, goes to X[l * ld_l + a * ld_a + c]; or, PACK, into the B operand of
-// the real embedding (k_tc.cu: k_pack_b, conj as there), rows 2a, 2a + 1 of
+// the real embedding (k_tc.cu: k_pack_b; conj: the conjugate one), rows 2a, 2a + 1 of
 // hi / lo[l * ld_l + 2 a * ld_a + c], BF16 pairs.
 // Many rows: 32 per tile (128-byte stores of BF16 pairs; 96,300 rows of hi/lo
 // pairs 0.24 -> 0.16 ms against 16), 16 at 512 points (shared memory).  Up to

@@ -1135,13 +1135,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 }
 
 // B operand of the real embedding from complex FP32 x[l][t][c] (element
-// src[l*s_l + t*s_t + c], c < nc): rows 2t / 2t+1 of dst[l][N_alloc][2 Kc]
-// (BF16, round to nearest even) at complex columns c0 + c:
-//   plain (D = A x):        row 2t = (Re x, -Im x),  row 2t+1 = (Im x,  Re x)
-//   conj  (D = conj(A) x):  row 2t = (Re x,  Im x),  row 2t+1 = (Im x, -Re x)
-// With `lo`, lo = bf16(v - hi) holds the low-order part of every entry.
+// src[l*s_l + t*s_t + c], c < nc), BF16, round to nearest even, at complex
+// columns c0 + c: rows 2t = (Re x, -Im x) and 2t+1 = (Im x, Re x) of
+// dst[l][N_alloc][2 Kc], or with `half` the first of them alone as row t (the
+// half-stored stage-2 operand).  With `lo`, lo = bf16(v - hi) holds the
+// low-order part of every entry.
 __global__ void k_pack_b(const float2* __restrict__ src, int Nb, int T, long long nc, long long s_l, long long s_t,
-                         long long c0, long long Kc, int N_alloc, int conj, __nv_bfloat162* __restrict__ hi,
+                         long long c0, long long Kc, int N_alloc, bool half, __nv_bfloat162* __restrict__ hi,
                          __nv_bfloat162* __restrict__ lo) {
   grid_dependency();
   const long long total = static_cast<long long>(Nb) * T * nc;
@@ -1151,24 +1151,14 @@ __global__ void k_pack_b(const float2* __restrict__ src, int Nb, int T, long lon
     const long long t = (e / nc) % T;
     const long long l = e / (nc * T);
     const float2 v = src[l * s_l + t * s_t + c];
-    if (conj == 2) {  // first half of the plain embedding only: row t = (Re, -Im)
-      const long long o = (l * N_alloc + t) * Kc + c0 + c;
-      const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, -v.y);
-      hi[o] = h;
-      if (lo != nullptr) lo[o] = __floats2bfloat162_rn(v.x - __low2float(h), -v.y - __high2float(h));
-      continue;
-    }
-    const float2 r0 = conj ? make_float2(v.x, v.y) : make_float2(v.x, -v.y);
-    const float2 r1 = conj ? make_float2(v.y, -v.x) : make_float2(v.y, v.x);
-    const long long o0 = (l * N_alloc + 2 * t) * Kc + c0 + c;
-    const __nv_bfloat162 h0 = __floats2bfloat162_rn(r0.x, r0.y);
-    const __nv_bfloat162 h1 = __floats2bfloat162_rn(r1.x, r1.y);
+    const long long o0 = (l * N_alloc + (half ? t : 2 * t)) * Kc + c0 + c;
+    const __nv_bfloat162 h0 = __floats2bfloat162_rn(v.x, -v.y);
     hi[o0] = h0;
+    if (lo != nullptr) lo[o0] = __floats2bfloat162_rn(v.x - __low2float(h0), -v.y - __high2float(h0));
+    if (half) continue;
+    const __nv_bfloat162 h1 = __floats2bfloat162_rn(v.y, v.x);
     hi[o0 + Kc] = h1;
-    if (lo != nullptr) {
-      lo[o0] = __floats2bfloat162_rn(r0.x - __low2float(h0), r0.y - __high2float(h0));
-      lo[o0 + Kc] = __floats2bfloat162_rn(r1.x - __low2float(h1), r1.y - __high2float(h1));
-    }
+    if (lo != nullptr) lo[o0 + Kc] = __floats2bfloat162_rn(v.y - __low2float(h1), v.x - __high2float(h1));
   }
 }
 
@@ -2027,12 +2017,12 @@ cudaError_t launch_tc_retransform(const CUtensorMap& tmT, const CUtensorMap* tmT
   const size_t a_slot = static_cast<size_t>(kBlockM) * BK * 2 * (split ? 2 : 1);
   const size_t t_slot = static_cast<size_t>(pair ? ncols / 2 : ncols) * BK * 2 * (split ? 2 : 1);
   TcRtArgs aa = a;
-  aa.ra = kRtFillWarps;  // k-block slots of A: a whole tile (BF16), one per fill warp (split)
+  constexpr int RA = kRtFillWarps;  // k-block slots of A: a whole tile (BF16), one per fill warp (split)
   // T slots fill the opt-in shared memory left by the A ring (up to four)
-  aa.rt = static_cast<int>((kSmemOptInLimit - 1024 - (8 * (2 * aa.ra + 2 * 4 + 4) + 16) - aa.ra * a_slot) / t_slot);
+  aa.rt = static_cast<int>((kSmemOptInLimit - 1024 - (8 * (2 * RA + 2 * 4 + 4) + 16) - RA * a_slot) / t_slot);
   if (aa.rt > 4) aa.rt = 4;
   if (aa.rt < 2) return cudaErrorInvalidValue;
-  const size_t smem = 1024 + aa.ra * a_slot + aa.rt * t_slot + 8 * (2 * aa.ra + 2 * aa.rt + 4) + 16;
+  const size_t smem = 1024 + RA * a_slot + aa.rt * t_slot + 8 * (2 * RA + 2 * aa.rt + 4) + 16;
   if (pair) {
     const void* kfn = reinterpret_cast<const void*>(k_tc_retransform<false, true>);
     cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
@@ -2078,10 +2068,10 @@ cudaError_t launch_tc_retransform(const CUtensorMap& tmT, const CUtensorMap* tmT
 }
 
 cudaError_t launch_pack_b(const float2* src, int Nb, int T, long long nc, long long s_l, long long s_t, long long c0,
-                          long long Kc, int N_alloc, int conj, void* hi, void* lo, cudaStream_t st) {
+                          long long Kc, int N_alloc, bool half, void* hi, void* lo, cudaStream_t st) {
   const long long total = static_cast<long long>(Nb) * T * nc;
   if (total <= 0) return cudaSuccess;
-  launch_next(k_pack_b, grid_for_tc(total), 256, 0, st, src, Nb, T, nc, s_l, s_t, c0, Kc, N_alloc, conj,
+  launch_next(k_pack_b, grid_for_tc(total), 256, 0, st, src, Nb, T, nc, s_l, s_t, c0, Kc, N_alloc, half,
               static_cast<__nv_bfloat162*>(hi), static_cast<__nv_bfloat162*>(lo));
   return cudaGetLastError();
 }

@@ -1275,7 +1275,7 @@ int load_adjoint_impl(s2w_ctx* ctx, int g0, int ng, const float* P, bool spectra
       if (ctx->tc_on) {
         ctx->launches += 1;
         CK(launch_pack_b(stage_s, static_cast<int>(Nb), static_cast<int>(No), rc, No * rc, rc, g0 + c, ctx->Ng_pad2,
-                         ctx->tc_p2h ? ctx->tc_n2 / 2 : ctx->tc_n2, ctx->tc_p2h ? 2 : 0, ctx->tc_p2, ctx->tc_p2_lo,
+                         ctx->tc_p2h ? ctx->tc_n2 / 2 : ctx->tc_n2, ctx->tc_p2h, ctx->tc_p2, ctx->tc_p2_lo,
                          st));
       }
       if (ctx->tc_adj) {  // Phat_l^T[g0 + c + r][o] (transposing copy; observations along K)

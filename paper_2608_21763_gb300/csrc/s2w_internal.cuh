@@ -186,8 +186,8 @@ cudaError_t launch_rfft_rows(const float* x, long long rows, int n_in, int Nt, c
                              const int* lens = nullptr);
 // launch_rfft_rows of rows of Nt samples straight into the B operand of the
 // real embedding (launch_pack_b with complex columns row % rows_a of operand
-// rows 2t, 2t + 1, t = row / rows_a: dst[l][N_alloc][Kc], hi and optional lo;
-// conj 0 or 1).
+// rows 2t, 2t + 1, t = row / rows_a: dst[l][N_alloc][Kc], hi and optional lo);
+// conj: the conjugate embedding, rows (Re, Im) and (Im, -Re).
 cudaError_t launch_rfft_pack(const float* x, long long rows, int Nt, const float2* tw, long long rows_a,
                              long long Kc, int N_alloc, int conj, void* hi, void* lo, cudaStream_t st,
                              const int* lens = nullptr);
@@ -385,7 +385,7 @@ cudaError_t launch_tc_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const
 // conj = 2 writes row 2t of the plain embedding, (Re, -Im), as row t only
 // (the half-stored B of TcArgs::b_half).
 cudaError_t launch_pack_b(const float2* src, int Nb, int T, long long nc, long long s_l, long long s_t, long long c0,
-                          long long Kc, int N_alloc, int conj, void* hi, void* lo, cudaStream_t st);
+                          long long Kc, int N_alloc, bool half, void* hi, void* lo, cudaStream_t st);
 // FP16 B operands: the power-of-two scale that keeps |x| * scale <= 2^14
 // (inside the FP16 range with room to spare), and its inverse.
 __device__ __forceinline__ float f16_scale(unsigned amax_bits) {
@@ -427,7 +427,7 @@ struct TcRtArgs {
   long long vld_l, vld_b;
   long long conj_row;             // > 0: write the conjugate-embedding B operand: (Re, Im) at the
                                   // output position and (Im, -Re) conj_row entries further
-  int ra, rt;                     // ring depths: A (one slot per fill warp) and T (set by the launcher)
+  int rt;                         // ring depth of T (set by the launcher)
   int* status;
 };
 // tmT2 (split): tensor map of T's low-order part; T maps then use 32-element
