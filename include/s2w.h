@@ -88,7 +88,9 @@ typedef enum { S2W_DT_BACKWARD = 0, S2W_DT_NONE = 1 } s2w_dt_mode;
 
 /* Contraction engine for s2w_waveforms.  STREAM: CUDA-core kernels that
  * stream the resident spectra once per up to 8 ruptures (FP32, BF16 and
- * BF16_HILO storage; memory permitting) or once per rupture (FP8, FP32_HILO).
+ * BF16_HILO storage; memory permitting), per two (FP32_HILO) or per rupture
+ * (FP8; its adjoint per four).  ENGINE_TENSOR contexts, which stream only the
+ * seafloor output and the adjoint without tc_adjoint, keep workspaces for one.
  * TENSOR: tcgen05 tensor-core GEMMs over the whole rupture batch (one pass
  * over the spectra per sub-batch); needs prec_g = BF16, BF16_HILO or
  * FP8_E4M3, Nt <= 256, No <= 128.  With BF16 the activations (slip and

@@ -18,7 +18,8 @@
 // them), eight warps and scalar operations the rows streamed at 0.40 of the
 // copy rate: 963 x 6,000 x 64 x 256, stage 1 (24 GB) 8.9 ms, 3.45 here (1.01
 // of the copy rate), the whole call 10.5 -> 3.8 ms.  16 x 1,024 x 4 x 32, two
-// ruptures, whole call 57 -> 33 us (with the transforms of k_df.cu).
+// ruptures, whole call 57 -> 23 us (with the transforms of k_df.cu and
+// chained launches).
 #include <cuda.h>
 
 #include <type_traits>

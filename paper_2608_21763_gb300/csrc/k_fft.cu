@@ -13,7 +13,8 @@ namespace {
 constexpr int kWarps = 8;
 constexpr int kThreads = 32 * kWarps;
 // CTAs per SM of the transform kernels (registers: 80 a thread, 128 at 512
-// points)
+// points, where they spill: k_rfft_rows 48 bytes, k_irfft_rows 264,
+// k_retransform 148, k_rfft_tile up to 32; at 256 points k_retransform 8)
 __host__ __device__ constexpr int fft_ctas(int P) { return P >= 16 ? 2 : 3; }
 __host__ __device__ constexpr int tile_ctas(int P) { return P >= 8 ? 2 : 3; }  // (shared memory)
 __host__ __device__ constexpr int irfft_ctas(int P) { return P >= 8 ? 2 : 3; }  // (a row of bins in flight)
@@ -91,10 +92,11 @@ __global__ void __launch_bounds__(kThreads, fft_ctas(P)) k_rfft_rows(const float
 // The same with the bins transposed, for the contractions: tile_rows rows per
 // CTA pass through a shared tile, so that each bin's stores cover adjacent
 // rows (with a warp per row storing one 8-byte entry per bin, 963 x 256 rows
-// of 256 samples took 0.58 ms, 0.24 now; with the packing 0.87 -> 0.25).  Bin l of row `row`, with a = row / rows_a and c = row %
-// rows_a, goes to X[l * ld_l + a * ld_a + c]; or, PACK, into the B operand of
-// the real embedding (k_tc.cu: k_pack_b; conj: the conjugate one), rows 2a, 2a + 1 of
-// hi / lo[l * ld_l + 2 a * ld_a + c], BF16 pairs.
+// of 256 samples took 0.58 ms, 0.24 now; with the packing 0.87 -> 0.25).  Bin
+// l of row `row`, with a = row / rows_a and c = row % rows_a, goes to X[l *
+// ld_l + a * ld_a + c]; or, PACK, into the B operand of the real embedding
+// (k_tc.cu: k_pack_b; conj: the conjugate one), rows 2a, 2a + 1 of hi / lo[l *
+// ld_l + 2 a * ld_a + c], BF16 pairs.
 // Many rows: 32 per tile (128-byte stores of BF16 pairs; 96,300 rows of hi/lo
 // pairs 0.24 -> 0.16 ms against 16), 16 at 512 points (shared memory).  Up to
 // kFewRows rows: 8 per tile, one per warp, to spread over the SMs.

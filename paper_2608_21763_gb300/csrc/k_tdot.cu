@@ -10,10 +10,11 @@
 // weights into the stage beside them.  The consumer warps split the
 // columns: a thread owns one 16-byte chunk of every row and keeps the
 // sums of its columns for all R ruptures in registers, so nothing is reduced
-// across threads over long rows.  Every 64 rows they are added to sums in
-// shared memory (1.5 % of the instructions), since one
-// accumulation over a whole unit showed in the result (3.2e-7 against 2.6e-7
-// of FP32 rounding at 501 x 10,007 x 33 x 128).  With fewer chunks than threads, groups of
+// across threads over long rows.  Each time a multiple of 64 rows is passed
+// (whole stages, so after 64 to 127 rows) they are added to sums in shared
+// memory (1.5 % of the instructions), since one accumulation over a whole unit
+// showed in the result (3.2e-7 against 2.6e-7 of FP32 rounding at 501 x 10,007
+// x 33 x 128).  With fewer chunks than threads, groups of
 // threads take the rows in turn and are added up at the end of the unit, in
 // fixed order.  A row's weights are one shared-memory broadcast per two
 // ruptures.
@@ -21,13 +22,14 @@
 // What bounds it: HBM up to about four FP32 ruptures, then the FMAs (4 per
 // stored entry and rupture) and their issue: packed FP32 products (chunk.cuh)
 // with the weights prepared by the producer warp, sixteen FP32 warps (four
-// per scheduler).  Measured, adjoint of 963 x 8,000 x 64 x 256: one rupture
+// per scheduler; at six and eight ruptures their 96 registers spill 12 and 28
+// bytes).  Measured, adjoint of 963 x 8,000 x 64 x 256: one rupture
 // 2.57 ms (2.61 before, rows split over eight warps), two 2.61, four 2.90,
 // eight 4.2 (20.8 one by one; eight warps with scalar FMAs 4.8, sixteen 4.5);
 // BF16, one 1.31 ms (1.87), eight 3.3 (14.8); 60 x 60,000 x 4 x 256, one 1.5 ms
 // (10.7: the old kernel gave a short row to a whole warp).  FP32 gradient
 // through autograd, 501 x 10,007 x 33 x 128, six ruptures, forward and
-// backward: 11.5 -> 2.25 ms.  The sums do not depend on R: a rupture's result
+// backward: 11.5 -> 2.17 ms.  The sums do not depend on R: a rupture's result
 // is the same bits alone or in a batch.
 #include "chunk.cuh"
 

@@ -77,9 +77,13 @@ struct s2w_ctx {
   int tc_nkc = 1;        // stage-2 K chunks (<= s2_max_chunks, the partials' allocation)
   int s2_min_chunks = 1;  // fewest stage-2 chunks the default and the autotuner take (split: kSplitChunkK)
   int s2_max_chunks = 0;  // stage-2 chunks the partials are sized for
-  int tc_pair = 0;       // 1: two-SM MMAs (CTA pairs per M = 256 tile) where the shape allows; kPairAuto: for N = 512
+  int tc_pair = 0;       // 1: two-SM MMAs (CTA pairs per M = 256 tile) where the shape allows; kPairAuto: the rule of tc_shape
   bool tc_rtpair = false;  // two-SM tiles for the BF16 retransform GEMM
-  int tc_min_batch = 2;  // AUTO: smallest B on the tensor engine
+  // AUTO: smallest B on the tensor engine, until s2w_autotune has measured it.
+  // Stream / tensor ms at 963 x 12,000 x 64 x 256: two ruptures FP8 1.91 / 1.68,
+  // BF16 2.02 / 2.01, four 2.53 / 2.05; hi/lo 3.91 / 4.38, four 4.00 / 4.45, eight
+  // 5.01 / 4.53 (small grids alike: 24 x 700 x 6 x 64 from six on)
+  int tc_min_batch = 2;
   // test hooks (s2w_opts.fault): what to inject, and the kernel wait bound
   int fault = S2W_FAULT_NONE;
   unsigned long long wait_ns = kWaitLimitNs;

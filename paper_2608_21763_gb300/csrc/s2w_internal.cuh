@@ -277,7 +277,7 @@ cudaError_t launch_stream_dot(const StreamArgs& a, int num_sms, cudaStream_t st)
 __host__ __device__ constexpr int chain_slabs(int slabs) { return slabs > 2 ? slabs / 2 : 0; }
 
 // k_multi.cu: the same for 2 .. kStreamMulti ruptures and FP32 / BF16 /
-// BF16 hi/lo rows of more than 64 16-byte chunks (launch_stream_dot calls it).
+// BF16 hi/lo rows of more than 16 16-byte chunks (launch_stream_dot calls it).
 cudaError_t launch_stream_multi(const StreamArgs& a, int num_sms, cudaStream_t st);
 // k_dfdot.cu: the same for FP32 pairs (any nb; two ruptures per pass).
 cudaError_t launch_stream_df(const StreamArgs& a, int num_sms, cudaStream_t st);
