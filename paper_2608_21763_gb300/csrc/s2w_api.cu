@@ -885,11 +885,15 @@ int s2w_create(int Ns, int Ng, int No, int Nt, const s2w_opts* opts, s2w_ctx** o
   ctx->L = ctx->single_pass ? 4 * Nt : 2 * Nt;
   ctx->Ns_pad = static_cast<int>(round_up(Ns, 8));
   ctx->nseg = static_cast<int>((Ng + 1023) / 1024);
-  // FP32 pairs: the stage-2 kernel's units are (bin, segment); a small grid is
-  // cut into shorter segments (128 points or more) until there are about two
-  // units per SM (16 x 1,024 x 4 x 32: 33 units, 10 us -> 264 units, 6 us)
-  if (o.prec_g == S2W_PREC_FP32_HILO)
-    ctx->nseg = std::max(ctx->nseg, std::min((304 + ctx->Nb - 1) / ctx->Nb, Ng / 128));
+  // FP32 pairs: the stage-2 kernel's units are (bin, segment, tile of 64
+  // observations); a small grid is cut into shorter segments (128 points or
+  // more) until there are about two units per SM (16 x 1,024 x 4 x 32: 33 units,
+  // 10 us -> 264 units, 6 us).  Many observations make units by themselves, and
+  // partials of every segment that the call without allocation has no room for
+  if (o.prec_g == S2W_PREC_FP32_HILO) {
+    const long long units = static_cast<long long>(ctx->Nb) * ((No + 63) / 64);
+    ctx->nseg = std::max(ctx->nseg, static_cast<int>(std::min<long long>((304 + units - 1) / units, Ng / 128)));
+  }
   ctx->RL = static_cast<int>(round_up((Ng + ctx->nseg - 1) / ctx->nseg, 8));
   ctx->opts = o;
   ctx->opts.tune_cache = nullptr;  // the caller's string is not kept
