@@ -122,7 +122,8 @@ typedef struct {
                      s2w_misfit_gradient run on the tensor engine for
                      batches (same rules as s2w_waveforms); doubles the
                      stage-1 operator memory.  0 (default): the adjoint
-                     streams the spectra once per up to 8 ruptures. */
+                     streams the spectra once per up to 8 ruptures (FP8 4,
+                     ENGINE_TENSOR 1). */
   int single_pass; /* 1: the single-pass variant (an ablation of the
                       truncate-and-retransform step): both operators are kept
                       at FFT length L = 4 Nt (2 Nt + 1 bins, twice the bytes),
@@ -281,7 +282,7 @@ int s2w_waveforms_active(s2w_ctx *ctx, const float *slip, const int *active_len,
  * evaluated as conj(Fhat_l) yhat_l per bin with zero padding to 2 Nt (no
  * wrap reaches the kept samples), and D_t^T w[n] = (w[n] - w[n+1]) / dt with
  * w[Nt] = 0.  Without opts.tc_adjoint: the streaming kernels, up to 8 ruptures
- * per pass, for every storage precision.  With opts.tc_adjoint (BF16 or
+ * per pass (FP8 4; ENGINE_TENSOR 1), for every storage precision but FP32_HILO.  With opts.tc_adjoint (BF16 or
  * BF16_HILO storage) and B >= the AUTO batch threshold (or ENGINE_TENSOR):
  * both correlations run as tcgen05 GEMMs over the sub-batch against the
  * transposed spectra, with the same hi/lo splitting as the forward tensor
